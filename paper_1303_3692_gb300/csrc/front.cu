@@ -185,8 +185,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         const bool look = ok && entry && m > 0 && d.krt != nullptr && m >= kk;
         const uint64_t x = look ? (w[0] >> (64u - 2u * kk)) : 0ull;
         uint4 h, e01, e23, e45;
-        ldg32_if(look, d.krt + 4 * x, &h, &e01);
-        ldg32_if(look, d.krt + 4 * x + 2, &e23, &e45);
+        ldg64_pairs_if(look, d.krt + 4 * x, &h, &e01, &e23, &e45);
         uint32_t L = look ? h.x - 1u : 0xFFFFFFFFu;  // 0xFFFFFFFF stands for -1
         uint32_t R = look ? h.y : d.n;
 
