@@ -184,15 +184,17 @@ typedef struct sa_search_params {
  * the search reads:
  *  - the key table kept in shared memory (first 64 bases of the suffixes at
  *    ranks floor((2p+1) n / 2^(l+1)), the top levels of the binary search);
- *  - one 32-byte record per rank (the first 112 bases of that suffix and its
- *    position), so that a probe reads one aligned sector;
+ *  - one 32-byte record per rank (the first 104 bases of that suffix, the
+ *    lengths of its common prefixes with the ranks beside it, at most 255,
+ *    and its position), so that a probe reads one aligned sector and often
+ *    settles the neighbouring ranks too;
  *  - unless SA_NO_KMER, the k-mer table: for each of the 4^k k-base
  *    strings x a 64-byte entry with lo = kmer[x] = number of suffixes that
  *    sort before x and hi = kmer[x + 1] (a query of m >= k bases whose first
  *    k bases are x lies strictly between ranks lo - 1 and hi), and the
- *    position and first 192 bases of the suffix at rank
- *    lo - 1 + (hi - lo + 1) / 2, the first pivot of the binary search over
- *    that bracket -- so one read brackets a query and makes its first probe.
+ *    position, first 192 bases and the two common prefixes of the suffix at
+ *    rank lo - 1 + (hi - lo + 1) / 2, the first pivot of the binary search
+ *    over that bracket -- so one read brackets a query and makes its first probe.
  *    Automatic k: the largest k with 4^k <= 3n, in 1..15 (64 * 4^k bytes:
  *    17 GB at k = 14 for 10^8 bases, 69 GB at k = 15).
  * Device memory: about n/4 + (width + 32) n bytes + the k-mer table.

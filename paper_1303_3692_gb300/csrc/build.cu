@@ -275,21 +275,66 @@ cudaError_t launch_build_keys(sa_index *idx, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Suffix records: for rank i, the first 112 bases of suffix SA[i] and SA[i]
-// itself in one 32-byte entry (one DRAM sector), so that a probe of the
-// search reads one aligned sector instead of an SA entry and then the text it
-// points to, and a query of up to 112 bases never reads the text.
+// Suffix records: for rank i, the first 104 bases of suffix SA[i], its common
+// prefixes with the suffixes at the ranks beside it, and SA[i] itself in one
+// 32-byte entry (one DRAM sector), so that a probe of the search reads one
+// aligned sector instead of an SA entry and then the text it points to, and a
+// query of up to 104 bases never reads the text.
+//
+// A warp makes the records of 30 ranks: its lanes hold 32 consecutive
+// suffixes' first 128 bases, each lane counts the bases it shares with the
+// next lane's (reading on in the text past 128 equal ones, up to 255), and
+// the outer two lanes only serve as neighbours.  The reads of the text (four
+// windows per rank, random) bound it, 6 % more of them for the two outer
+// lanes.
+constexpr int kRecRanks = 30;  // ranks per warp
+
 template <typename IdxT>
 __global__ void build_records_kernel(const uint64_t *__restrict__ T, const IdxT *__restrict__ sa, uint64_t n,
                                      uint4 *rec) {
-    GS_LOOP(i, n) {
-        const uint64_t pos = sa[i];
-        const uint64_t w0 = text_window(T, pos);
-        const uint64_t w1 = text_window(T, pos + 32);
-        const uint64_t w2 = text_window(T, pos + 64);
-        const uint64_t w3 = text_window(T, pos + 96);
-        rec[2 * i] = make_uint4((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32));
-        rec[2 * i + 1] = make_uint4((uint32_t)w2, (uint32_t)(w2 >> 32), (uint32_t)(w3 >> 32), (uint32_t)pos);
+    const unsigned lane = threadIdx.x & 31u;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    const uint64_t groups = (n + kRecRanks - 1) / kRecRanks;
+    for (uint64_t g = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < groups; g += warps) {
+        const uint64_t i = g * kRecRanks + lane - 1u;  // lane 0 of the first group: no rank (wraps)
+        const bool live = i < n;
+        const uint64_t pos = live ? (uint64_t)sa[i] : 0;
+        uint64_t w[4] = {0, 0, 0, 0};
+        if (live) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint64_t b = pos + 32ull * j;
+                w[j] = b < n ? text_window(T, b) : 0ull;
+            }
+        }
+        // bases shared with the next lane's suffix
+        const uint64_t npos = __shfl_down_sync(0xFFFFFFFFu, pos, 1);
+        const bool nlive = __shfl_down_sync(0xFFFFFFFFu, (int)live, 1) != 0 && lane < 31u;
+        uint32_t same = 0;
+        bool more = true;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const uint64_t x = w[j] ^ __shfl_down_sync(0xFFFFFFFFu, w[j], 1);
+            if (more) same += x ? (uint32_t)(__clzll((long long)x) >> 1) : 32u;
+            more = more && x == 0;
+        }
+        uint32_t ln = 0;
+        if (live && nlive) {
+            const uint64_t far = pos > npos ? pos : npos;
+            const uint32_t room = n - far < kLcpCap ? (uint32_t)(n - far) : kLcpCap;
+            while (more && same < room) {
+                const uint64_t x = text_window(T, pos + same) ^ text_window(T, npos + same);
+                same += x ? (uint32_t)(__clzll((long long)x) >> 1) : 32u;
+                more = x == 0;
+            }
+            ln = same < room ? same : room;
+        }
+        const uint32_t lp = __shfl_up_sync(0xFFFFFFFFu, ln, 1);  // 0 at rank 0: lane 0 held no suffix
+        if (live && lane >= 1u && lane <= (unsigned)kRecRanks) {
+            rec[2 * i] = make_uint4((uint32_t)w[0], (uint32_t)(w[0] >> 32), (uint32_t)w[1], (uint32_t)(w[1] >> 32));
+            rec[2 * i + 1] = make_uint4((uint32_t)w[2], (uint32_t)(w[2] >> 32),
+                                        ((uint32_t)(w[3] >> 32) & 0xFFFF0000u) | (lp << 8) | ln, (uint32_t)pos);
+        }
     }
 }
 
@@ -323,8 +368,9 @@ __global__ void build_kmer_kernel(const uint4 *__restrict__ rec, uint64_t n, uin
 //     than k that falls between the two), lo = number of suffixes sorting
 //     before x; when hi > lo, pos is the position of the suffix at rank
 //     M = lo - 1 + (hi - lo + 1) / 2 -- the first pivot of the lockstep binary
-//     search over (lo - 1, hi) -- and clamp = min(192, n - pos) the number of
-//     its first 192 bases that exist;
+//     search over (lo - 1, hi) -- and the last word holds clamp = min(192, n -
+//     pos), the number of its first 192 bases that exist, and its record's two
+//     common prefixes with the ranks beside it;
 //   three uint4: the first 192 bases of that suffix as six packed words.
 // One aligned 64-byte read therefore brackets a query of m >= k bases and
 // makes its first probe.
@@ -337,10 +383,11 @@ __global__ void build_krt_kernel(const uint32_t *__restrict__ kmer, const uint4 
         uint64_t e[6] = {0, 0, 0, 0, 0, 0};
         if (hi > lo) {
             const uint32_t M = lo + (hi - lo + 1u) / 2u - 1u;
-            const uint64_t pos = rec[2 * (uint64_t)M + 1].w;
+            const uint4 r1 = rec[2 * (uint64_t)M + 1];
+            const uint64_t pos = r1.w;
             const uint64_t left = n - pos;  // >= 1
             h.z = (uint32_t)pos;
-            h.w = (uint32_t)(left < 192 ? left : 192);
+            h.w = (uint32_t)(left < 192 ? left : 192) | (((r1.z >> 8) & 0xFFu) << 8) | ((r1.z & 0xFFu) << 16);
 #pragma unroll
             for (int j = 0; j < 6; j++) {
                 const uint64_t b = pos + 32ull * j;
@@ -385,7 +432,7 @@ cudaError_t launch_copy_kmer_counts(const sa_index *idx, uint32_t *dst, cudaStre
 }
 
 cudaError_t launch_build_records(sa_index *idx, cudaStream_t s) {
-    const unsigned g = grid_for(idx->n);
+    const unsigned g = grid_for((idx->n + kRecRanks - 1) / kRecRanks * 32);
     if (idx->width == 4)
         build_records_kernel<uint32_t><<<g, kThreads, 0, s>>>(idx->text, reinterpret_cast<const uint32_t *>(idx->sa),
                                                               idx->n, idx->rec);

@@ -186,15 +186,14 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         const uint64_t x = look ? (w[0] >> (64u - 2u * kk)) : 0ull;
         uint4 h, e01, e23, e45;
         ldg64_pairs_if(look, d.krt + 4 * x, &h, &e01, &e23, &e45);
-        uint32_t L = look ? h.x - 1u : 0xFFFFFFFFu;  // 0xFFFFFFFF stands for -1
-        uint32_t R = look ? h.y : d.n;
+        Bounds bd;
+        bd.start(look ? h.x - 1u : 0xFFFFFFFFu, look ? h.y : d.n);  // 0xFFFFFFFF stands for -1
 
-        bool done = !live || !ok || m == 0 || (look && R - L <= 1u);
+        bool done = !live || !ok || m == 0 || (look && bd.R - bd.L <= 1u);
         if (live && !ok) store_result_sum(a, q, ~0ull, ~0ull);
         if (live && ok && m == 0) store_result_sum(a, q, 0, d.n);
-        if (live && ok && m > 0 && look && R - L <= 1u) store_result_sum(a, q, R, R);
+        if (live && ok && m > 0 && look && bd.R - bd.L <= 1u) store_result_sum(a, q, bd.R, bd.R);
 
-        uint32_t lcpL = 0, lcpR = 0, HL = 0, HR = 0, hlcpL = 0, hlcpR = 0, lo = 0, phase = 0;
         bool go = !done && look;
         // in list order, bases 128-191 are the record's last 16 bytes (read
         // again when a compare gets there: an L1 or L2 hit)
@@ -202,37 +201,13 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
                               kFromList ? reinterpret_cast<const uint64_t *>(a.wrec_in + 4 * (size_t)lslot + 3)
                                         : nullptr,
                               kFromList ? 2u : 0u};
-        // One compare's outcome c at pivot M with common prefix l.
-        auto step = [&](int c, uint32_t M, uint32_t l) {
-            if (c == CMP_PREFIX && phase == 0) {
-                HL = M;
-                hlcpL = m;
-                HR = R;
-                hlcpR = lcpR;
-                R = M;
-                lcpR = m;
-                phase = 1;
-            } else if (c == CMP_LESS || (c == CMP_PREFIX && phase == 1)) {
-                R = M;
-                lcpR = l;
-            } else {
-                L = M;
-                lcpL = l;
-            }
-            if (R - L <= 1u) {
-                if (phase == 1) {
-                    lo = R;
-                    L = HL;
-                    R = HR;
-                    lcpL = hlcpL;
-                    lcpR = hlcpR;
-                    phase = 2;
-                }
-                if (R - L <= 1u) {
-                    store_result_sum(a, q, phase == 0 ? R : lo, R);
-                    done = true;
-                    go = false;
-                }
+        // One compare's outcome c at pivot M with common prefix l (lp, ln: the
+        // pivot's own common prefixes with its neighbours).
+        auto step = [&](int c, uint32_t M, uint32_t l, uint32_t lp, uint32_t ln) {
+            if (bd.step(c, M, l, m, lp, ln)) {
+                store_result_sum(a, q, bd.first(), bd.R);
+                done = true;
+                go = false;
             }
         };
         if (go) {  // the first probe: the entry's pivot
@@ -240,22 +215,23 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
                                    ((uint64_t)e23.y << 32) | e23.x, ((uint64_t)e23.w << 32) | e23.z,
                                    ((uint64_t)e45.y << 32) | e45.x, ((uint64_t)e45.w << 32) | e45.z};
             uint32_t l;
-            const int c = cmp_entry(w, m, e, h.z, h.w, d.n, d.text, qw, &l);
-            step(c, L + ((R - L) >> 1), l);
+            const int c = cmp_entry(w, m, e, h.z, h.w & 0xFFu, d.n, d.text, qw, &l);
+            step(c, bd.pivot(), l, (h.w >> 8) & 0xFFu, (h.w >> 16) & 0xFFu);
         }
         // Further probes, one suffix record each; queries without a k-mer
         // bracket go straight to the worklist (the persistent kernel descends
         // the shared-memory key table first).
         for (uint32_t p = 1; p < a.front_probes && __any_sync(0xFFFFFFFFu, go); p++) {
-            const uint32_t M = L + ((R - L) >> 1);
+            const uint32_t M = bd.pivot();
             uint4 r0, r1;
             ldg32_if(go, d.rec + 2 * (size_t)M, &r0, &r1);
             if (go) {
                 uint32_t l;
                 bool und = false;
                 int c = cmp_record(w[0], w[1], w[2], w[3], m, r0, r1, d.n, &l, &und);
-                if (und) c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, max(112u, min(lcpL, lcpR)), &l);
-                step(c, M, l);
+                if (und)
+                    c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
+                step(c, M, l, (r1.z >> 8) & 0xFFu, r1.z & 0xFFu);
             }
         }
 
@@ -274,7 +250,8 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
             }
             if (rest) {
                 const uint32_t slot = staged + __popc(bal & lanemask_lt);
-                s_stage[wib][slot][0] = make_uint4(phase == 2 ? lo - 1u : L, phase == 1 ? HR : R, m, (uint32_t)q);
+                s_stage[wib][slot][0] = make_uint4(bd.phase == 2 ? bd.lo - 1u : bd.L,
+                                                     bd.phase == 1 ? bd.HR : bd.R, m, (uint32_t)q);
                 const uint64_t w4 = m > 128u ? qw(128u) : 0ull;  // bases 128-159 for the persistent pass
                 s_stage[wib][slot][1] =
                     make_uint4((uint32_t)qa, (uint32_t)(qa >> 32) | (r << 16), (uint32_t)w4, (uint32_t)(w4 >> 32));

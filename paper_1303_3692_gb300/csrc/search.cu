@@ -151,15 +151,11 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s for the key-table copy
 //             the key table first;
 //   descent   compare with the key of level-order node k in shared memory
 //             (k = 0 once the table's depth is passed or the bounds split);
-//   deep      load the suffix record of rank M = L + (R - L)/2 (32 bytes: 112
-//             bases and SA[M]) -- with query bases 64-127 from the worklist
-//             record in the same round -- and compare; only when all 112
+//   deep      load the suffix record of rank M = L + (R - L)/2 (32 bytes: 104
+//             bases, the common prefixes with the ranks beside M, SA[M]) -- with query bases 64-127 from the worklist
+//             record in the same round -- and compare; only when all 104
 //             bases tie does the compare continue in the packed text.
-// Ranks are 32-bit modular: L = 0xFFFFFFFF stands for -1, and since every
-// rank is in [-1, n] with n < 2^32 - 1, R - L and L + (R - L)/2 are exact.
-// phase 0: both bounds share (L, R); a prefix match splits them into the
-// lower bound in (L, M] (phase 1) and the upper bound in [M, R), kept in
-// (HL, HR) until phase 1 ends (phase 2).
+// (The bounds' own arithmetic: Bounds in sa_internal.cuh.)
 // Warps take chunks of worklist entries from one global counter, each
 // chunk's base fetched while the previous chunk is handed out.
 // Launch bounds: 1024 threads, one CTA per SM, at most 64 registers (no
@@ -224,8 +220,9 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
     bool active = false, fresh = false;
     uint32_t wi = 0, qout = 0, m = 0;
     uint64_t qa = 0, q0 = 0, q1 = 0;
-    uint32_t L = 0, R = 0, HL = 0, HR = 0, lcpL = 0, lcpR = 0, hlcpL = 0, hlcpR = 0, lo = 0;
-    uint32_t k = 0, phase = 0;
+    Bounds bd;
+    bd.start(0, 0);
+    uint32_t k = 0;
 
     for (;;) {
         unsigned need = __ballot_sync(0xFFFFFFFFu, !active);
@@ -258,7 +255,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
         // the suffix record at the pivot and query bases 64-127 (deep).
         const bool init = fresh;
         const bool deep = !init && k == 0;
-        uint32_t M = L + ((R - L) >> 1);
+        uint32_t M = bd.pivot();
         const uint4 *wrec = a.wrec + 4 * (size_t)wi;
         uint4 r0, r1;
         ldg32_if(init || deep, init ? (const void *)wrec : (const void *)(REC + 2 * (size_t)M), &r0, &r1);
@@ -285,16 +282,13 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             qa = ((uint64_t)(r1.y & 0xFFFFu) << 32) | r1.x;
             q0 = x2;
             q1 = x3;
-            lcpL = lcpR = 0;
-            phase = 0;
-            L = r0.x;
-            R = r0.y;
+            bd.start(r0.x, r0.y);
             k = (KM != nullptr && m >= kk) ? 0u : (depth ? 1u : 0u);
             continue;
         }
 
         int c;
-        uint32_t l;
+        uint32_t l, lp = kLcpUnknown, ln = kLcpUnknown;
         if (k != 0) {
             // Descent: node k at level lvl samples rank floor((2p+1) n / 2^(lvl+1)).
             const uint32_t lvl = 31u - __clz(k);
@@ -313,41 +307,17 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             if (und) {
                 // query bases 96-127 are x3, 128-159 the worklist record's second word pair
                 const QueryWindows qw{a.tq, qa, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};
-                c = cmp_suffix_qw(T, n, r1.w, qw, m, max(112u, min(lcpL, lcpR)), &l);
+                c = cmp_suffix_qw(T, n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
             }
+            lp = (r1.z >> 8) & 0xFFu;
+            ln = r1.z & 0xFFu;
         }
-        if (c == CMP_PREFIX && phase == 0) {
-            HL = M;
-            hlcpL = m;
-            HR = R;
-            hlcpR = lcpR;
-            R = M;
-            lcpR = m;
-            phase = 1;
-            k = 0;
-        } else if (c == CMP_LESS || (c == CMP_PREFIX && phase == 1)) {
-            R = M;
-            lcpR = l;
-        } else {
-            L = M;
-            lcpL = l;
-        }
-        // Finished intervals: move to the upper bound, or write the result.
-        if (R - L <= 1u) {
-            if (phase == 1) {
-                lo = R;
-                L = HL;
-                R = HR;
-                lcpL = hlcpL;
-                lcpR = hlcpR;
-                phase = 2;
-                k = 0;
-            }
-            if (R - L <= 1u) {
-                const uint32_t lo_out = phase == 0 ? R : lo;
-                store_result_sum(a, qout, lo_out, R);
-                active = false;
-            }
+        const uint32_t phase = bd.phase;
+        const bool finished = bd.step(c, M, l, m, lp, ln);
+        if (bd.phase != phase) k = 0;  // the descent's nodes halve the whole range only
+        if (finished) {
+            store_result_sum(a, qout, bd.first(), bd.R);
+            active = false;
         }
     }
 }
