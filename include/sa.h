@@ -168,8 +168,7 @@ typedef struct sa_search_params {
 /* sa_search_params.flags: each query names its strand -- bit 31 of q_ref[q]
  * set means search query q's reverse complement (as SA_PARAM_REVERSE_COMPLEMENT
  * does for a whole batch); the reference id is q_ref[q] & 0x7FFFFFFF.  q_ref
- * is then required, also with one index (ids 0), and the batch is packed in
- * both directions (twice the packed batch's scratch).  Not together with
+ * is then required, also with one index (ids 0).  Not together with
  * SA_PARAM_REVERSE_COMPLEMENT (SA_ERR_ARG).  sa_locate ignores bit 31 of q_ref. */
 #define SA_PARAM_STRAND_PER_QUERY 0x20u
 

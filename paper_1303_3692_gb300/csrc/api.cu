@@ -256,12 +256,11 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     if (strand_bits && (revcomp || !q_ref)) return SA_ERR_ARG;
     cudaError_t err = cudaSuccess;
     const uint64_t nwords = (total + 31) / 32;
-    // both packings, one after the other, when each query names its strand
-    const uint64_t tq_words = (nwords + SA_TQ_PAD_WORDS) * (strand_bits ? 2 : 1);
+    const uint64_t tq_words = nwords + SA_TQ_PAD_WORDS;
     // list and worklist records hold a query's first base in 48 bits (a batch
     // that large could not be resident anyway)
     if (!plain && tq_words * 32 >= kListMaxBase) return SA_ERR_ARG;
-    uint64_t *tq = sc.get<uint64_t>(tq_words);
+    uint64_t *tq = sc.get<uint64_t>(SA_TQ_LEAD_WORDS + tq_words) + SA_TQ_LEAD_WORDS;
     uint32_t *tv = sc.get<uint32_t>(tq_words);
     uint4 *wrec = plain ? nullptr : sc.get<uint4>(4 * n_q);
     uint64_t ktotal = 0;
@@ -269,17 +268,19 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
         if (refs[r]->krt) ktotal += 1ull << (2 * refs[r]->kmer_k);
     const bool kmer_order = !plain && use_kmer_order(refs, n_refs, n_q, order);
     uint4 *wrec_in = kmer_order ? sc.get<uint4>(4 * list_capacity(n_q)) : nullptr;
-    uint32_t *bplan = kmer_order ? sc.get<uint32_t>(kPlanWords) : nullptr;
-    // [0] pack error, [1] status, [2] worklist count, [3] bad reference id,
-    // [4] records of the k-mer-ordered list, [5] a non-base byte in the batch
-    int *flags = sc.get<int>(8);
-    unsigned long long *counter = sc.get<unsigned long long>(1);
+    // What starts at zero, in one block: flags [0] pack error, [1] status, [2]
+    // worklist count, [3] bad reference id, [4] records of the k-mer-ordered
+    // list, [5] a non-base byte in the batch; the persistent pass's counter;
+    // the k-mer order's plan; the bitmap of packed words with a non-base byte.
+    const size_t plan_words = kmer_order ? kPlanWords : 0, bitmap_words = tq_words / 32 + 1;
+    uint32_t *zeroed = sc.get<uint32_t>(10 + plan_words + bitmap_words);
     if (sc.failed) return SA_ERR_NOMEM;
+    int *flags = reinterpret_cast<int *>(zeroed);
+    unsigned long long *counter = reinterpret_cast<unsigned long long *>(zeroed + 8);
+    uint32_t *bplan = kmer_order ? zeroed + 10 : nullptr;
+    uint32_t *tvb = zeroed + 10 + plan_words;
     if (((uintptr_t)wrec & 31u) != 0) return SA_ERR_CUDA;  // the search reads 32-byte records
-    if ((err = cudaMemsetAsync(flags, 0, 8 * sizeof(int), s)) != cudaSuccess) return status_from_cuda(err);
-    if ((err = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s)) != cudaSuccess)
-        return status_from_cuda(err);
-    if (bplan && (err = cudaMemsetAsync(bplan, 0, kPlanWords * sizeof(uint32_t), s)) != cudaSuccess)
+    if ((err = cudaMemsetAsync(zeroed, 0, (10 + plan_words + bitmap_words) * sizeof(uint32_t), s)) != cudaSuccess)
         return status_from_cuda(err);
     *flags_out = flags;
 
@@ -294,6 +295,7 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.width = width;
     L.ascii = ascii;
     L.tq = tq;
+    L.tvb = tvb;
     L.tv = tv;
     L.nwords = nwords;
     L.q_off = q_off;
@@ -317,7 +319,6 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
                                                     : (kmer_order ? 3u : default_front_probes(refs, n_refs));
     L.revcomp = revcomp;
     L.strand_bits = strand_bits;
-    L.rc_base = strand_bits ? (nwords + SA_TQ_PAD_WORDS) * 32 : 0;
     L.expire_waits = params && (params->flags & SA_PARAM_EXPIRE_WAITS);
     L.trunc_cap = trunc_cap;
     L.tile_kept = tile_kept;
@@ -329,7 +330,7 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.bad_ref = flags + 3;
     L.batch_dirty = flags + 5;
 
-    if ((err = launch_pack_batch(L, tq, tv, s)) != cudaSuccess) return status_from_cuda(err);
+    if ((err = launch_pack_batch(L, tq, tvb, tv, s)) != cudaSuccess) return status_from_cuda(err);
     cudaEvent_t ev0 = params ? reinterpret_cast<cudaEvent_t>(params->search_events[0]) : nullptr;
     cudaEvent_t ev1 = params ? reinterpret_cast<cudaEvent_t>(params->search_events[1]) : nullptr;
     if (ev0 && (err = cudaEventRecord(ev0, s)) != cudaSuccess) return status_from_cuda(err);

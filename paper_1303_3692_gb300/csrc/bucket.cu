@@ -56,18 +56,19 @@ struct BucketRef {
     uint32_t kmer_k;  // 0: no k-mer table
 };
 
-// The query's first base in the packed batch (in the reverse-complement
-// packing for the other strand), its length, its reference id (*r, the strand
-// bit cleared) and whether the range and the reference id are usable.
-__device__ __forceinline__ bool query_range(const SearchLaunch &a, uint64_t q, uint32_t *r, uint64_t *qa_out,
+// The query's place in the packed batch (which names its strand), its length,
+// its reference id (*r, the strand bit cleared) and whether the range and the
+// reference id are usable.
+template <bool kStrands>
+__device__ __forceinline__ bool query_range(const SearchLaunch &a, uint64_t q, uint32_t *r, uint64_t *at_out,
                                             uint32_t *m_out, bool *bad_range, bool *bad_ref) {
     const uint64_t qa = __ldg(a.q_off + q) - a.first, qe = __ldg(a.q_off + q + 1) - a.first;
-    const bool rc = a.revcomp || (a.strand_bits && (*r & kStrandBit));
-    if (a.strand_bits) *r &= ~kStrandBit;
+    const bool rc = kStrands && (a.revcomp || (a.strand_bits && (*r & kStrandBit)));
+    if (kStrands && a.strand_bits) *r &= ~kStrandBit;
     const bool range_ok = qa <= qe && qe <= a.total && qe - qa < (1ull << 31);
     *bad_range = !range_ok;
     *bad_ref = range_ok && *r >= a.n_refs;
-    *qa_out = range_ok ? strand_start(qa, qe, a.total, rc, a.rc_base) : qa;
+    *at_out = range_ok ? query_place(qa, qe, rc) : 0;
     *m_out = range_ok ? (uint32_t)(qe - qa) : 0u;
     return range_ok && *r < a.n_refs;
 }
@@ -81,14 +82,7 @@ __device__ __forceinline__ uint16_t bucket_of(const SearchLaunch &a, const Bucke
     return (uint16_t)kNumBuckets;  // no k-mer bracket: the key-table descent
 }
 
-// The query's first 32 bases from the packed batch (qa's word and the next).
-__device__ __forceinline__ uint64_t first_word(const uint64_t *__restrict__ tq, uint64_t qa) {
-    const uint64_t wl = qa >> 5;
-    const uint32_t sh = (uint32_t)(qa & 31u) * 2u;
-    return (__ldg(tq + wl) << sh) | ((__ldg(tq + wl + 1) >> 1) >> (63u - sh));
-}
-
-template <bool kSingle>
+template <bool kSingle, bool kStrands>
 __global__ void __launch_bounds__(kSampleThreads) bucket_sample_kernel(const __grid_constant__ SearchLaunch a) {
     __shared__ uint32_t hist[kNumBuckets + 1];
     __shared__ BucketRef sref[SA_MAX_REFS];
@@ -102,12 +96,12 @@ __global__ void __launch_bounds__(kSampleThreads) bucket_sample_kernel(const __g
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_s; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t q = i * kListSampleStride;
         uint32_t r = kSingle ? 0u : __ldg(a.q_ref + q);
-        uint64_t qa;
+        uint64_t at;
         uint32_t m;
         bool bad_range, bad_ref;
         // an estimate: the bases' validity is left to the scatter
-        if (query_range(a, q, &r, &qa, &m, &bad_range, &bad_ref) && m > 0)
-            atomicAdd(&hist[bucket_of(a, sref[kSingle ? 0u : r], m, first_word(a.tq, qa))], 1u);
+        if (query_range<kStrands>(a, q, &r, &at, &m, &bad_range, &bad_ref) && m > 0)
+            atomicAdd(&hist[bucket_of(a, sref[kSingle ? 0u : r], m, query_window<kStrands>(a.tq, at, 0))], 1u);
     }
     __syncthreads();
     for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x)
@@ -157,7 +151,7 @@ constexpr int kScatterItems = 2;
 constexpr uint32_t kScatterTile = (uint32_t)kScatterThreads * kScatterItems;  // 32 KB of records
 constexpr size_t kScatterSmem = (size_t)kScatterTile * 64;
 
-template <bool kSingle>
+template <bool kSingle, bool kStrands>
 __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(const __grid_constant__ SearchLaunch a,
                                                                            uint4 *__restrict__ list) {
     extern __shared__ uint4 srec[];  // kScatterTile records of 4 uint4
@@ -175,11 +169,11 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
         sref[r] = BucketRef{d.kbase, d.n, d.krt != nullptr ? d.kmer_k : 0u};
     }
     // a batch without a non-base byte needs no validity masks
-    const bool dirty = a.batch_dirty == nullptr || *a.batch_dirty != 0;
+    const bool dirty = *a.batch_dirty != 0;
     const uint64_t tile = (uint64_t)blockIdx.x * kScatterTile;
     uint16_t b[kScatterItems];
     uint32_t rank[kScatterItems], r[kScatterItems], m[kScatterItems];
-    uint64_t qa[kScatterItems], w[kScatterItems][4];
+    uint64_t at[kScatterItems], w[kScatterItems][4];
     bool any_bad = false, any_bad_ref = false;
     __syncthreads();
     // Every item's loads are issued before the tile's bookkeeping, so that
@@ -192,12 +186,12 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
 #pragma unroll
     for (int it = 0; it < kScatterItems; it++) {
         const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
-        qa[it] = 0;
+        at[it] = 0;
         m[it] = 0;
         b[it] = kNoQuery;
         if (q < a.n_q) {
             bool bad_range, bad_ref;
-            const bool ok = query_range(a, q, &r[it], &qa[it], &m[it], &bad_range, &bad_ref);
+            const bool ok = query_range<kStrands>(a, q, &r[it], &at[it], &m[it], &bad_range, &bad_ref);
             any_bad |= bad_range;
             any_bad_ref |= bad_ref;
             b[it] = ok ? 0u : kNoQuery;  // usable so far; the bucket follows
@@ -208,8 +202,8 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
         const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
         // a query without a record reads the batch's first words (always there)
         const bool ok = b[it] != kNoQuery;
-        const bool valid = load_query_head(a.tq, a.tv, ok ? qa[it] >> 5 : 0, ok ? (uint32_t)(qa[it] & 31u) : 0u,
-                                           m[it], ok && m[it] > 0 && dirty, w[it]);
+        query_windows<4, kStrands>(a.tq, ok ? at[it] : 0, 0, w[it]);
+        const bool valid = !(ok && m[it] > 0 && dirty) || query_valid(a.tvb, a.tv, place_first(at[it], m[it]), m[it]);
         if (q >= a.n_q) continue;
         if (!ok || !valid) {
             if (ok) any_bad = true;
@@ -263,22 +257,16 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
         const uint32_t slot = off[b[it]] + rank[it];
         // bases 128-191 (the first pass then reads none of a query of up to
         // 192 bases from the batch)
-        uint64_t t0 = 0, t1 = 0;
-        if (m[it] > 128u) {
-            const uint64_t wl = qa[it] >> 5;
-            const uint32_t sh = (uint32_t)(qa[it] & 31u) * 2u;
-            const uint64_t x4 = __ldg(a.tq + wl + 4), x5 = __ldg(a.tq + wl + 5), x6 = __ldg(a.tq + wl + 6);
-            t0 = (x4 << sh) | ((x5 >> 1) >> (63u - sh));
-            t1 = (x5 << sh) | ((x6 >> 1) >> (63u - sh));
-        }
+        uint64_t t[2] = {0, 0};
+        if (m[it] > 128u) query_windows<2, kStrands>(a.tq, at[it], 128u, t);
         uint4 *dst = srec + 4 * slot;
-        dst[0] = make_uint4(m[it], (uint32_t)q, (uint32_t)qa[it],
-                            (uint32_t)(qa[it] >> 32) | (r[it] << 16) | (entry ? kListNeedsEntry : 0u));
+        dst[0] = make_uint4(m[it], (uint32_t)q, (uint32_t)at[it],
+                            place_high(at[it], r[it]) | (entry ? kListNeedsEntry : 0u));
         dst[1] = make_uint4((uint32_t)w[it][0], (uint32_t)(w[it][0] >> 32), (uint32_t)w[it][1],
                             (uint32_t)(w[it][1] >> 32));
         dst[2] = make_uint4((uint32_t)w[it][2], (uint32_t)(w[it][2] >> 32), (uint32_t)w[it][3],
                             (uint32_t)(w[it][3] >> 32));
-        dst[3] = make_uint4((uint32_t)t0, (uint32_t)(t0 >> 32), (uint32_t)t1, (uint32_t)(t1 >> 32));
+        dst[3] = make_uint4((uint32_t)t[0], (uint32_t)(t[0] >> 32), (uint32_t)t[1], (uint32_t)(t[1] >> 32));
         slot_bucket[slot] = b[it];
     }
     __syncthreads();
@@ -334,13 +322,14 @@ cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, cuda
     uint64_t sblocks = (n_s + kSampleThreads - 1) / kSampleThreads;
     const uint64_t scap = (uint64_t)device_sm_count() * 8;
     if (sblocks > scap) sblocks = scap;
-    if (single)
-        bucket_sample_kernel<true><<<(unsigned)sblocks, kSampleThreads, 0, s>>>(L);
-    else
-        bucket_sample_kernel<false><<<(unsigned)sblocks, kSampleThreads, 0, s>>>(L);
+    const bool strands = L.revcomp || L.strand_bits;
+    auto sample = single ? (strands ? bucket_sample_kernel<true, true> : bucket_sample_kernel<true, false>)
+                         : (strands ? bucket_sample_kernel<false, true> : bucket_sample_kernel<false, false>);
+    sample<<<(unsigned)sblocks, kSampleThreads, 0, s>>>(L);
     bucket_plan_kernel<<<1, 32, 0, s>>>(L);
     const uint64_t stiles = (L.n_q + kScatterTile - 1) / kScatterTile;
-    auto scatter = single ? bucket_scatter_kernel<true> : bucket_scatter_kernel<false>;
+    auto scatter = single ? (strands ? bucket_scatter_kernel<true, true> : bucket_scatter_kernel<true, false>)
+                          : (strands ? bucket_scatter_kernel<false, true> : bucket_scatter_kernel<false, false>);
     cudaError_t e = cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
     if (e != cudaSuccess) return e;
     scatter<<<(unsigned)stiles, kScatterThreads, kScatterSmem, s>>>(L, wrec_in);

@@ -40,9 +40,10 @@ struct FrontDesc {
 // P (bases 0-127 in w, the rest from qw; length m >= 1) against the pivot of
 // a k-mer entry: its first 192 bases in e (clamp of them exist), then the
 // text from position pos + 192 when all 192 tie.
+template <bool kStrands>
 __device__ __forceinline__ int cmp_entry(const uint64_t w[4], uint32_t m, const uint64_t e[6], uint32_t pos,
                                          uint32_t clamp, uint32_t n, const uint64_t *__restrict__ T,
-                                         const QueryWindows &qw, uint32_t *lcp) {
+                                         const QueryWindows<kStrands> &qw, uint32_t *lcp) {
 #pragma unroll
     for (int j = 0; j < 6; j++) {
         const uint32_t off = 32u * j;
@@ -78,7 +79,7 @@ __device__ __forceinline__ uint32_t list_slot(const uint32_t *prefix, const uint
 // kFromList: the queries come from the k-mer-ordered list of bucket.cu (one
 // 64-byte record each: length, index, reference, first base in the packed
 // batch and first 192 bases, already checked) instead of the batch's offsets.
-template <bool kSingle, bool kFromList>
+template <bool kSingle, bool kFromList, bool kStrands>
 __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_constant__ SearchLaunch a) {
     __shared__ FrontDesc sdesc[SA_MAX_REFS];
     __shared__ uint4 s_stage[kFrontThreads / 32][32][4];  // worklist records staged per warp
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
 
     const uint64_t n_items = kFromList ? (uint64_t)*a.wl_in_count : a.n_q;
     // a batch without a non-base byte needs no per-query validity check
-    const bool dirty = a.batch_dirty == nullptr || *a.batch_dirty != 0;
+    const bool dirty = *a.batch_dirty != 0;
     // Offsets and reference of this lane's next query, read one query ahead.
     uint64_t nqa = 0, nqe = 0;
     uint32_t nr = 0;
@@ -144,8 +145,8 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
             ldg32_if(live, src + 2, &c2, &c3);
             m = c0.x;
             q = c0.y;
-            qa = ((uint64_t)(c0.w & 0xFFFFu) << 32) | c0.z;
-            r = (c0.w >> 16) & 0x7FFFu;
+            qa = place_of(c0.z, c0.w);
+            r = ref_of(c0.w);
             entry = (c0.w & kListNeedsEntry) != 0u;
             w[0] = ((uint64_t)c1.y << 32) | c1.x;
             w[1] = ((uint64_t)c1.w << 32) | c1.z;
@@ -162,20 +163,19 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
                 nqe = __ldg(a.q_off + base + stride + lane + 1);
                 if (!kSingle) nr = __ldg(a.q_ref + base + stride + lane);
             }
-            const bool rc = a.revcomp || (a.strand_bits && (r & kStrandBit));
-            if (a.strand_bits) r &= ~kStrandBit;
+            const bool rc = kStrands && (a.revcomp || (a.strand_bits && (r & kStrandBit)));
+            if (kStrands && a.strand_bits) r &= ~kStrandBit;
             const bool range_ok = live && qa <= qe && qe <= a.total && qe - qa < (1ull << 31);
             if (live && !range_ok) any_bad = true;
             ok = range_ok && r < a.n_refs;
             if (range_ok && r >= a.n_refs) any_bad_ref = true;
             m = ok ? (uint32_t)(qe - qa) : 0u;
-            if (range_ok) qa = strand_start(qa, qe, a.total, rc, a.rc_base);
-
-            // First 128 bases and the validity of every base of the query.
-            if (!load_query_head(tq, a.tv, ok ? (qa >> 5) : 0, (uint32_t)(qa & 31u), m, ok && m > 0 && dirty, w)) {
+            if (ok && m > 0 && dirty && !query_valid(a.tvb, a.tv, qa, m)) {
                 ok = false;
                 any_bad = true;
             }
+            if (range_ok) qa = query_place(qa, qe, rc);
+            query_windows<4, kStrands>(tq, ok ? qa : 0, 0, w);  // first 128 bases
         }
 
         FrontDesc d = sdesc[0];
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         bool go = !done && look;
         // in list order, bases 128-191 are the record's last 16 bytes (read
         // again when a compare gets there: an L1 or L2 hit)
-        const QueryWindows qw{tq, qa, w[3],
+        const QueryWindows<kStrands> qw{tq, qa, w[3],
                               kFromList ? reinterpret_cast<const uint64_t *>(a.wrec_in + 4 * (size_t)lslot + 3)
                                         : nullptr,
                               kFromList ? 2u : 0u};
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
                                                      bd.phase == 1 ? bd.HR : bd.R, m, (uint32_t)q);
                 const uint64_t w4 = m > 128u ? qw(128u) : 0ull;  // bases 128-159 for the persistent pass
                 s_stage[wib][slot][1] =
-                    make_uint4((uint32_t)qa, (uint32_t)(qa >> 32) | (r << 16), (uint32_t)w4, (uint32_t)(w4 >> 32));
+                    make_uint4((uint32_t)qa, place_high(qa, r), (uint32_t)w4, (uint32_t)(w4 >> 32));
                 s_stage[wib][slot][2] =
                     make_uint4((uint32_t)w[0], (uint32_t)(w[0] >> 32), (uint32_t)w[1], (uint32_t)(w[1] >> 32));
                 s_stage[wib][slot][3] =
@@ -277,13 +277,19 @@ cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s) {
     if (L.n_q == 0) return cudaSuccess;
     const bool single = L.n_refs == 1 && L.q_ref == nullptr;
     const bool list = L.wrec_in != nullptr;
-    static int per_sm[4][64] = {};
+    const bool strands = L.revcomp || L.strand_bits;
+    static int per_sm[8][64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    auto kernel = single ? (list ? front_kernel<true, true> : front_kernel<true, false>)
-                         : (list ? front_kernel<false, true> : front_kernel<false, false>);
-    int &bps = per_sm[(single ? 1 : 0) + (list ? 2 : 0)][dev];
+    using Kernel = void (*)(SearchLaunch);
+    static const Kernel kernels[8] = {front_kernel<false, false, false>, front_kernel<true, false, false>,
+                                      front_kernel<false, true, false>,  front_kernel<true, true, false>,
+                                      front_kernel<false, false, true>,  front_kernel<true, false, true>,
+                                      front_kernel<false, true, true>,   front_kernel<true, true, true>};
+    const int which = (single ? 1 : 0) + (list ? 2 : 0) + (strands ? 4 : 0);
+    const Kernel kernel = kernels[which];
+    int &bps = per_sm[which][dev];
     if (bps == 0) {
         int b = 0;
         const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kFrontThreads, 0);

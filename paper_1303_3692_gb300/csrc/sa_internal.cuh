@@ -10,10 +10,14 @@
 //
 // Packed query batch: the bases of a whole batch (q_offsets[0] ..
 // q_offsets[n_q]) packed like a text, 32 per word, with SA_TQ_PAD_WORDS zero
-// words after the last, and one 32-bit mask per word whose bit i marks base
-// 32 w + i as not in {A,C,G,T,a,c,g,t}.  Query q's bases start at base
-// q_offsets[q] - q_offsets[0], so any of its 32-base windows is one
-// text_window read.
+// words after the last and room for SA_TQ_LEAD_WORDS words of no meaning
+// before the first.  Query q's bases start at base q_offsets[q] -
+// q_offsets[0], so any of its 32-base windows is one window read; a window of
+// its reverse complement is the window ending there, complemented and put in
+// reverse order (QueryWindow helpers below), so one packing serves both
+// strands.  A bitmap has bit w % 32 of word w / 32 set when packed word w
+// holds a byte that is not in {A,C,G,T,a,c,g,t}, and only those words have a
+// 32-bit mask, whose bit i marks base 32 w + i.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -22,6 +26,7 @@
 
 #define SA_PAD_WORDS 2
 #define SA_TQ_PAD_WORDS 6
+#define SA_TQ_LEAD_WORDS 6
 #define SA_MAX_REFS 64
 #define SA_MAX_KEY_DEPTH 14
 
@@ -47,12 +52,14 @@ struct RefDesc {
 // call's indexes, plus one bucket for queries without a k-mer bracket.
 constexpr uint32_t kNumBuckets = 256;
 // The k-mer-ordered list's 64-byte records (bucket.cu writes, front.cu reads):
-//   {m, q, qa.lo, qa.hi | ref << 16 | kListNeedsEntry}  length, index, first
-//       base in the packed batch (qa < 2^48), reference id (< 2^15), and
-//       whether the query has a k-mer bracket to read
+//   {m, q, at.lo, at.hi | ref << 16 | strand | kListNeedsEntry}  length, index,
+//       place in the packed batch (at < 2^48, and kRecordRc for the other
+//       strand), reference id (< 2^14), and whether the query has a k-mer
+//       bracket to read
 //   {w0, w1}, {w2, w3}, {w4, w5}  its first 192 bases as packed words (the
 //       words past the query's end are not its bases)
 constexpr uint32_t kListNeedsEntry = 0x80000000u;
+constexpr uint32_t kRecordRc = 0x40000000u;  // in list and worklist records
 constexpr uint64_t kListMaxBase = 1ull << 48;
 // The list's plan (bucket.cu), 32-bit words: every kListSampleStride-th
 // query's bucket counted; from those counts each bucket's region of the list
@@ -171,13 +178,69 @@ __device__ __forceinline__ uint64_t pack_word(const uint8_t *__restrict__ a, uin
 // q_ref bit 31 under SA_PARAM_STRAND_PER_QUERY: search the query's reverse complement.
 constexpr uint32_t kStrandBit = 0x80000000u;
 
-// A query's first base in the packed batch tq: its own range [qa, qe), or
-// for the other strand the mirrored range of the reverse-complement packing,
-// which starts at base rc_base of tq (base i of that packing is the
-// complement of batch base total - 1 - i).
-__device__ __forceinline__ uint64_t strand_start(uint64_t qa, uint64_t qe, uint64_t total, bool rc,
-                                                 uint64_t rc_base) {
-    return rc ? rc_base + (total - qe) : qa;
+// A query's place in the packed batch: its first base, or for the other
+// strand one past its last base with kPlaceRc set (base i of the reverse
+// complement is the complement of base end - 1 - i).
+constexpr uint64_t kPlaceRc = 1ull << 63;
+
+__device__ __forceinline__ uint64_t query_place(uint64_t qa, uint64_t qe, bool rc) { return rc ? qe | kPlaceRc : qa; }
+
+// The first base in the packed batch of a query of m bases at place at.
+__device__ __forceinline__ uint64_t place_first(uint64_t at, uint32_t m) {
+    return (at & kPlaceRc) ? (at & ~kPlaceRc) - m : at;
+}
+
+// The place's halves as list and worklist records hold them, with the reference.
+__device__ __forceinline__ uint32_t place_high(uint64_t at, uint32_t ref) {
+    return (uint32_t)((at & ~kPlaceRc) >> 32) | (ref << 16) | ((at & kPlaceRc) ? kRecordRc : 0u);
+}
+__device__ __forceinline__ uint64_t place_of(uint32_t lo, uint32_t hi) {
+    return ((uint64_t)(hi & 0xFFFFu) << 32) | lo | ((hi & kRecordRc) ? kPlaceRc : 0ull);
+}
+__device__ __forceinline__ uint32_t ref_of(uint32_t hi) { return (hi >> 16) & 0x3FFFu; }
+
+// The reverse complement of a window of 32 bases: every bit flipped and the
+// bits reversed, then the two bits of each code swapped back.
+__device__ __forceinline__ uint64_t rc_window(uint64_t x) {
+    const uint64_t f = __brevll(~x);
+    return ((f >> 1) & 0x5555555555555555ull) | ((f & 0x5555555555555555ull) << 1);
+}
+
+// The N 32-base windows of a query at bases off, off + 32, ... (N + 1 words
+// read; bits past the query are not its bases).  The other strand's windows
+// end at the query's place and may begin up to 31 + 32 (N - 1) bases before
+// the query, in the words before it (or the batch's lead words).  kStrands:
+// some query of the call may be of the other strand; a call of forward
+// queries only runs kernels without that branch (with it, 1571 -> 1668 us a
+// call of 1.6*10^7 queries over four genomes, 775 -> 819 us of 2^20 1024-base
+// ones).
+template <int N, bool kStrands>
+__device__ __forceinline__ void query_windows(const uint64_t *__restrict__ tq, uint64_t at, uint32_t off,
+                                              uint64_t w[N]) {
+    const bool rc = kStrands && (at & kPlaceRc) != 0;
+    const int64_t b = rc ? (int64_t)(at & ~kPlaceRc) - (int64_t)off - 32 * N : (int64_t)at + off;
+    const uint64_t *p = tq + (b >> 5);
+    const unsigned sh = (unsigned)(b & 31) * 2u;
+    uint64_t t[N + 1];
+#pragma unroll
+    for (int i = 0; i <= N; i++) t[i] = ldg_u64(p + i);
+#pragma unroll
+    for (int j = 0; j < N; j++) w[j] = (t[j] << sh) | ((t[j + 1] >> 1) >> (63u - sh));
+    if (rc) {
+#pragma unroll
+        for (int j = 0; j < (N + 1) / 2; j++) {
+            const uint64_t x = rc_window(w[j]), y = rc_window(w[N - 1 - j]);
+            w[j] = y;
+            w[N - 1 - j] = x;
+        }
+    }
+}
+
+template <bool kStrands>
+__device__ __forceinline__ uint64_t query_window(const uint64_t *__restrict__ tq, uint64_t at, uint32_t off) {
+    uint64_t w[1];
+    query_windows<1, kStrands>(tq, at, off, w);
+    return w[0];
 }
 
 // Bits [lo, hi) of a 32-bit mask (0 <= lo <= hi <= 32).
@@ -186,39 +249,24 @@ __device__ __forceinline__ uint32_t bit_range(uint32_t lo, uint32_t hi) {
     return upto & ~((1u << lo) - 1u);
 }
 
-// The head of a query of the packed batch: its first 128 bases as four
-// packed words w[0..3] (base 0 in the top bits of w[0]; bits past the query
-// hold the batch's next bases), read as five words from word w_lo = qa / 32
-// of tq with the shift of qa % 32.  With check set, returns whether all m
-// bases (from bit qa % 32 of word w_lo on) are marked valid in the per-word
-// masks tv; else returns true without reading the masks.
-__device__ __forceinline__ bool load_query_head(const uint64_t *__restrict__ tq, const uint32_t *__restrict__ tv,
-                                                uint64_t w_lo, uint32_t b0, uint32_t m, bool check,
-                                                uint64_t w[4]) {
-    const uint32_t sh = b0 * 2u;
-    uint64_t t[5];
-#pragma unroll
-    for (int i = 0; i < 5; i++) t[i] = __ldg(tq + w_lo + i);
-#pragma unroll
-    for (int j = 0; j < 4; j++) w[j] = (t[j] << sh) | ((t[j + 1] >> 1) >> (63u - sh));
-    if (!check) return true;
-    uint32_t v[5];
-#pragma unroll
-    for (int i = 0; i < 5; i++) v[i] = __ldg(tv + w_lo + i);
-    uint32_t badbits = 0;
-    const uint64_t end = (uint64_t)b0 + m;  // one past the query's last bit, from word w_lo
-#pragma unroll
-    for (int i = 0; i < 5; i++) {
-        const uint32_t lo = i == 0 ? b0 : 0u;
-        const uint64_t wend = 32ull * (i + 1);
-        const uint32_t hi = end >= wend ? 32u : (end > 32ull * i ? (uint32_t)(end - 32ull * i) : 0u);
-        if (hi > lo) badbits |= v[i] & bit_range(lo, hi);
+// Whether all m >= 1 bases from base qa of the batch on are bases: the bits of
+// their words in the bitmap tvb (one or two of its words for a query of up to
+// 1024 bases), then the masks tv of the few words that are marked.
+__device__ __forceinline__ bool query_valid(const uint32_t *__restrict__ tvb, const uint32_t *__restrict__ tv,
+                                            uint64_t qa, uint32_t m) {
+    const uint64_t w0 = qa >> 5, w1 = (qa + m - 1) >> 5;
+    for (uint64_t g = w0 >> 5; g <= (w1 >> 5); g++) {
+        uint32_t marked = __ldg(tvb + g);
+        if (g == (w0 >> 5)) marked &= 0xFFFFFFFFu << (w0 & 31u);
+        if (g == (w1 >> 5)) marked &= 0xFFFFFFFFu >> (31u - (uint32_t)(w1 & 31u));
+        for (; marked != 0u; marked &= marked - 1u) {
+            const uint64_t w = g * 32 + (__ffs(marked) - 1);
+            const uint32_t lo = w == w0 ? (uint32_t)(qa & 31u) : 0u;
+            const uint32_t hi = w == w1 ? (uint32_t)((qa + m - 1) & 31u) + 1u : 32u;
+            if (__ldg(tv + w) & bit_range(lo, hi)) return false;
+        }
     }
-    for (uint64_t i = 5; 32ull * i < end; i++) {  // queries longer than 128 bases
-        const uint32_t hi = end >= 32ull * (i + 1) ? 32u : (uint32_t)(end - 32ull * i);
-        badbits |= __ldg(tv + w_lo + i) & bit_range(0, hi);
-    }
-    return badbits == 0;
+    return true;
 }
 
 // One query's result, written as one 32-byte store (a whole DRAM sector, so a
@@ -454,9 +502,10 @@ struct Bounds {
     __device__ __forceinline__ uint32_t first() const { return phase == 0 ? R : lo; }
 };
 
-// Query P (length m >= 1, bases at base qa of the packed batch tq) against
+// Query P (length m >= 1, at place qa of the packed batch tq) against
 // the suffix at p of a text of n < 2^32 bases, from the 32-aligned base below
 // `start` (< m; all bases before it are known equal).
+template <bool kStrands>
 __device__ __forceinline__ int cmp_suffix_tq(const uint64_t *__restrict__ T, uint32_t n, uint32_t p,
                                              const uint64_t *__restrict__ tq, uint64_t qa, uint32_t m,
                                              uint32_t start, uint32_t *lcp) {
@@ -465,7 +514,7 @@ __device__ __forceinline__ int cmp_suffix_tq(const uint64_t *__restrict__ T, uin
     for (;;) {
         const uint32_t qlen = min(32u, m - off);
         const uint32_t tlen = off < rem ? min(32u, rem - off) : 0u;
-        const uint64_t q = text_window(tq, qa + off);
+        const uint64_t q = query_window<kStrands>(tq, qa, off);
         const uint64_t t = tlen ? text_window(T, (uint64_t)(p + off)) : 0ull;
         const int c = cmp_window(q, t, qlen, tlen, off, m, lcp);
         if (c != 2) return c;
@@ -477,6 +526,7 @@ __device__ __forceinline__ int cmp_suffix_tq(const uint64_t *__restrict__ T, uin
 // 96 from w3 (the query's fourth packed word), bases 128 .. 128 + 32
 // tail_words - 1 from `tail` (later words its record carries, read again from
 // the record when a compare gets there), the rest from the packed batch.
+template <bool kStrands>
 struct QueryWindows {
     const uint64_t *tq;
     uint64_t qa;
@@ -486,13 +536,14 @@ struct QueryWindows {
     __device__ __forceinline__ uint64_t operator()(uint32_t off) const {
         if (off == 96u) return w3;
         if (off >= 128u && ((off - 128u) >> 5) < tail_words) return __ldg(tail + ((off - 128u) >> 5));
-        return text_window(tq, qa + off);
+        return query_window<kStrands>(tq, qa, off);
     }
 };
 
 // cmp_suffix_tq with the query's windows from qw (start >= 96).
+template <bool kStrands>
 __device__ __forceinline__ int cmp_suffix_qw(const uint64_t *__restrict__ T, uint32_t n, uint32_t p,
-                                             const QueryWindows &qw, uint32_t m, uint32_t start, uint32_t *lcp) {
+                                             const QueryWindows<kStrands> &qw, uint32_t m, uint32_t start, uint32_t *lcp) {
     uint32_t off = start & ~31u;
     const uint32_t rem = n - p;
     for (;;) {
@@ -570,8 +621,9 @@ struct SearchLaunch {
     uint32_t n_refs;
     uint32_t width;
     const char *ascii;        // query bases, indexed by q_off[q] - first
-    const uint64_t *tq;       // packed batch: nwords + SA_TQ_PAD_WORDS words
-    const uint32_t *tv;       // per packed word: bit i set = base 32 w + i is not a base
+    const uint64_t *tq;       // packed batch: SA_TQ_LEAD_WORDS before it, nwords + SA_TQ_PAD_WORDS from it on
+    const uint32_t *tvb;      // bitmap of the packed words that hold a byte that is not a base
+    const uint32_t *tv;       // masks of those words: bit i set = base 32 w + i is not a base
     uint64_t nwords;          // ceil(total / 32)
     const uint64_t *q_off;    // n_q + 1 offsets
     uint64_t first;           // q_off[0]
@@ -585,17 +637,15 @@ struct SearchLaunch {
     sa_result *out;
     int *pack_err;            // device flag: some query had a non-ACGT byte or bad offsets
     int *batch_dirty;         // device flag set by the packing: some byte of the batch is not a base
-                              // (null: assume so).  With the flag, tv holds every mask only for a batch
-                              // that is not clean; a clean batch needs (and has) none.
+                              // (a clean batch's bitmap and masks need not be read)
     int *bad_ref;             // device flag: some query named a reference id >= n_refs
     unsigned long long *counter;
     int *status;
     uint32_t smem_bytes;      // shared-memory key tables
     uint32_t threads, blocks, chunk;
     uint32_t front_probes;    // probes per query in the first pass
-    bool revcomp;             // search every query's reverse complement (the batch is packed reversed)
-    bool strand_bits;         // q_ref bit 31 selects each query's strand (both packings in tq)
-    uint64_t rc_base;         // first base of the reverse-complement packing in tq (0: it is the only one)
+    bool revcomp;             // search every query's reverse complement
+    bool strand_bits;         // q_ref bit 31 selects each query's strand
     bool expire_waits;        // test hook: the bounded key-table wait gives up at once
     uint32_t trunc_cap;       // the locate cap of sa_search_locate (SA_RESULT_TRUNCATED), else ~0u
     // k-mer order (bucket.cu)
@@ -634,11 +684,12 @@ __device__ __forceinline__ void store_result_sum(const SearchLaunch &a, uint64_t
 // Worklist record of a query the first pass did not finish (64 bytes):
 //   {L, R, m, q}            a bracket (L, R) holding both bounds (L = -1 is
 //                           0xFFFFFFFF), the length and the query's index
-//   {qa.lo, qa.hi | ref << 16, w4.lo, w4.hi}  its first base in the packed
-//                           batch (qa < 2^48), reference id (< 2^15) and
-//                           bases 128-159
+//   {at.lo, at.hi | ref << 16 | strand, w4.lo, w4.hi}  its place in the packed
+//                           batch (at < 2^48, and kRecordRc for the other
+//                           strand), reference id (< 2^14), bases 128-159
 //   {w0, w1}, {w2, w3}      its first 128 bases (packed words)
-cudaError_t launch_pack_batch(const SearchLaunch &L, uint64_t *tq, uint32_t *tv, cudaStream_t s);
+// Packs L.ascii; tvb is zero before, or null (then tv receives every word's mask).
+cudaError_t launch_pack_batch(const SearchLaunch &L, uint64_t *tq, uint32_t *tvb, uint32_t *tv, cudaStream_t s);
 cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s);
 // The batch's queries as records in k-mer order (wrec_in), the first pass's
 // input in that order.

@@ -160,7 +160,7 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s for the key-table copy
 // chunk's base fetched while the previous chunk is handed out.
 // Launch bounds: 1024 threads, one CTA per SM, at most 64 registers (no
 // spills); smaller CTAs may share an SM up to 1024 threads in all.
-template <typename IdxT, bool kSingle>
+template <typename IdxT, bool kSingle, bool kStrands>
 __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__ SearchLaunch a) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ SmemDesc sdesc[SA_MAX_REFS];
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
         if (init) {
             fresh = false;
             qout = r0.w;
-            const uint32_t r = (r1.y >> 16) & 0x7FFFu;
+            const uint32_t r = ref_of(r1.y);
             if (!kSingle) {
                 const SmemDesc d = sdesc[r < a.n_refs ? r : 0u];
                 T = d.text;
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
                 depth = d.depth;
             }
             m = r0.z;
-            qa = ((uint64_t)(r1.y & 0xFFFFu) << 32) | r1.x;
+            qa = place_of(r1.x, r1.y);
             q0 = x2;
             q1 = x3;
             bd.start(r0.x, r0.y);
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             const uint32_t klen = Ktab[(16u << depth) + k];
             bool und = false;
             c = cmp_key(q0, q1, m, kv, klen, &l, &und);
-            if (und) c = cmp_suffix_tq(T, n, (uint32_t)sa_at<IdxT>(SAp, M), a.tq, qa, m, 64u, &l);
+            if (und) c = cmp_suffix_tq<kStrands>(T, n, (uint32_t)sa_at<IdxT>(SAp, M), a.tq, qa, m, 64u, &l);
             const uint32_t nk = 2u * k + (c == CMP_GREATER ? 1u : 0u);
             k = (c == CMP_PREFIX || nk >= (1u << depth)) ? 0u : nk;
         } else {
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             c = cmp_record(q0, q1, x2, x3, m, r0, r1, n, &l, &und);
             if (und) {
                 // query bases 96-127 are x3, 128-159 the worklist record's second word pair
-                const QueryWindows qw{a.tq, qa, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};
+                const QueryWindows<kStrands> qw{a.tq, qa, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};
                 c = cmp_suffix_qw(T, n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
             }
             lp = (r1.z >> 8) & 0xFFu;
@@ -341,24 +341,13 @@ template <typename IdxT>
 __global__ void __launch_bounds__(256) search_plain_kernel(const __grid_constant__ SearchLaunch a) {
     const uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= a.n_q) return;
-    uint64_t a0 = __ldg(a.q_off + q) - a.first;
-    uint64_t a1 = __ldg(a.q_off + q + 1) - a.first;
-    uint32_t r = a.q_ref ? __ldg(a.q_ref + q) : 0u;
-    const bool rc = a.revcomp || (a.strand_bits && (r & kStrandBit));
-    if (a.strand_bits) r &= ~kStrandBit;
-    const bool range_ok = a0 <= a1 && a1 <= a.total && a1 - a0 < (1ull << 31);
-    if (range_ok) {  // the other strand sits at the mirrored range of its packing
-        const uint64_t len = a1 - a0;
-        a0 = strand_start(a0, a1, a.total, rc, a.rc_base);
-        a1 = a0 + len;
-    }
-    bool bad = !range_ok;
+    const uint64_t a0 = __ldg(a.q_off + q) - a.first;
+    const uint64_t a1 = __ldg(a.q_off + q + 1) - a.first;
+    const uint32_t r = a.q_ref ? __ldg(a.q_ref + q) : 0u;
+    bool bad = !(a0 <= a1 && a1 <= a.total && a1 - a0 < (1ull << 31));
     // every base of the query must be one of A, C, G, T (nothing to check in
     // a batch the packing found clean)
-    if (range_ok && (a.batch_dirty == nullptr || *a.batch_dirty != 0)) {
-        for (uint64_t b = a0; b < a1; b++)
-            if ((__ldg(a.tv + (b >> 5)) >> (b & 31u)) & 1u) bad = true;
-    }
+    if (!bad && a1 > a0 && *a.batch_dirty != 0) bad = !query_valid(a.tvb, a.tv, a0, (uint32_t)(a1 - a0));
     if (bad || r >= a.n_refs) {
         if (bad) atomicOr(a.pack_err, 1);
         if (!bad) atomicOr(a.bad_ref, 1);
@@ -455,7 +444,10 @@ cudaError_t launch_search(const SearchLaunch &L, cudaStream_t s) {
     auto pick = [&](auto idx_tag, auto single_tag) {
         using I = decltype(idx_tag);
         constexpr bool S = decltype(single_tag)::value;
-        go(search_kernel<I, S>);
+        if (L.revcomp || L.strand_bits)
+            go(search_kernel<I, S, true>);
+        else
+            go(search_kernel<I, S, false>);
     };
     if (L.width == 4)
         single ? pick(uint32_t{}, std::true_type{}) : pick(uint32_t{}, std::false_type{});

@@ -362,7 +362,7 @@ int sa_stree_search(const sa_stree *t, const char *q_bases, const uint64_t *q_of
         L.ascii = q_bases ? q_bases + fl[0] : nullptr;
         L.total = total;
         L.nwords = nwords;
-        e = launch_pack_batch(L, tq, tv, s);
+        e = launch_pack_batch(L, tq, nullptr, tv, s);
     }
     if (e == cudaSuccess) {
         const unsigned blocks = (unsigned)((n_q + kThreads - 1) / kThreads);

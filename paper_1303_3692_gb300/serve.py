@@ -53,14 +53,15 @@ class Request:
 
 def scratch_bytes(n_q: int, n_bases: int, both_strands: bool = False) -> int:
     """Device scratch one search call takes from the library's pool, at most:
-    the packed batch (8 bytes per 32 bases) and its validity masks (4 bytes
-    per 32 bases), twice when queries name their strands; 64 bytes of worklist
-    room per query; in k-mer order the ordered list (64-byte records, room
-    for about 2.125 per query plus 257 * 256); small flags, and 256 bytes of
-    alignment per allocation."""
-    words = ((n_bases + 31) // 32 + 6) * (2 if both_strands else 1)
+    the packed batch (8 bytes per 32 bases), its validity masks (4 bytes per 32
+    bases) and the bitmap of words that have one (a bit per 32 bases); 64
+    bytes of worklist room per query; in k-mer order the ordered list (64-byte
+    records, room for about 2.125 per query plus 257 * 256); small flags, and
+    256 bytes of alignment per allocation.  Queries of both strands
+    (both_strands) take no more: they are read from one packing."""
+    words = (n_bases + 31) // 32 + 12
     listed = ((n_q + 32) * 9 // 8 + 256 * 257 + n_q) * 64
-    return 12 * words + 64 * n_q + listed + 1288 * 4 + 80 + 8 * 256
+    return 12 * words + words // 8 + 4 + 64 * n_q + listed + 1288 * 4 + 80 + 8 * 256
 
 
 def kept(counts: np.ndarray, cap: int) -> np.ndarray:
