@@ -97,7 +97,8 @@ typedef struct sa_search_params {
     uint32_t threads_per_block; /* 32..1024, multiple of 32 */
     uint32_t blocks_per_sm;     /* persistent CTAs per SM (at most 1024 threads per SM in all:
                                    larger requests are reduced to that) */
-    uint32_t key_depth;         /* shared-memory key-table depth d (<= the index's) */
+    uint32_t key_depth;         /* shared-memory key-table depth d (<= the index's) of the
+                                   indexes without a k-mer table */
     uint32_t chunk;             /* queries a warp takes from the global counter at once */
     void *search_events[2];     /* optional cudaEvent_t pair, recorded on the stream right
                                    before and after the search kernel (kernel timing) */
@@ -233,9 +234,9 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
  * The work runs as three kernels on the stream: the batch's bases are packed
  * 2 bits each beside a per-base validity mask; a one-thread-per-query pass
  * brackets each query of m >= k bases by the k-mer table and probes it up to
- * sa_search_params.front_probes times; a persistent kernel finishes the
- * queries that remain (and every query of an index without a k-mer table or
- * shorter than k).  Scratch device memory from the library pool: about
+ * sa_search_params.front_probes times, and answers a shorter query from the
+ * table's counts; a persistent kernel finishes the queries that remain (and
+ * every query of an index without a k-mer table).  Scratch device memory from the library pool: about
  * 12 * ceil(total / 32) + 64 n_q bytes (total = the batch's bases), plus the
  * staging copies of host inputs.
  *

@@ -194,13 +194,14 @@ int check_refs(const sa_index *const *refs, uint32_t n_refs, uint32_t *width) {
     return SA_OK;
 }
 
-// Per-index table depths for one call: each index's own depth, capped by the
-// request, then the deepest tables are trimmed until all fit the budget.
+// Per-index table depths for one call: none for an index with a k-mer table
+// (its queries start from their k-mer bracket), else the index's own depth
+// capped by the request, then the deepest tables are trimmed until all fit the budget.
 uint32_t fill_ref_table(const sa_index *const *refs, uint32_t n_refs, uint32_t want_depth, RefTable *t,
                         uint32_t budget = kSmemBudget) {
     uint32_t use[SA_MAX_REFS];
     for (uint32_t r = 0; r < n_refs; r++) {
-        use[r] = refs[r]->depth < want_depth ? refs[r]->depth : want_depth;
+        use[r] = refs[r]->krt ? 0 : (refs[r]->depth < want_depth ? refs[r]->depth : want_depth);
     }
     for (;;) {
         uint32_t total = 0, deepest = 0;

@@ -2,10 +2,9 @@
 //
 // search_kernel (second pass of the product path).  Persistent CTAs, one
 //   query of the first pass's worklist per lane (the queries front_kernel
-//   did not finish: wide brackets, queries shorter than k, indexes without a
-//   k-mer table).
-//   * Each CTA first copies every index's sampled-key table into shared
-//     memory with bulk asynchronous copies (cp.async.bulk, completion on an
+//   did not finish: wide brackets, indexes without a k-mer table).
+//   * Each CTA first copies the sampled-key table of every index without a
+//     k-mer table into shared memory with bulk asynchronous copies (cp.async.bulk, completion on an
 //     mbarrier with a bounded wait).  The table holds the first 64 bases of
 //     the suffixes at ranks floor((2p+1) n / 2^(l+1)) in level order, so
 //     walking it is the first d levels of the binary search, in shared
@@ -41,7 +40,6 @@ struct SmemDesc {
     uint64_t n;
     uint32_t off;
     uint32_t depth;
-    uint32_t kmer_k;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -171,7 +169,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
 
     for (unsigned r = tid; r < a.n_refs; r += blockDim.x) {
         const RefDesc &d = a.refs.r[r];
-        sdesc[r] = SmemDesc{d.text, d.sa, d.rec, d.krt, d.n, d.smem_off, d.use_depth, d.kmer_k};
+        sdesc[r] = SmemDesc{d.text, d.sa, d.rec, d.krt, d.n, d.smem_off, d.use_depth};
     }
     if (tid == 0) {
         mbar_init(&mbar, 1);
@@ -208,7 +206,6 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
     const void *SAp = d0.sa;
     const uint4 *REC = d0.rec;
     const uint4 *KM = d0.krt;
-    uint32_t kk = d0.kmer_k;
     uint32_t n = (uint32_t)d0.n;
     const uint8_t *Ktab = smem + d0.off;
     uint32_t depth = d0.depth;
@@ -273,7 +270,6 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
                 SAp = d.sa;
                 REC = d.rec;
                 KM = d.krt;
-                kk = d.kmer_k;
                 n = (uint32_t)d.n;
                 Ktab = smem + d.off;
                 depth = d.depth;
@@ -283,7 +279,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             q0 = x2;
             q1 = x3;
             bd.start(r0.x, r0.y);
-            k = (KM != nullptr && m >= kk) ? 0u : (depth ? 1u : 0u);
+            k = KM != nullptr ? 0u : (depth ? 1u : 0u);
             continue;
         }
 
