@@ -449,9 +449,9 @@ uint32_t auto_kmer_k(uint64_t n) {
 }
 
 // Allocates the device arrays of an index whose n, width, depth and kmer_k
-// are set: first the text, suffix array and key table; the records (32n
-// bytes) and the k-mer table (64 * 4^k bytes) are allocated separately,
-// after the build's scratch has been returned, so the two never coexist.
+// are set: the text, suffix array and key table here; the records (32n bytes)
+// and the k-mer table (64 * 4^k bytes) in alloc_search_arrays, before the
+// suffix array is built when they also serve as that build's scratch.
 int alloc_index(sa_index *idx) {
     idx->nwords = (idx->n + 31) / 32;
     const size_t tb = (idx->nwords + SA_PAD_WORDS) * sizeof(uint64_t);
@@ -574,6 +574,17 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
             return SA_ERR_BASE;
         }
     }
+    // Prefix doubling takes its scratch (46n bytes) from the records and the
+    // k-mer table, which are not written before the suffix array is there
+    // (32n + 64 * 4^k bytes, at least 80n with the automatic k below 15):
+    // mapping that much into the pool and trimming it again for every build
+    // took 17 of 49 ms at 10^8 bases.  The other constructions' scratch is
+    // returned first, so that it never coexists with the two.
+    const bool scratch_in_place = !(flags & (SA_BUILD_HOST | SA_BUILD_DC3));
+    if (scratch_in_place && (st = alloc_search_arrays(idx)) != SA_OK) {
+        free_index(idx);
+        return st;
+    }
     if (flags & SA_BUILD_HOST) {
         std::vector<char> copy;
         const char *host_text = text;
@@ -596,11 +607,14 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
     } else if (flags & SA_BUILD_DC3) {
         st = build_suffix_array_dc3(idx, s);
     } else {
-        st = build_suffix_array(idx, s);
+        Arena arenas[2] = {{reinterpret_cast<char *>(idx->rec), idx->n * 2 * sizeof(uint4)}, {nullptr, 0}};
+        if (idx->krt)
+            arenas[1] = {reinterpret_cast<char *>(idx->krt), (1ull << (2 * idx->kmer_k)) * 4 * sizeof(uint4)};
+        st = build_suffix_array(idx, s, arenas, 2);
     }
     cudaStreamSynchronize(s);
     cudaMemPoolTrimTo(scratch_pool(idx->device), 0);
-    if (st == SA_OK) st = alloc_search_arrays(idx);
+    if (st == SA_OK && !scratch_in_place) st = alloc_search_arrays(idx);
     if (st == SA_OK) {
         cudaError_t err = launch_build_keys(idx, s);
         if (err == cudaSuccess) err = launch_build_records(idx, s);
@@ -1177,7 +1191,7 @@ int sa_suffix_array_gpu(const char *text, uint64_t n, uint32_t width, uint32_t f
         if (err == cudaSuccess) err = cudaStreamSynchronize(s);
         if (err != cudaSuccess) return status_from_cuda(err);
         if (hflag) return SA_ERR_BASE;
-        st = (flags & SA_BUILD_DC3) ? build_suffix_array_dc3(&tmp, s) : build_suffix_array(&tmp, s);
+        st = (flags & SA_BUILD_DC3) ? build_suffix_array_dc3(&tmp, s) : build_suffix_array(&tmp, s, nullptr, 0);
         cudaStreamSynchronize(s);
     }
     cudaMemPoolTrimTo(scratch_pool(tmp.device), 0);

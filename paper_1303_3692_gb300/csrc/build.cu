@@ -105,12 +105,22 @@ int bit_length(uint64_t x) {
 
 struct Pool {
     cudaStream_t s;
+    Arena *arenas = nullptr;
+    int n_arenas = 0;
     std::vector<void *> ptrs;
     cudaError_t err = cudaSuccess;
     template <typename T>
     T *get(size_t count) {
         void *p = nullptr;
         if (err != cudaSuccess) return nullptr;
+        const size_t need = (count * sizeof(T) + 255) / 256 * 256;
+        for (int i = 0; i < n_arenas; i++) {
+            if (arenas[i].left < need) continue;
+            p = arenas[i].at;
+            arenas[i].at += need;
+            arenas[i].left -= need;
+            return reinterpret_cast<T *>(p);
+        }
         err = scratch_alloc(&p, count * sizeof(T) + 16, s);
         if (err == cudaSuccess) ptrs.push_back(p);
         return reinterpret_cast<T *>(p);
@@ -128,9 +138,9 @@ struct Pool {
         if (e_ != cudaSuccess) return status_from_cuda(e_); \
     } while (0)
 
-int build_suffix_array(sa_index *idx, cudaStream_t s) {
+int build_suffix_array(sa_index *idx, cudaStream_t s, Arena *arenas, int n_arenas) {
     const uint64_t n = idx->n;
-    Pool pool{s};
+    Pool pool{s, arenas, n_arenas};
     uint64_t *kA = pool.get<uint64_t>(n), *kB = pool.get<uint64_t>(n);
     uint32_t *vA = pool.get<uint32_t>(n), *vB = pool.get<uint32_t>(n);
     uint32_t *isa = pool.get<uint32_t>(n), *sa32 = pool.get<uint32_t>(n);

@@ -602,7 +602,13 @@ int device_sm_count();
 // Kernels launched from the API translation unit.
 cudaError_t launch_pack_text(const char *ascii, uint64_t n, uint64_t *words, uint64_t nwords_padded,
                              int *err_flag, cudaStream_t s);
-int build_suffix_array(sa_index *idx, cudaStream_t s);
+// A stretch of device memory a build may use as scratch (no longer than the call).
+struct Arena {
+    char *at;
+    size_t left;
+};
+// Scratch comes from the arenas (may be null) while they last, then from the pool.
+int build_suffix_array(sa_index *idx, cudaStream_t s, Arena *arenas, int n_arenas);
 // The same array by the paper's DC3 construction, on the GPU (dc3_gpu.cu).
 int build_suffix_array_dc3(sa_index *idx, cudaStream_t s);
 cudaError_t launch_build_keys(sa_index *idx, cudaStream_t s);
