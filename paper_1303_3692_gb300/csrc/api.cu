@@ -555,7 +555,7 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
         Scratch sc{s};
         cudaError_t err = cudaSuccess;
         const char *text_d = device_view(text, n, sc, &err);
-        int *flag = sc.get<int>(1);
+        int *flag = reinterpret_cast<int *>(idx->keys);  // the key table is written later
         if (sc.failed) {
             free_index(idx);
             return SA_ERR_NOMEM;

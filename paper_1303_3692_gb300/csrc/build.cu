@@ -383,33 +383,60 @@ __global__ void build_kmer_kernel(const uint4 *__restrict__ rec, uint64_t n, uin
 //     common prefixes with the ranks beside it;
 //   three uint4: the first 192 bases of that suffix as six packed words.
 // One aligned 64-byte read therefore brackets a query of m >= k bases and
-// makes its first probe.
-__global__ void build_krt_kernel(const uint32_t *__restrict__ kmer, const uint4 *__restrict__ rec,
-                                 const uint64_t *__restrict__ T, uint64_t n, uint32_t k, uint4 *__restrict__ krt) {
-    const uint64_t entries = 1ull << (2 * k);
-    GS_LOOP(x, entries) {
-        const uint32_t lo = kmer[x], hi = kmer[x + 1];
-        uint4 h = make_uint4(lo, hi, 0u, 0u);
-        uint64_t e[6] = {0, 0, 0, 0, 0, 0};
-        if (hi > lo) {
-            const uint32_t M = lo + (hi - lo + 1u) / 2u - 1u;
-            const uint4 r1 = rec[2 * (uint64_t)M + 1];
-            const uint64_t pos = r1.w;
-            const uint64_t left = n - pos;  // >= 1
-            h.z = (uint32_t)pos;
-            h.w = (uint32_t)(left < 192 ? left : 192) | (((r1.z >> 8) & 0xFFu) << 8) | ((r1.z & 0xFFu) << 16);
+// makes its first probe.  The pivot's record gives its first 96 bases, so only
+// the second 96 are read from the text (random; the records are read in
+// order), and each half entry is one 32-byte store: 10^8 bases (17 GB of
+// entries) 5.2 -> 3.9 ms against six text windows and four 16-byte stores,
+// 6*10^8 (69 GB) 23.7 -> 21.1 ms, bound there by the text reads.
+__device__ __forceinline__ void st32(void *p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
+    asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+
+__device__ __forceinline__ void write_krt_entry(uint64_t x, uint32_t lo, uint32_t hi, const uint4 *__restrict__ rec,
+                                                const uint64_t *__restrict__ T, uint64_t n, uint4 *krt) {
+    uint64_t pos = 0, e[6] = {0, 0, 0, 0, 0, 0};
+    uint32_t last = 0;
+    if (hi > lo) {
+        const uint32_t M = lo + (hi - lo + 1u) / 2u - 1u;
+        uint4 r0, r1;
+        ldg32(rec + 2 * (uint64_t)M, &r0, &r1);
+        pos = r1.w;
+        const uint64_t left = n - pos;  // >= 1
+        last = (uint32_t)(left < 192 ? left : 192) | (((r1.z >> 8) & 0xFFu) << 8) | ((r1.z & 0xFFu) << 16);
+        e[0] = ((uint64_t)r0.y << 32) | r0.x;
+        e[1] = ((uint64_t)r0.w << 32) | r0.z;
+        e[2] = ((uint64_t)r1.y << 32) | r1.x;
 #pragma unroll
-            for (int j = 0; j < 6; j++) {
-                const uint64_t b = pos + 32ull * j;
-                e[j] = b < n ? text_window(T, b) : 0ull;
-            }
+        for (int i = 3; i < 6; i++) {
+            const uint64_t b = pos + 32ull * i;
+            e[i] = b < n ? text_window(T, b) : 0ull;
         }
-        uint4 *dst = krt + 4 * x;
-        dst[0] = h;
-        dst[1] = make_uint4((uint32_t)e[0], (uint32_t)(e[0] >> 32), (uint32_t)e[1], (uint32_t)(e[1] >> 32));
-        dst[2] = make_uint4((uint32_t)e[2], (uint32_t)(e[2] >> 32), (uint32_t)e[3], (uint32_t)(e[3] >> 32));
-        dst[3] = make_uint4((uint32_t)e[4], (uint32_t)(e[4] >> 32), (uint32_t)e[5], (uint32_t)(e[5] >> 32));
     }
+    uint4 *dst = krt + 4 * x;
+    st32(dst, ((uint64_t)hi << 32) | lo, ((uint64_t)last << 32) | pos, e[0], e[1]);
+    st32(dst + 2, e[2], e[3], e[4], e[5]);
+}
+
+// Entries [first, end) from the counts kmer[first .. end], which no entry of
+// this launch is written over.
+__global__ void build_krt_kernel(const uint32_t *kmer, const uint4 *__restrict__ rec, const uint64_t *__restrict__ T,
+                                 uint64_t n, uint64_t first, uint64_t end, uint4 *krt) {
+    GS_LOOP(j, end - first) write_krt_entry(first + j, kmer[first + j], kmer[first + j + 1], rec, T, n, krt);
+}
+
+// The last entries, at most one per thread of the one block: every count is
+// read before any entry is written over it.
+__global__ void build_krt_last_kernel(const uint32_t *kmer, const uint4 *__restrict__ rec,
+                                      const uint64_t *__restrict__ T, uint64_t n, uint64_t first, uint64_t end,
+                                      uint4 *krt) {
+    const uint64_t x = first + threadIdx.x;
+    uint32_t lo = 0, hi = 0;
+    if (x < end) {
+        lo = kmer[x];
+        hi = kmer[x + 1];
+    }
+    __syncthreads();
+    if (x < end) write_krt_entry(x, lo, hi, rec, T, n, krt);
 }
 
 // The plain counts kmer[x] = lo of every entry, and kmer[4^k] = n.
@@ -420,19 +447,24 @@ __global__ void krt_lo_kernel(const uint4 *__restrict__ krt, uint64_t n, uint32_
 
 cudaError_t launch_build_kmer(sa_index *idx, cudaStream_t s) {
     if (!idx->krt) return cudaSuccess;
+    // The counts kmer[0 .. 4^k] wait in the end of the entries' own memory, so
+    // that they need none of their own (4.3 GB at k = 15, mapped and unmapped
+    // for every build).  Each launch writes the entries from s on that lie
+    // before the counts from s on, all but a sixteenth of the rest, and the
+    // counts of those it wrote are free to be written over by the next.
+    constexpr uint64_t kLast = 256;
     const uint64_t entries = 1ull << (2 * idx->kmer_k);
-    uint32_t *kmer = nullptr;
-    cudaError_t e = scratch_alloc(reinterpret_cast<void **>(&kmer), (entries + 1) * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    uint32_t *kmer = reinterpret_cast<uint32_t *>(idx->krt) + 16 * entries - (entries + 1);
     build_kmer_kernel<<<grid_for(idx->n + 1), kThreads, 0, s>>>(idx->rec, idx->n, idx->kmer_k, kmer);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) {
-        build_krt_kernel<<<grid_for(entries), kThreads, 0, s>>>(kmer, idx->rec, idx->text, idx->n, idx->kmer_k,
-                                                                idx->krt);
-        e = cudaGetLastError();
+    uint64_t done = 0;
+    while (entries - done > kLast) {
+        const uint64_t end = entries - (entries - done + 1 + 15) / 16;
+        build_krt_kernel<<<grid_for(end - done), kThreads, 0, s>>>(kmer, idx->rec, idx->text, idx->n, done, end,
+                                                                   idx->krt);
+        done = end;
     }
-    scratch_free(kmer, s);
-    return e;
+    build_krt_last_kernel<<<1, kLast, 0, s>>>(kmer, idx->rec, idx->text, idx->n, done, entries, idx->krt);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_copy_kmer_counts(const sa_index *idx, uint32_t *dst, cudaStream_t s) {
