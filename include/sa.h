@@ -178,8 +178,8 @@ typedef struct sa_search_params {
  *
  * Packs the bases 2 bits each (A=0, C=1, G=2, T=3, base 0 in the most
  * significant bits of each 64-bit word), builds the suffix array of the text
- * on the GPU by prefix doubling (radix sorts of rank pairs; the result is the
- * unique suffix array of Table I's definition) -- or, with SA_BUILD_HOST, on
+ * on the GPU by prefix doubling (radix sorts of short prefixes and then of
+ * rank pairs; the result is the unique suffix array of Table I's definition) -- or, with SA_BUILD_HOST, on
  * the host by DC3 as Section III does -- and derives the structures
  * the search reads:
  *  - the key table kept in shared memory (first 64 bases of the suffixes at

@@ -4,15 +4,28 @@
 //
 // The paper builds its suffix array on the host (the straightforward sort or
 // DC3, Section III).  Here the text is already packed in device memory, so
-// the array is built there: every suffix is first ranked by its first 29
-// bases (58 bits of packed text plus a 6-bit length that puts a proper prefix
-// first, the order of Table I).  Then, while some group of equal ranks has
-// more than one member, only the members of such groups are re-sorted by the
-// pair (rank[i], rank[i + h]) and h doubles.  Ranks are the suffix-array
-// position of the first member of the group, so they order groups globally
-// and a finished group's rank is its final position.  The radix sorts, scans
-// and compactions come from CUB (a source-only library shipped with the CUDA
-// toolkit); the key computation, rank scatter and key table are kernels here.
+// the array is built there, by radix sorts of short keys that leave few
+// suffixes to look at again (build_suffix_array):
+//   1. all suffixes are sorted by their first 16 bases (a 32-bit key: 16 bytes
+//      moved per suffix and pass, four passes);
+//   2. a group of at most 32 suffixes that are still equal is ordered by
+//      comparing them in the text, each with the others (refine_kernel), and
+//      only larger groups, or suffixes that stay equal for long, go on;
+//   3. those are sorted by (their group, their next ~20 bases), and refined
+//      again, round by round, while that is cheaper than what follows;
+//   4. what then remains (long repeats) goes through prefix doubling: the ranks
+//      of all suffixes are written out, the remaining ones re-sorted by the
+//      pair (rank[i], rank[i + h]), h the depth the order is known to, and h
+//      doubles.  Ranks are the suffix-array position of the first member of
+//      the group, so they order groups globally and a finished group's rank
+//      is its final position.
+// A suffix that ends within the compared bases is packed with A's (zeros)
+// after its end; it sorts before every other suffix with the same key, the
+// shorter of two such first (the order of Table I).  The first sort starts
+// from descending text positions and every sort is stable, so they come in
+// that order by themselves, and each counts as a group of its own.
+// The radix sorts, scans and compactions come from CUB (a source-only library
+// shipped with the CUDA toolkit); the rest are kernels here.
 #include <cub/cub.cuh>
 #include <thrust/iterator/counting_iterator.h>
 #include <vector>
@@ -36,36 +49,191 @@ unsigned grid_for(uint64_t n) {
 #define GS_LOOP(i, n) \
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (uint64_t)gridDim.x * blockDim.x)
 
-// Initial key of suffix i: its first 29 bases, then min(29, n - i).  Bits past
-// the text are zero, so equal packed prefixes are ordered by length.
-__global__ void init_keys_kernel(const uint64_t *__restrict__ T, uint64_t n, uint64_t *keys, uint32_t *vals) {
-    GS_LOOP(i, n) {
-        const uint64_t w = text_window(T, i);
-        const uint64_t len = (n - i) < 29 ? (n - i) : 29;
-        keys[i] = (w & ~0x3Full) | len;
-        vals[i] = (uint32_t)i;
+constexpr uint64_t kFirstBases = 16;
+
+// The first sort's keys, from the last suffix to the first: 16 bases.
+__global__ void init_keys_kernel(const uint64_t *__restrict__ T, uint64_t n, uint32_t *keys, uint32_t *vals) {
+    GS_LOOP(t, n) {
+        const uint64_t i = n - 1 - t;
+        keys[t] = (uint32_t)(text_window(T, i) >> 32);
+        vals[t] = (uint32_t)i;
     }
 }
 
-// head value: j if position j starts a group of equal keys, else 0.
+// The order of the suffixes at i and j (different; both longer than depth and
+// equal so far) by up to `windows` further windows of 32 bases: -1 when S_j
+// sorts before S_i, 1 after, 0 when they stay equal.
+__device__ __forceinline__ int order_beyond(const uint64_t *__restrict__ T, uint64_t n, uint64_t i, uint64_t j,
+                                            uint64_t depth, uint32_t windows) {
+    const uint64_t shorter = n - (i > j ? i : j);  // bases of the shorter suffix
+    for (uint32_t w = 0; w < windows; w++) {
+        const uint64_t at = depth + 32ull * w;
+        const uint64_t a = text_window(T, i + at), b = text_window(T, j + at), x = a ^ b;
+        const uint64_t same = x ? (uint64_t)(__clzll((long long)x) >> 1) : 32u;
+        const uint64_t left = shorter - at;
+        if (same < left && same < 32) return b < a ? -1 : 1;
+        if (left <= 32) return j > i ? -1 : 1;  // the shorter one ends first
+    }
+    return 0;
+}
+
+// One sort's outcome: items 0 .. cnt - 1 (suffix vals[t], going to suffix-array
+// slot pos[t], or t itself when pos is null) ordered by key, equal keys (no
+// suffix of the two ended within `depth` bases) being groups that share their
+// first `depth` bases.  Writes every item to its slot: a group of one as it
+// is; one of up to kSmallGroup members in the order the text gives, member by
+// member the number of the others that sort before it (its compares read the
+// same few lines of text as theirs); a larger one in the order it has.
+// unresolved[t] marks the items of the list that are not settled, headb[slot]
+// the first of each group of them.
+// A block takes kRefineOut items with kSmallGroup more on each side, whose
+// heads it needs to find the groups; one ballot per warp gives a word of
+// heads.  A member's first window beyond depth is read once, into shared
+// memory, where the others find it; only members equal there are compared in
+// the text, over at most kRefineWindows windows per item in all.  Bound by
+// those random reads: 2.0 ms for 10^8 human-like bases, of whose suffixes the
+// first sort leaves about a third in groups, 20 ms for 6*10^8 (the text past
+// L2).  Sorting by 64-bit keys of 29 bases instead, eight passes of 24 bytes,
+// and prefix doubling for the rest took 15 ms in all at 10^8, this 9.
+constexpr int kRefineThreads = 512;
+constexpr int kSmallGroup = 32;
+constexpr int kRefineOut = kRefineThreads - 2 * kSmallGroup;
+constexpr uint32_t kRefineWindows = 64;
+
+template <typename K>
+__global__ void __launch_bounds__(kRefineThreads) refine_kernel(const K *__restrict__ keys,
+                                                                const uint32_t *__restrict__ vals, uint64_t cnt,
+                                                                const uint32_t *__restrict__ pos,
+                                                                const uint64_t *__restrict__ T, uint64_t n,
+                                                                uint64_t depth, uint32_t *sa, uint8_t *unresolved,
+                                                                uint8_t *headb) {
+    __shared__ uint32_t heads[kRefineThreads / 32];
+    __shared__ uint64_t next[kRefineThreads];
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint64_t tiles = (cnt + kRefineOut - 1) / kRefineOut;
+    for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t t = (int64_t)(tile * kRefineOut) + threadIdx.x - kSmallGroup;
+        const bool live = t >= 0 && t < (int64_t)cnt;
+        uint32_t i = 0;
+        bool head = t >= (int64_t)cnt;  // past the end: a boundary
+        if (live) {
+            i = vals[t];
+            head = t == 0 || keys[t] != keys[t - 1] || n - i <= depth || n - vals[t - 1] <= depth;
+        }
+        const unsigned word = __ballot_sync(0xFFFFFFFFu, head);
+        if (lane == 0) heads[warp] = word;
+        __syncthreads();
+        // the group's start (at or before t) and end (after t)
+        const uint32_t upto = word & (0xFFFFFFFFu >> (31u - lane));
+        const uint32_t above = lane < 31u ? word & (0xFFFFFFFFu << (lane + 1u)) : 0u;
+        const uint32_t before = warp > 0 ? heads[warp - 1] : 0u;
+        const uint32_t after = warp < kRefineThreads / 32 - 1 ? heads[warp + 1] : 0u;
+        uint32_t back = kSmallGroup, ahead = kSmallGroup + 1;  // members before t; distance to the end
+        if (upto)
+            back = lane - (31u - __clz(upto));
+        else if (before)
+            back = lane + 1u + __clz(before);
+        if (above)
+            ahead = (uint32_t)__ffs(above) - 1u - lane;
+        else if (after)
+            ahead = 31u - lane + (uint32_t)__ffs(after);
+        const uint32_t size = back + ahead;
+        // (of the items beside the block's own, those of a group that reaches
+        // into it: no head between them and it)
+        const bool left_of = warp == 0, right_of = warp == kRefineThreads / 32 - 1;
+        const bool reaches = left_of ? above == 0u : !right_of || upto == 0u;
+        if (live && reaches && size > 1u && size <= (uint32_t)kSmallGroup)
+            next[threadIdx.x] = text_window(T, (uint64_t)i + depth);
+        __syncthreads();
+        if (live && !left_of && !right_of) {
+            uint64_t at = t;  // the item's place in the list
+            bool more = false, first = false;
+            if (size > (uint32_t)kSmallGroup) {
+                more = true;
+                first = head;
+            } else if (size > 1u) {
+                const uint64_t a = t - back;
+                const uint32_t windows = kRefineWindows / size;
+                const uint64_t mine = next[threadIdx.x];
+                uint32_t less = 0, ties = 0, ties_before = 0;
+                for (uint32_t u = 0; u < size; u++) {
+                    if (u == back) continue;
+                    const uint64_t theirs = next[threadIdx.x - back + u];
+                    int c = theirs < mine ? -1 : 1;
+                    const uint32_t j = vals[a + u];
+                    const uint64_t x = mine ^ theirs;
+                    const uint64_t same = x ? (uint64_t)(__clzll((long long)x) >> 1) : 32u;
+                    const uint64_t left = n - (i > j ? i : j) - depth;  // bases of the shorter one there
+                    if (same >= left)
+                        c = j > i ? -1 : 1;  // it ends first
+                    else if (x == 0)
+                        c = left > 32 ? order_beyond(T, n, i, j, depth + 32, windows) : (j > i ? -1 : 1);
+                    less += c < 0 ? 1u : 0u;
+                    ties += c == 0 ? 1u : 0u;
+                    ties_before += (c == 0 && u < back) ? 1u : 0u;
+                }
+                at = a + less + ties_before;
+                more = ties != 0u;
+                first = ties_before == 0u;
+            }
+            const uint64_t slot = pos ? pos[at] : at;
+            sa[slot] = i;
+            unresolved[at] = more ? 1 : 0;
+            if (more) headb[slot] = first ? 1 : 0;
+        }
+        __syncthreads();
+    }
+}
+
+// 1 where the list's item t is the first of its group.
+__global__ void group_heads_kernel(const uint32_t *__restrict__ pos, uint64_t cnt, const uint8_t *__restrict__ headb,
+                                   uint32_t *g) {
+    GS_LOOP(t, cnt) g[t] = headb[pos[t]];
+}
+
+// A later sort's keys: the item's group number (from 1, in list order) above
+// its next `bases` bases from `depth` on.
+__global__ void group_keys_kernel(const uint64_t *__restrict__ T, const uint32_t *__restrict__ pos, uint64_t cnt,
+                                  const uint32_t *__restrict__ sa, const uint32_t *__restrict__ group,
+                                  uint64_t depth, uint32_t bases, uint64_t *keys, uint32_t *vals) {
+    GS_LOOP(t, cnt) {
+        const uint32_t i = sa[pos[t]];
+        keys[t] = ((uint64_t)(group[t] - 1u) << (2u * bases)) | (text_window(T, (uint64_t)i + depth) >> (64u - 2u * bases));
+        vals[t] = i;
+    }
+}
+
+// Prefix doubling starts from every suffix's rank: its slot, or for the
+// suffixes still in groups the slot of their group's head.
+__global__ void slot_ranks_kernel(const uint32_t *__restrict__ sa, uint64_t n, uint32_t *isa) {
+    GS_LOOP(j, n) isa[sa[j]] = (uint32_t)j;
+}
+
+__global__ void head_slots_kernel(const uint32_t *__restrict__ pos, uint64_t cnt, const uint8_t *__restrict__ headb,
+                                  uint32_t *hv) {
+    GS_LOOP(t, cnt) hv[t] = headb[pos[t]] ? pos[t] : 0u;
+}
+
+__global__ void group_ranks_kernel(const uint32_t *__restrict__ pos, uint64_t cnt, const uint32_t *__restrict__ sa,
+                                   const uint32_t *__restrict__ rank, uint32_t *isa) {
+    GS_LOOP(t, cnt) isa[sa[pos[t]]] = rank[t];
+}
+
+// head value: pos[t] if item t starts a group of equal keys, else 0.
 __global__ void head_values_kernel(const uint64_t *__restrict__ keys, uint64_t cnt,
                                    const uint32_t *__restrict__ pos, uint32_t *hv) {
-    GS_LOOP(t, cnt) {
-        const bool head = t == 0 || keys[t] != keys[t - 1];
-        hv[t] = head ? (pos ? pos[t] : (uint32_t)t) : 0u;
-    }
+    GS_LOOP(t, cnt) hv[t] = t == 0 || keys[t] != keys[t - 1] ? pos[t] : 0u;
 }
 
 // After the scan, rank[t] is the SA position of t's group head.  Writes the
 // ranks, the suffix-array entries, and flags members of groups of size > 1.
 __global__ void scatter_ranks_kernel(const uint64_t *__restrict__ keys, uint64_t cnt,
-                                     const uint32_t *__restrict__ pos,   // SA positions (null = identity)
+                                     const uint32_t *__restrict__ pos,   // SA positions
                                      const uint32_t *__restrict__ sorted_vals, const uint32_t *__restrict__ rank,
                                      uint32_t *isa, uint32_t *sa, uint8_t *unresolved) {
     GS_LOOP(t, cnt) {
         const uint32_t i = sorted_vals[t];
-        const uint32_t j = pos ? pos[t] : (uint32_t)t;
-        sa[j] = i;
+        sa[pos[t]] = i;
         isa[i] = rank[t];
         const bool head = t == 0 || keys[t] != keys[t - 1];
         const bool tail = t + 1 == cnt || keys[t + 1] != keys[t];
@@ -138,57 +306,110 @@ struct Pool {
         if (e_ != cudaSuccess) return status_from_cuda(e_); \
     } while (0)
 
+// Sorts by groups and next bases (step 3 above) are cheaper than prefix
+// doubling, whose ranks cost one random write per suffix, as long as they
+// handle few suffixes: at most half as many as the text has, in all, and at
+// most one round per 2^22 suffixes (a round's launches and its read of the
+// count take 0.1 ms, the ranks of 4*10^6 suffixes as long), 48 in the end.
+constexpr uint64_t kRoundSuffixes = 1ull << 22;
+constexpr uint64_t kMostRounds = 48;
+
 int build_suffix_array(sa_index *idx, cudaStream_t s, Arena *arenas, int n_arenas) {
     const uint64_t n = idx->n;
+    const uint64_t *T = idx->text;
     Pool pool{s, arenas, n_arenas};
     uint64_t *kA = pool.get<uint64_t>(n), *kB = pool.get<uint64_t>(n);
     uint32_t *vA = pool.get<uint32_t>(n), *vB = pool.get<uint32_t>(n);
-    uint32_t *isa = pool.get<uint32_t>(n), *sa32 = pool.get<uint32_t>(n);
-    uint32_t *hv = pool.get<uint32_t>(n), *rank = pool.get<uint32_t>(n);
+    // the 32-bit array is built in place, a 64-bit one widened from scratch
+    uint32_t *sa32 = idx->width == 4 ? reinterpret_cast<uint32_t *>(idx->sa) : pool.get<uint32_t>(n);
+    uint32_t *isa = pool.get<uint32_t>(n), *hv = pool.get<uint32_t>(n);
     uint32_t *posA = pool.get<uint32_t>(n), *posB = pool.get<uint32_t>(n);
-    uint8_t *flag = pool.get<uint8_t>(n);
+    uint8_t *flag = pool.get<uint8_t>(n), *headb = pool.get<uint8_t>(n);
     uint64_t *d_count = pool.get<uint64_t>(1);
     if (pool.err != cudaSuccess) return SA_ERR_NOMEM;
+    uint32_t *group = isa;  // group numbers, before the ranks are needed
 
     // Temporary storage sized for the largest call of each CUB routine.
-    size_t t_sort = 0, t_scan = 0, t_sel = 0, t_sel0 = 0;
+    size_t t_bytes = 0;
     thrust::counting_iterator<uint32_t> iota(0);
+    cub::DoubleBuffer<uint32_t> kb32(reinterpret_cast<uint32_t *>(kA), reinterpret_cast<uint32_t *>(kB));
     {
         cub::DoubleBuffer<uint64_t> kb(kA, kB);
         cub::DoubleBuffer<uint32_t> vb(vA, vB);
-        CK(cub::DeviceRadixSort::SortPairs(nullptr, t_sort, kb, vb, n, 0, 64, s));
-        CK(cub::DeviceScan::InclusiveScan(nullptr, t_scan, hv, rank, MaxOp(), n, s));
-        CK(cub::DeviceSelect::Flagged(nullptr, t_sel, posA, flag, posB, d_count, n, s));
-        CK(cub::DeviceSelect::Flagged(nullptr, t_sel0, iota, flag, posB, d_count, n, s));
+        size_t t[6] = {};
+        CK(cub::DeviceRadixSort::SortPairs(nullptr, t[0], kb, vb, n, 0, 64, s));
+        CK(cub::DeviceRadixSort::SortPairs(nullptr, t[1], kb32, vb, n, 0, 32, s));
+        CK(cub::DeviceScan::InclusiveScan(nullptr, t[2], hv, hv, MaxOp(), n, s));
+        CK(cub::DeviceScan::InclusiveSum(nullptr, t[3], group, group, n, s));
+        CK(cub::DeviceSelect::Flagged(nullptr, t[4], posA, flag, posB, d_count, n, s));
+        CK(cub::DeviceSelect::Flagged(nullptr, t[5], iota, flag, posB, d_count, n, s));
+        for (size_t x : t) t_bytes = x > t_bytes ? x : t_bytes;
     }
-    size_t t_bytes = t_sort > t_scan ? t_sort : t_scan;
-    if (t_sel > t_bytes) t_bytes = t_sel;
-    if (t_sel0 > t_bytes) t_bytes = t_sel0;
     void *temp = pool.get<uint8_t>(t_bytes);
     if (pool.err != cudaSuccess) return SA_ERR_NOMEM;
+    uint64_t cnt = 0;
+    auto read_count = [&]() -> cudaError_t {
+        const cudaError_t e = cudaMemcpyAsync(&cnt, d_count, sizeof cnt, cudaMemcpyDeviceToHost, s);
+        return e != cudaSuccess ? e : cudaStreamSynchronize(s);
+    };
+    const uint64_t most_tiles = (uint64_t)device_sm_count() * 16;
+    auto refine_grid = [&](uint64_t c) {
+        const uint64_t tiles = (c + kRefineOut - 1) / kRefineOut;
+        return (unsigned)(tiles < most_tiles ? tiles : most_tiles);
+    };
 
     const unsigned g = grid_for(n);
-    // Round 0: rank by the first 29 bases.
-    init_keys_kernel<<<g, kThreads, 0, s>>>(idx->text, n, kA, vA);
+    init_keys_kernel<<<g, kThreads, 0, s>>>(T, n, kb32.Current(), vA);
     CK(cudaGetLastError());
-    cub::DoubleBuffer<uint64_t> kb(kA, kB);
     cub::DoubleBuffer<uint32_t> vb(vA, vB);
-    CK(cub::DeviceRadixSort::SortPairs(temp, t_bytes, kb, vb, n, 0, 64, s));
-    head_values_kernel<<<g, kThreads, 0, s>>>(kb.Current(), n, nullptr, hv);
-    CK(cudaGetLastError());
-    CK(cub::DeviceScan::InclusiveScan(temp, t_bytes, hv, rank, MaxOp(), n, s));
-    scatter_ranks_kernel<<<g, kThreads, 0, s>>>(kb.Current(), n, nullptr, vb.Current(), rank, isa, sa32, flag);
+    CK(cub::DeviceRadixSort::SortPairs(temp, t_bytes, kb32, vb, n, 0, 32, s));
+    uint64_t depth = kFirstBases;
+    refine_kernel<uint32_t><<<refine_grid(n), kRefineThreads, 0, s>>>(kb32.Current(), vb.Current(), n, nullptr, T, n,
+                                                                      depth, sa32, flag, headb);
     CK(cudaGetLastError());
     // Unresolved SA positions, in increasing order.
     CK(cub::DeviceSelect::Flagged(temp, t_bytes, iota, flag, posA, d_count, n, s));
-    uint64_t cnt = 0;
-    CK(cudaMemcpyAsync(&cnt, d_count, sizeof cnt, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-
-    const int rank_bits = bit_length(n);
-    uint64_t h = 29;
+    CK(read_count());
     uint32_t *pos = posA, *pos_next = posB;
-    while (cnt > 0) {
+
+    const uint64_t rounds = n / kRoundSuffixes < kMostRounds ? n / kRoundSuffixes : kMostRounds;
+    uint64_t handled = 0;
+    for (uint64_t r = 0; r < rounds && cnt > 0 && (handled += cnt) <= n / 2; r++) {
+        const unsigned gc = grid_for(cnt);
+        // every group has two members or more
+        const int group_bits = bit_length(cnt / 2) > 0 ? bit_length(cnt / 2) : 1;
+        const uint32_t bases = (uint32_t)(64 - group_bits) / 2;
+        group_heads_kernel<<<gc, kThreads, 0, s>>>(pos, cnt, headb, group);
+        CK(cudaGetLastError());
+        CK(cub::DeviceScan::InclusiveSum(temp, t_bytes, group, group, cnt, s));
+        group_keys_kernel<<<gc, kThreads, 0, s>>>(T, pos, cnt, sa32, group, depth, bases, kA, vA);
+        CK(cudaGetLastError());
+        cub::DoubleBuffer<uint64_t> rk(kA, kB);
+        cub::DoubleBuffer<uint32_t> rv(vA, vB);
+        CK(cub::DeviceRadixSort::SortPairs(temp, t_bytes, rk, rv, cnt, 0, group_bits + 2 * (int)bases, s));
+        depth += bases;
+        refine_kernel<uint64_t><<<refine_grid(cnt), kRefineThreads, 0, s>>>(rk.Current(), rv.Current(), cnt, pos, T, n,
+                                                                            depth, sa32, flag, headb);
+        CK(cudaGetLastError());
+        CK(cub::DeviceSelect::Flagged(temp, t_bytes, pos, flag, pos_next, d_count, cnt, s));
+        CK(read_count());
+        uint32_t *tmp = pos;
+        pos = pos_next;
+        pos_next = tmp;
+    }
+
+    if (cnt > 0) {
+        slot_ranks_kernel<<<g, kThreads, 0, s>>>(sa32, n, isa);
+        CK(cudaGetLastError());
+        const unsigned gc = grid_for(cnt);
+        head_slots_kernel<<<gc, kThreads, 0, s>>>(pos, cnt, headb, hv);
+        CK(cudaGetLastError());
+        CK(cub::DeviceScan::InclusiveScan(temp, t_bytes, hv, hv, MaxOp(), cnt, s));
+        group_ranks_kernel<<<gc, kThreads, 0, s>>>(pos, cnt, sa32, hv, isa);
+        CK(cudaGetLastError());
+    }
+    const int rank_bits = bit_length(n);
+    for (uint64_t h = depth; cnt > 0; h *= 2) {
         const unsigned gc = grid_for(cnt);
         pair_keys_kernel<<<gc, kThreads, 0, s>>>(pos, cnt, sa32, isa, n, h, kA, vA);
         CK(cudaGetLastError());
@@ -197,20 +418,16 @@ int build_suffix_array(sa_index *idx, cudaStream_t s, Arena *arenas, int n_arena
         CK(cub::DeviceRadixSort::SortPairs(temp, t_bytes, rk, rv, cnt, 0, 32 + rank_bits, s));
         head_values_kernel<<<gc, kThreads, 0, s>>>(rk.Current(), cnt, pos, hv);
         CK(cudaGetLastError());
-        CK(cub::DeviceScan::InclusiveScan(temp, t_bytes, hv, rank, MaxOp(), cnt, s));
-        scatter_ranks_kernel<<<gc, kThreads, 0, s>>>(rk.Current(), cnt, pos, rv.Current(), rank, isa, sa32, flag);
+        CK(cub::DeviceScan::InclusiveScan(temp, t_bytes, hv, hv, MaxOp(), cnt, s));
+        scatter_ranks_kernel<<<gc, kThreads, 0, s>>>(rk.Current(), cnt, pos, rv.Current(), hv, isa, sa32, flag);
         CK(cudaGetLastError());
         CK(cub::DeviceSelect::Flagged(temp, t_bytes, pos, flag, pos_next, d_count, cnt, s));
-        CK(cudaMemcpyAsync(&cnt, d_count, sizeof cnt, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
+        CK(read_count());
         uint32_t *tmp = pos;
         pos = pos_next;
         pos_next = tmp;
-        h *= 2;
     }
-    if (idx->width == 4) {
-        CK(cudaMemcpyAsync(idx->sa, sa32, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-    } else {
+    if (idx->width == 8) {
         widen_kernel<<<g, kThreads, 0, s>>>(sa32, n, reinterpret_cast<uint64_t *>(idx->sa));
         CK(cudaGetLastError());
     }
