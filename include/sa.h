@@ -231,8 +231,14 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
  *             since each result is stored as one 32-byte sector).
  *  stream     CUDA stream or NULL.
  *
- * The work runs as three kernels on the stream: the batch's bases are packed
- * 2 bits each beside a per-base validity mask; a one-thread-per-query pass
+ * A small batch (up to 2^19 queries and 2^26 bases; less where brackets are
+ * wide or an index has no k-mer table) runs as one kernel that packs each
+ * query itself, brackets it by the k-mer table and finishes wide brackets
+ * with whole warps; it takes no scratch.  The tuning knobs and search orders
+ * of sa_search_params, when set, select the path below.
+ *
+ * A larger one runs as three kernels on the stream: the batch's bases are packed
+ * 2 bits each beside a validity bitmap; a one-thread-per-query pass
  * brackets each query of m >= k bases by the k-mer table and probes it up to
  * sa_search_params.front_probes times, and answers a shorter query from the
  * table's counts; a persistent kernel finishes the queries that remain (and

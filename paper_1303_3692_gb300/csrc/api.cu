@@ -235,16 +235,47 @@ uint32_t fill_ref_table(const sa_index *const *refs, uint32_t n_refs, uint32_t w
     return off;
 }
 
+// Launches a call's search kernels between the caller's two events, if given.
+template <typename Launch>
+int search_timed(const sa_search_params *params, cudaStream_t s, Launch launch) {
+    cudaEvent_t ev0 = params ? reinterpret_cast<cudaEvent_t>(params->search_events[0]) : nullptr;
+    cudaEvent_t ev1 = params ? reinterpret_cast<cudaEvent_t>(params->search_events[1]) : nullptr;
+    cudaError_t err = ev0 ? cudaEventRecord(ev0, s) : cudaSuccess;
+    if (err == cudaSuccess) err = launch();
+    if (err == cudaSuccess && ev1) err = cudaEventRecord(ev1, s);
+    return status_from_cuda(err);
+}
+
+// Whether a batch is searched by one kernel from its ASCII bases (small.cu):
+// the cost of the other path's launches and passes, about 50 us, against that
+// kernel's slower rate per query and base.  Measured on the GB300, one kernel
+// against the other path, us a call: 5*10^5 queries of 100 bases at 100 Mbp 99
+// against 126, of 20-300 bases (84 M) 224 against 197, 65,536 of 1024 bases
+// (67 M) 233 against 309, 131,072 of them 379 against 343.  With more suffixes
+// than k-mers more brackets are wide and finished by whole warps: at 3.1 Gbp
+// 262,144 queries of 32 bases 101 against 109, of 150 bases (39 M) 162 against
+// 155.  Without a k-mer table every query is: 32,768 queries 64-87 against
+// 80-97, 65,536 99-150 against 81-110.
+constexpr uint64_t kSmallQueries = 1ull << 19;
+constexpr uint64_t kSmallQueriesNoTable = 1ull << 15;
+constexpr uint64_t kSmallBases = 1ull << 26;
+bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uint64_t total) {
+    for (uint32_t r = 0; r < n_refs; r++)
+        if (!refs[r]->krt && n_q > kSmallQueriesNoTable) return false;
+    return n_q <= kSmallQueries && total <= (default_front_probes(refs, n_refs) == 1 ? kSmallBases / 2 : kSmallBases);
+}
+
 // The search of a batch whose inputs are in device memory: ascii holds the
 // batch's bases from offset `first` on (query q is ascii[q_off[q] - first ..
 // q_off[q + 1] - first)), q_off and q_ref are device arrays and out device
 // results.  Scratch comes from sc, on stream s.  *flags_out receives the
 // call's device flags ([0] a byte that is not a base, [1] a wait that ran
-// out, [3] a bad reference id).
+// out, [3] a bad reference id), or null when !need_flags and the search keeps
+// none.
 int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, const char *ascii,
                   const uint64_t *q_off, const uint32_t *q_ref, uint64_t n_q, uint64_t first, uint64_t total,
                   sa_result *out, cudaStream_t s, const sa_search_params *params, bool plain, uint32_t trunc_cap,
-                  Scratch &sc, int **flags_out, uint64_t *tile_kept = nullptr) {
+                  Scratch &sc, int **flags_out, bool need_flags, uint64_t *tile_kept = nullptr) {
     const uint32_t order = params ? params->flags & (SA_PARAM_KMER_ORDER | SA_PARAM_INPUT_ORDER) : 0u;
     if (order == (SA_PARAM_KMER_ORDER | SA_PARAM_INPUT_ORDER)) return SA_ERR_ARG;
     const uint32_t threads = params && params->threads_per_block ? params->threads_per_block : 1024;
@@ -256,6 +287,34 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     const bool revcomp = params && (params->flags & SA_PARAM_REVERSE_COMPLEMENT);
     if (strand_bits && (revcomp || !q_ref)) return SA_ERR_ARG;
     cudaError_t err = cudaSuccess;
+    const bool knobs = params && (params->threads_per_block || params->blocks_per_sm || params->key_depth ||
+                                  params->chunk || params->front_probes || (params->flags & SA_PARAM_EXPIRE_WAITS));
+    if (!plain && !knobs && order == 0 && small_batch(refs, n_refs, n_q, total)) {
+        int *flags = need_flags ? sc.get<int>(4) : nullptr;
+        if (sc.failed) return SA_ERR_NOMEM;
+        if (flags && (err = cudaMemsetAsync(flags, 0, 4 * sizeof(int), s)) != cudaSuccess) return status_from_cuda(err);
+        *flags_out = flags;
+        SearchLaunch L;
+        memset(&L, 0, sizeof L);
+        fill_ref_table(refs, n_refs, 0, &L.refs);
+        L.n_refs = n_refs;
+        L.width = width;
+        L.ascii = ascii;
+        L.q_off = q_off;
+        L.first = first;
+        L.total = total;
+        L.q_ref = q_ref;
+        L.n_q = n_q;
+        L.out = out;
+        L.pack_err = flags;
+        L.bad_ref = flags ? flags + 3 : nullptr;
+        L.revcomp = revcomp;
+        L.strand_bits = strand_bits;
+        L.trunc_cap = trunc_cap;
+        L.tile_kept = tile_kept;
+        L.tile_sum_by_warp = true;
+        return search_timed(params, s, [&] { return launch_search_small(L, s); });
+    }
     const uint64_t nwords = (total + 31) / 32;
     const uint64_t tq_words = nwords + SA_TQ_PAD_WORDS;
     // list and worklist records hold a query's first base in 48 bits (a batch
@@ -332,19 +391,12 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.batch_dirty = flags + 5;
 
     if ((err = launch_pack_batch(L, tq, tvb, tv, s)) != cudaSuccess) return status_from_cuda(err);
-    cudaEvent_t ev0 = params ? reinterpret_cast<cudaEvent_t>(params->search_events[0]) : nullptr;
-    cudaEvent_t ev1 = params ? reinterpret_cast<cudaEvent_t>(params->search_events[1]) : nullptr;
-    if (ev0 && (err = cudaEventRecord(ev0, s)) != cudaSuccess) return status_from_cuda(err);
-    if (plain) {
-        err = launch_search_plain(L, s);
-    } else {
-        if (kmer_order) err = launch_bucketed_worklist(L, wrec_in, s);
-        if (err == cudaSuccess) err = launch_front(L, s);
-        if (err == cudaSuccess) err = launch_search(L, s);
-    }
-    if (err != cudaSuccess) return status_from_cuda(err);
-    if (ev1 && (err = cudaEventRecord(ev1, s)) != cudaSuccess) return status_from_cuda(err);
-    return SA_OK;
+    return search_timed(params, s, [&] {
+        if (plain) return launch_search_plain(L, s);
+        cudaError_t e = kmer_order ? launch_bucketed_worklist(L, wrec_in, s) : cudaSuccess;
+        if (e == cudaSuccess) e = launch_front(L, s);
+        return e == cudaSuccess ? launch_search(L, s) : e;
+    });
 }
 
 // The call's status from its device flags read back to the host.
@@ -373,8 +425,14 @@ int search_impl(const sa_index *const *refs, uint32_t n_refs, const char *q_base
         last = params->q_first + params->q_total;
     } else if (off_dev) {
         uint64_t fl[2];
-        cudaError_t e = cudaMemcpyAsync(&fl[0], q_offsets, 8, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&fl[1], q_offsets + n_q, 8, cudaMemcpyDeviceToHost, s);
+        // both in one copy of two rows n_q offsets apart, where the pitch allows it
+        cudaError_t e = cudaSuccess;
+        if (n_q * 8 <= 0x7FFFFFFFull) {
+            e = cudaMemcpy2DAsync(fl, 8, q_offsets, n_q * 8, 8, 2, cudaMemcpyDeviceToHost, s);
+        } else {
+            e = cudaMemcpyAsync(&fl[0], q_offsets, 8, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&fl[1], q_offsets + n_q, 8, cudaMemcpyDeviceToHost, s);
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return status_from_cuda(e);
         first = fl[0];
@@ -411,7 +469,7 @@ int search_impl(const sa_index *const *refs, uint32_t n_refs, const char *q_base
     if (err != cudaSuccess) return status_from_cuda(err);
     int *flags = nullptr;
     st = search_device(refs, n_refs, width, bases_d, off_d, ref_d, n_q, first, total, out_d, s, params, plain,
-                       trunc_cap, sc, &flags, tile_kept);
+                       trunc_cap, sc, &flags, dstatus || !out_dev, tile_kept);
     if (st) return st;
     if (dstatus && (err = launch_search_status(flags, dstatus, s)) != cudaSuccess) return status_from_cuda(err);
     if (!out_dev) {
@@ -902,7 +960,7 @@ int search_pipelined(const sa_index *const *refs, uint32_t n_refs, uint32_t widt
             Scratch csc{t};
             int *flags = nullptr;
             st = search_device(refs, n_refs, width, slot_bases[i], slot_off[i], ref_c, nq, ba, nb, out_d + a, t, &cp,
-                               false, locate ? cap : ~0u, csc, &flags);
+                               false, locate ? cap : ~0u, csc, &flags, true);
             if (st) break;
             if ((err = launch_fold_status(flags, stat_d, t)) != cudaSuccess) break;
             if (locate) {

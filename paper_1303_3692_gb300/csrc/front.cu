@@ -22,71 +22,13 @@
 // appended to a worklist -- a 64-byte record holding a bracket of both
 // bounds, its length, index, reference, first base in the packed batch and
 // first 160 bases -- which the persistent kernel of search.cu then finishes.
-#include "sa_internal.cuh"
+#include "first_pass.cuh"
 
 namespace sa {
 
 namespace {
 
 constexpr int kFrontThreads = 256;
-
-struct FrontDesc {
-    const uint64_t *text;
-    const uint4 *rec;
-    const uint4 *krt;
-    uint64_t tail;  // the text's last 32 bases (all, when it has fewer), the last in the low bits
-    uint32_t n;
-    uint32_t kmer_k;
-};
-
-// How many suffixes shorter than k equal the string q (qlen bases, as a
-// number) followed by some A's.
-__device__ __forceinline__ uint32_t short_suffixes(uint64_t tail, uint32_t n, uint32_t k, uint64_t q, uint32_t qlen) {
-    uint32_t c = 0;
-    for (uint32_t len = qlen; len < k && len <= n; len++)
-        c += (tail & ((1ull << (2u * len)) - 1ull)) == (q << (2u * (len - qlen))) ? 1u : 0u;
-    return c;
-}
-
-// The interval of a query of 1 <= m < k bases (p as a number), from the counts
-// of two k-mer entries: kmer[x] is the number of suffixes that sort before the
-// k-base string x.  P's first suffix comes before P A..A only as P, P A, P AA,
-// ... at the text's end, so lo = kmer[P A..A] less those of them that are
-// suffixes.  P's successor p + 1 is Q followed by A's, Q ending in the base
-// that was raised; of the suffixes before (p + 1) A..A only Q, Q A, ... do not
-// start with P or sort before it.  Two reads of random entries per query; the
-// descent of a key table and the binary search below it took about 2 log2 of
-// the count more (2*10^6 queries of 8-31 bases at 100 Mbp: 594 -> 375 us a
-// call).
-__device__ __forceinline__ void brief_interval(const FrontDesc &d, uint64_t p, uint32_t m, uint32_t *lo, uint32_t *hi) {
-    const uint32_t k = d.kmer_k, up = 2u * (k - m);
-    const uint64_t next = p + 1;
-    const bool last = next == 1ull << (2u * m);  // P is T..T: no successor, every suffix from lo on
-    const uint32_t klo = __ldg(reinterpret_cast<const uint32_t *>(d.krt + 4 * (p << up)));
-    const uint32_t khi = last ? d.n : __ldg(reinterpret_cast<const uint32_t *>(d.krt + 4 * (next << up)));
-    const uint32_t raised = ((uint32_t)__ffsll((long long)next) - 1u) >> 1;  // trailing A's of p + 1
-    *lo = klo - short_suffixes(d.tail, d.n, k, p, m);
-    *hi = last ? d.n : khi - short_suffixes(d.tail, d.n, k, next >> (2u * raised), m - raised);
-}
-
-// P (bases 0-127 in w, the rest from qw; length m >= 1) against the pivot of
-// a k-mer entry: its first 192 bases in e (clamp of them exist), then the
-// text from position pos + 192 when all 192 tie.
-template <bool kStrands>
-__device__ __forceinline__ int cmp_entry(const uint64_t w[4], uint32_t m, const uint64_t e[6], uint32_t pos,
-                                         uint32_t clamp, uint32_t n, const uint64_t *__restrict__ T,
-                                         const QueryWindows<kStrands> &qw, uint32_t *lcp) {
-#pragma unroll
-    for (int j = 0; j < 6; j++) {
-        const uint32_t off = 32u * j;
-        const uint32_t qlen = min(32u, m - off);
-        const uint32_t tlen = clamp > off ? min(32u, clamp - off) : 0u;
-        const uint64_t q = j < 4 ? w[j] : qw(off);
-        const int c = cmp_window(q, e[j], qlen, tlen, off, m, lcp);
-        if (c != 2) return c;
-    }
-    return cmp_suffix_qw(T, n, pos, qw, m, 192u, lcp);
-}
 
 // The list slot of the j-th record of the k-mer-ordered list: region by
 // region (in the largest bucket b whose regions before it hold at most j
@@ -118,9 +60,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
     __shared__ uint32_t s_lprefix[kNumBuckets + 2];        // the list's numbering (list input)
     __shared__ uint32_t s_lstart[kNumBuckets + 1];
     for (unsigned r = threadIdx.x; r < a.n_refs; r += blockDim.x) {
-        const RefDesc &d = a.refs.r[r];
-        const uint64_t tail = d.n >= 32 ? text_window(d.text, d.n - 32) : ldg_u64(d.text) >> (64u - 2u * (uint32_t)d.n);
-        sdesc[r] = FrontDesc{d.text, d.rec, d.krt, tail, (uint32_t)d.n, d.kmer_k};
+        sdesc[r] = front_desc(a.refs.r[r]);
     }
     if (kFromList) {
         for (unsigned i = threadIdx.x; i < kNumBuckets + 2; i += blockDim.x) s_lprefix[i] = a.bplan[kPlanPrefix + i];

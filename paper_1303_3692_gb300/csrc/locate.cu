@@ -24,6 +24,10 @@ namespace {
 constexpr int kTileThreads = 512;
 constexpr int kItems = 8;
 constexpr uint64_t kTile = (uint64_t)kTileThreads * kItems;
+// Up to this many tiles (2^21 queries) each tile of the gather adds up the
+// sums of those before it itself, one thread per tile, and the scan's launch
+// is saved; beyond, a scan puts them in place first.
+constexpr uint64_t kDirectTiles = kTileThreads;
 
 __device__ __forceinline__ uint64_t kept(const sa_result &r, uint32_t cap) {
     if (r.count == ~0ull) return 0;  // invalid query (reported as all-ones)
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(1024) scan_partials_kernel(uint64_t *partials,
 template <typename IdxT>
 __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __grid_constant__ LocateLaunch a) {
     constexpr int kWarps = kTileThreads / 32;
-    __shared__ uint64_t s_warp[kWarps];
+    __shared__ uint64_t s_warp[kWarps], s_before[kWarps];
     // each item's kept count and lower bound from the first pass (32 KB), so
     // the second pass does not read the results again: at 3.1 Gbp the L2 no
     // longer holds them by then
@@ -113,7 +117,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __gr
     __shared__ uint32_t s_lo[kItems][kTileThreads];
     const uint64_t tile_base = (uint64_t)blockIdx.x * kTile;
     const uint64_t ntiles = gridDim.x;
-    if (blockIdx.x == ntiles - 1 && threadIdx.x == 0) a.out_offsets[a.n_q] = a.partials[ntiles];
+    const bool direct = ntiles <= kDirectTiles;  // the partials are the tile sums themselves
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint64_t warp_base = tile_base + (uint64_t)warp * (32 * kItems);
     IdxT *pos = reinterpret_cast<IdxT *>(a.out_pos);
@@ -136,9 +140,19 @@ __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __gr
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xFFFFFFFFu, tot, o);
     if (lane == 0) s_warp[warp] = tot;
+    if (direct) {  // the tiles before this one, a thread each
+        uint64_t before = threadIdx.x < blockIdx.x ? a.partials[threadIdx.x] : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+        if (lane == 0) s_before[warp] = before;
+    }
     __syncthreads();
-    uint64_t run = a.partials[blockIdx.x];
+    uint64_t run = direct ? (a.base_in ? *a.base_in : 0) : a.partials[blockIdx.x];
+    if (direct)
+        for (int w = 0; w < kWarps; w++) run += s_before[w];
     for (unsigned w = 0; w < warp; w++) run += s_warp[w];
+    // the last warp of the last tile ends at the total
+    if (blockIdx.x == ntiles - 1 && threadIdx.x == kTileThreads - 1) a.out_offsets[a.n_q] = run + tot;
 
     // Second pass over the items, from shared memory.
 #pragma unroll
@@ -212,7 +226,7 @@ cudaError_t launch_locate(const LocateLaunch &L, cudaStream_t s) {
         return cudaMemsetAsync(L.out_offsets, 0, sizeof(uint64_t), s);
     }
     if (!L.presummed) tile_sums_kernel<<<(unsigned)tiles, kTileThreads, 0, s>>>(L.res, L.n_q, L.cap, L.partials);
-    scan_partials_kernel<<<1, 1024, 0, s>>>(L.partials, tiles, L.base_in);
+    if (tiles > kDirectTiles) scan_partials_kernel<<<1, 1024, 0, s>>>(L.partials, tiles, L.base_in);
     if (L.width == 4)
         tile_gather_kernel<uint32_t><<<(unsigned)tiles, kTileThreads, 0, s>>>(L);
     else

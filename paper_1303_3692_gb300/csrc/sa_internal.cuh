@@ -541,9 +541,9 @@ struct QueryWindows {
 };
 
 // cmp_suffix_tq with the query's windows from qw (start >= 96).
-template <bool kStrands>
+template <typename Windows>
 __device__ __forceinline__ int cmp_suffix_qw(const uint64_t *__restrict__ T, uint32_t n, uint32_t p,
-                                             const QueryWindows<kStrands> &qw, uint32_t m, uint32_t start, uint32_t *lcp) {
+                                             const Windows &qw, uint32_t m, uint32_t start, uint32_t *lcp) {
     uint32_t off = start & ~31u;
     const uint32_t rem = n - p;
     for (;;) {
@@ -701,6 +701,9 @@ cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s);
 // input in that order.
 cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, cudaStream_t s);
 cudaError_t launch_search(const SearchLaunch &L, cudaStream_t s);
+// A small batch in one kernel, straight from its ASCII bases (L.tq, L.tv,
+// L.wrec and the like are not used; L.pack_err and L.bad_ref may be null).
+cudaError_t launch_search_small(const SearchLaunch &L, cudaStream_t s);
 cudaError_t launch_search_plain(const SearchLaunch &L, cudaStream_t s);
 // One thread: *dst = the call's status from its device flags (flags[1] a
 // wait that ran out, flags[0] a query that is not bases, flags[3] a bad

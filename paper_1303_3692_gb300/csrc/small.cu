@@ -1,0 +1,264 @@
+// small.cu -- the search of a small batch (Section IV) in one kernel.
+//
+// A batch of some thousand queries does not fill the GPU, so what it costs is
+// latency: the launches, the packing, the first and the persistent pass one
+// after the other, and in those the dependent reads of the query with the
+// longest binary search.  Here one kernel does it all:
+//   * a thread packs its query from the ASCII bases itself and checks them;
+//   * the k-mer entry of its first k bases and up to kLaneProbes probes settle
+//     most queries, as in the first pass (front.cu);
+//   * a query that remains -- a wide bracket, an index without a k-mer table --
+//     is finished by its whole warp: the 32 lanes probe 32 ranks spread over
+//     the bracket at once, so a bracket of 1000 suffixes takes two rounds
+//     of reads instead of ten, and one of 10^8 six instead of 27;
+//   * a warp takes few queries when the batch is small (as many as give every
+//     resident warp some), so that those rounds follow one another seldom.
+// A round reads 32 records where a step of the binary search reads one: right
+// while the GPU has nothing else to do, wrong for a large batch (api.cu:
+// small_batch has the line between the two and both sides' times).
+//
+// Bound by the latency of a handful of dependent reads: 20 queries against 5
+// Mbp 51 -> 24 us a call (of which a call that reads nothing takes about 20),
+// 10^5 queries of 32 bases at 1 Mbp 57 -> 26 us, 20,011 of 20-300 bases of
+// both strands over four genomes, with locate, 83 -> 47 us.
+#include "first_pass.cuh"
+
+namespace sa {
+
+namespace {
+
+constexpr int kSmallThreads = 128;
+constexpr int kSmallPerSm = 8;  // CTAs
+constexpr uint32_t kLaneProbes = 2;
+
+// A query's windows packed from its ASCII bases: bytes [qa, qa + m) of the
+// batch, or their reverse complement.
+struct AsciiWindows {
+    const uint8_t *ascii;
+    uint64_t total;
+    uint64_t qa;
+    uint32_t m;
+    bool rc;
+    __device__ __forceinline__ uint64_t packed(uint32_t off, uint32_t *bad) const {  // off < m
+        const uint32_t nb = m - off < 32u ? m - off : 32u;
+        if (!rc) return pack_word(ascii, total, qa + off, nb, bad);
+        // the nb bytes that end off bases before the query's end
+        return rc_window(pack_word(ascii, total, qa + (m - off - nb), nb, bad)) << (64u - 2u * nb);
+    }
+    __device__ __forceinline__ uint64_t operator()(uint32_t off) const {
+        uint32_t bad = 0;
+        return packed(off, &bad);
+    }
+};
+
+__device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
+    return __shfl_sync(0xFFFFFFFFu, (unsigned long long)v, src);
+}
+
+// Query q (m bases, its first 128 in w, all in qw) against ranks (L, R) by the
+// whole warp; every argument is the same in all lanes.  Each round's lanes
+// probe ranks spread over what is open: while no rank with the query as prefix
+// is known, all over (L, R); then the lower 16 over (loL, loR) and the upper
+// 16 over (hiL, hiR), which hold the two ends of the interval.
+__device__ __forceinline__ void finish_by_warp(const FrontDesc &d, const AsciiWindows &qw, const uint64_t w[4],
+                                               uint32_t m, uint32_t L, uint32_t R, uint64_t *lo, uint64_t *hi) {
+    const unsigned lane = threadIdx.x & 31u;
+    bool split = false;  // a match is known: (L, R) is (loL, loR), and (hL, hR) the upper end's
+    uint32_t hL = 0, hR = 0;
+    for (;;) {
+        const bool open_lo = R - L > 1u, open_hi = split && hR - hL > 1u;
+        if (!open_lo && !open_hi) break;
+        // this lane's interval and its place among the lanes that share it
+        const bool both = open_lo && open_hi;
+        const bool upper = both ? lane >= 16u : !open_lo;
+        const uint32_t lanes = both ? 16u : 32u, at = both ? (lane & 15u) : lane;
+        const uint32_t a = upper ? hL : L, b = upper ? hR : R;
+        const uint32_t inside = b - a - 1u;  // ranks strictly between
+        const bool live = at < inside;
+        const uint32_t M = inside <= lanes ? a + 1u + at : a + (uint32_t)(((uint64_t)(b - a) * (at + 1u)) / (lanes + 1u));
+        uint4 r0, r1;
+        ldg32_if(live, d.rec + 2 * (size_t)M, &r0, &r1);
+        int c = 2;
+        if (live) {
+            uint32_t l;
+            bool und = false;
+            c = cmp_record(w[0], w[1], w[2], w[3], m, r0, r1, d.n, &l, &und);
+            if (und) c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, kRecBases, &l);
+        }
+        const uint32_t cut = min(m, kLcpCap);
+        const unsigned match = __ballot_sync(0xFFFFFFFFu, c == CMP_PREFIX);
+        const unsigned less = __ballot_sync(0xFFFFFFFFu, c == CMP_LESS);
+        const unsigned greater = __ballot_sync(0xFFFFFFFFu, c == CMP_GREATER);
+        // matches whose neighbour is known not to match settle an end
+        const unsigned low_end = __ballot_sync(0xFFFFFFFFu, c == CMP_PREFIX && ((r1.z >> 8) & 0xFFu) < cut);
+        const unsigned high_end = __ballot_sync(0xFFFFFFFFu, c == CMP_PREFIX && (r1.z & 0xFFu) < cut);
+        auto rank_of = [&](int src) { return __shfl_sync(0xFFFFFFFFu, M, src); };
+        const unsigned lo_lanes = both ? 0x0000FFFFu : (split && !open_lo ? 0u : 0xFFFFFFFFu);
+        const unsigned hi_lanes = both ? 0xFFFF0000u : (split && open_lo ? 0u : (split ? 0xFFFFFFFFu : 0u));
+        // the lower end's lanes (before the split: all lanes serve both ends)
+        const unsigned g = greater & lo_lanes, p = match & lo_lanes, s = less & lo_lanes;
+        const uint32_t last_g = rank_of(g ? 31 - __clz(g) : 0), first_p = rank_of(p ? __ffs(p) - 1 : 0);
+        const uint32_t last_p = rank_of(p ? 31 - __clz(p) : 0), first_s = rank_of(s ? __ffs(s) - 1 : 0);
+        const bool low_known = p && ((low_end >> (__ffs(p) - 1)) & 1u);
+        const bool high_known = p && ((high_end >> (31 - __clz(p))) & 1u);
+        // the upper end's lanes after the split
+        const unsigned hp = match & hi_lanes, hs = less & hi_lanes;
+        const uint32_t h_last_p = rank_of(hp ? 31 - __clz(hp) : 0), h_first_s = rank_of(hs ? __ffs(hs) - 1 : 0);
+        const bool h_known = hp && ((high_end >> (31 - __clz(hp))) & 1u);
+        if (g) L = last_g;
+        if (!split) {
+            if (p) {
+                split = true;
+                hL = last_p;
+                hR = high_known ? last_p + 1u : (s ? first_s : R);
+                R = first_p;
+                if (low_known) L = first_p - 1u;
+            } else if (s) {
+                R = first_s;
+            }
+        } else {
+            if (p) {
+                R = first_p;
+                if (low_known) L = first_p - 1u;
+            }
+            if (hs) hR = h_first_s;
+            if (hp) {
+                hL = h_last_p;
+                if (h_known) hR = h_last_p + 1u;
+            }
+        }
+    }
+    *lo = R;
+    *hi = split ? hR : R;
+}
+
+template <bool kSingle>
+__global__ void __launch_bounds__(kSmallThreads, kSmallPerSm) small_kernel(const __grid_constant__ SearchLaunch a,
+                                                                          uint32_t per_warp) {
+    __shared__ FrontDesc sdesc[SA_MAX_REFS];
+    const unsigned lane = threadIdx.x & 31u;
+    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t q = warp * per_warp + lane;
+    const bool live = lane < per_warp && q < a.n_q;
+    uint64_t qa = 0, qe = 0;
+    uint32_t r = 0;
+    if (live) {
+        qa = __ldg(a.q_off + q) - a.first;
+        qe = __ldg(a.q_off + q + 1) - a.first;
+        if (!kSingle) r = __ldg(a.q_ref + q);
+    }
+    for (unsigned i = threadIdx.x; i < a.n_refs; i += blockDim.x) sdesc[i] = front_desc(a.refs.r[i]);
+    __syncthreads();
+    if (warp * per_warp >= a.n_q) return;  // (whole warps)
+
+    const bool rc = a.revcomp || (a.strand_bits && (r & kStrandBit));
+    if (a.strand_bits) r &= ~kStrandBit;
+    const bool range_ok = live && qa <= qe && qe <= a.total && qe - qa < (1ull << 31);
+    bool ok = range_ok && r < a.n_refs;
+    const bool bad_ref = range_ok && !ok;
+    const uint32_t m = ok ? (uint32_t)(qe - qa) : 0u;
+    const AsciiWindows qw{reinterpret_cast<const uint8_t *>(a.ascii), a.total, qa, m, rc};
+    uint64_t w[4] = {0, 0, 0, 0};
+    uint32_t bad = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+        if (m > 32u * j) w[j] = qw.packed(32u * j, &bad);
+    for (uint32_t off = 128u; off < m; off += 32u) (void)qw.packed(off, &bad);
+    ok = ok && bad == 0u;
+
+    FrontDesc d = sdesc[0];
+    if (!kSingle && ok) d = sdesc[r];
+    const uint32_t kk = d.kmer_k;
+    const bool look = ok && m > 0 && d.krt != nullptr && m >= kk;
+    uint4 h, e01, e23, e45;
+    ldg64_pairs_if(look, d.krt + 4 * (look ? (w[0] >> (64u - 2u * kk)) : 0ull), &h, &e01, &e23, &e45);
+    Bounds bd;
+    bd.start(look ? h.x - 1u : 0xFFFFFFFFu, look ? h.y : d.n);
+    bool done = !live || !ok || m == 0 || (look && bd.R - bd.L <= 1u);
+    uint64_t lo = bd.R, hi = bd.R;  // a bracket without suffixes
+    if (live && !ok) lo = hi = ~0ull;
+    if (live && ok && m == 0) {
+        lo = 0;
+        hi = d.n;
+    }
+    if (live && ok && m > 0 && d.krt != nullptr && m < kk) {
+        uint32_t l, u;
+        brief_interval(d, w[0] >> (64u - 2u * m), m, &l, &u);
+        lo = l;
+        hi = u;
+        done = true;
+    }
+    bool go = !done && look;
+    auto step = [&](int c, uint32_t M, uint32_t l, uint32_t lp, uint32_t ln) {
+        if (bd.step(c, M, l, m, lp, ln)) {
+            lo = bd.first();
+            hi = bd.R;
+            done = true;
+            go = false;
+        }
+    };
+    if (go) {
+        const uint64_t e[6] = {((uint64_t)e01.y << 32) | e01.x, ((uint64_t)e01.w << 32) | e01.z,
+                               ((uint64_t)e23.y << 32) | e23.x, ((uint64_t)e23.w << 32) | e23.z,
+                               ((uint64_t)e45.y << 32) | e45.x, ((uint64_t)e45.w << 32) | e45.z};
+        uint32_t l;
+        const int c = cmp_entry(w, m, e, h.z, h.w & 0xFFu, d.n, d.text, qw, &l);
+        step(c, bd.pivot(), l, (h.w >> 8) & 0xFFu, (h.w >> 16) & 0xFFu);
+    }
+    for (uint32_t p = 0; p < kLaneProbes && __any_sync(0xFFFFFFFFu, go); p++) {
+        const uint32_t M = bd.pivot();
+        uint4 r0, r1;
+        ldg32_if(go, d.rec + 2 * (size_t)M, &r0, &r1);
+        if (go) {
+            uint32_t l;
+            bool und = false;
+            int c = cmp_record(w[0], w[1], w[2], w[3], m, r0, r1, d.n, &l, &und);
+            if (und) c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
+            step(c, M, l, (r1.z >> 8) & 0xFFu, r1.z & 0xFFu);
+        }
+    }
+    // one bracket of both bounds, as for the worklist of front.cu
+    const uint32_t L = bd.phase == 2 ? bd.lo - 1u : bd.L, R = bd.phase == 1 ? bd.HR : bd.R;
+    unsigned rest = __ballot_sync(0xFFFFFFFFu, live && !done);
+    while (rest != 0u) {
+        const int src = __ffs(rest) - 1;
+        rest &= rest - 1u;
+        uint64_t wq[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) wq[j] = shfl64(w[j], src);
+        const uint32_t mq = __shfl_sync(0xFFFFFFFFu, m, src), rq = __shfl_sync(0xFFFFFFFFu, r, src);
+        const AsciiWindows qwq{qw.ascii, qw.total, shfl64(qa, src), mq, __shfl_sync(0xFFFFFFFFu, (int)rc, src) != 0};
+        uint64_t l, u;
+        finish_by_warp(sdesc[kSingle ? 0u : rq], qwq, wq, mq, __shfl_sync(0xFFFFFFFFu, L, src),
+                       __shfl_sync(0xFFFFFFFFu, R, src), &l, &u);
+        if ((int)lane == src) {
+            lo = l;
+            hi = u;
+        }
+    }
+    if (live) store_result_sum(a, q, lo, hi);
+    const bool any_bad = __any_sync(0xFFFFFFFFu, live && !ok && !bad_ref);
+    const bool any_bad_ref = __any_sync(0xFFFFFFFFu, bad_ref);
+    if (lane == 0 && any_bad && a.pack_err != nullptr) atomicOr(a.pack_err, 1);
+    if (lane == 0 && any_bad_ref && a.bad_ref != nullptr) atomicOr(a.bad_ref, 1);
+}
+
+}  // namespace
+
+cudaError_t launch_search_small(const SearchLaunch &L, cudaStream_t s) {
+    if (L.n_q == 0) return cudaSuccess;
+    // the fewest queries per warp (a power of two) with which the batch's
+    // warps are all resident
+    const uint64_t warps = (uint64_t)device_sm_count() * kSmallPerSm * (kSmallThreads / 32);
+    uint32_t per_warp = 1;
+    while (per_warp < 32 && per_warp * warps < L.n_q) per_warp *= 2;
+    const uint64_t per_cta = (uint64_t)per_warp * (kSmallThreads / 32);
+    const unsigned blocks = (unsigned)((L.n_q + per_cta - 1) / per_cta);
+    if (L.n_refs == 1 && L.q_ref == nullptr)
+        small_kernel<true><<<blocks, kSmallThreads, 0, s>>>(L, per_warp);
+    else
+        small_kernel<false><<<blocks, kSmallThreads, 0, s>>>(L, per_warp);
+    return cudaGetLastError();
+}
+
+}  // namespace sa
