@@ -106,8 +106,8 @@ typedef struct sa_search_params {
                                    SA_PARAM_REVERSE_COMPLEMENT: search the other strand */
     uint32_t front_probes;      /* probes per query in the one-thread-per-query first
                                    pass before a query joins the worklist of the
-                                   persistent kernel, at most 64 (0: 1 when some
-                                   index has more suffixes than k-mers, else 3) */
+                                   persistent kernel, at most 64 (0: 1 in input
+                                   order, 3 in k-mer order) */
     uint64_t q_first;           /* q_offsets[0] */
     uint64_t q_total;           /* q_offsets[n_q] - q_offsets[0] */
     int32_t *device_status;     /* optional caller-owned int32 in device memory: at the end

@@ -144,18 +144,24 @@ uint32_t floor_log2(uint64_t x) {
 }
 
 constexpr uint32_t kDefaultDepth = 13;
-// First-pass probes when the caller sets none.  With fewer suffixes than
-// k-mers the entry's pivot settles most queries and two more probes settle
-// nearly all; with more suffixes than k-mers (brackets of several suffixes and
-// repeat copies) the first pass's warps would idle on their widest lanes, so
-// every query the entry does not settle goes straight to the persistent pass.
-// (Measured: 3 probes best at n/4^k = 0.37 and 0.72, 1 probe at 2.9.)
-uint32_t default_front_probes(const sa_index *const *refs, uint32_t n_refs) {
+// First-pass probes when the caller sets none.  In input order one, the
+// entry's pivot: what it does not settle goes to the persistent pass, whose
+// lanes stay full, where more probes here would leave the first pass's warps
+// to their widest lanes (1, 2 and 3 probes: 10^7 reads at 100 Mbp 866, 873,
+// 886 us a call; four genomes 1549, 1621, 1671; 1024-base queries 663, 694,
+// 744).  In k-mer order neighbouring lanes share lines, and three do best (3.1
+// Gbp 9885, 7763, 7677; four 7781).
+constexpr uint32_t kInputOrderProbes = 1;
+constexpr uint32_t kKmerOrderProbes = 3;
+
+// Whether some index has more suffixes than k-mers: brackets of several
+// suffixes then are the rule.
+bool wide_brackets(const sa_index *const *refs, uint32_t n_refs) {
     for (uint32_t r = 0; r < n_refs; r++) {
         const sa_index *x = refs[r];
-        if (x->kmer_k && x->n > (1ull << (2 * x->kmer_k))) return 1;
+        if (x->kmer_k && x->n > (1ull << (2 * x->kmer_k))) return true;
     }
-    return 3;
+    return false;
 }
 constexpr uint32_t kSmemBudget = 200 * 1024;
 
@@ -262,7 +268,7 @@ constexpr uint64_t kSmallBases = 1ull << 26;
 bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uint64_t total) {
     for (uint32_t r = 0; r < n_refs; r++)
         if (!refs[r]->krt && n_q > kSmallQueriesNoTable) return false;
-    return n_q <= kSmallQueries && total <= (default_front_probes(refs, n_refs) == 1 ? kSmallBases / 2 : kSmallBases);
+    return n_q <= kSmallQueries && total <= (wide_brackets(refs, n_refs) ? kSmallBases / 2 : kSmallBases);
 }
 
 // The search of a batch whose inputs are in device memory: ascii holds the
@@ -373,10 +379,8 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.threads = threads;
     L.blocks = (uint32_t)sms * bps;
     L.chunk = params && params->chunk ? params->chunk : 64;
-    // with the queries in k-mer order neighbouring lanes share pages and rows,
-    // and the first pass does best with three probes (measured)
     L.front_probes = params && params->front_probes ? params->front_probes
-                                                    : (kmer_order ? 3u : default_front_probes(refs, n_refs));
+                                                    : (kmer_order ? kKmerOrderProbes : kInputOrderProbes);
     L.revcomp = revcomp;
     L.strand_bits = strand_bits;
     L.expire_waits = params && (params->flags & SA_PARAM_EXPIRE_WAITS);

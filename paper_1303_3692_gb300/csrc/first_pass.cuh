@@ -57,13 +57,12 @@ template <typename Windows>
 __device__ __forceinline__ int cmp_entry(const uint64_t w[4], uint32_t m, const uint64_t e[6], uint32_t pos,
                                          uint32_t clamp, uint32_t n, const uint64_t *__restrict__ T,
                                          const Windows &qw, uint32_t *lcp) {
+    bool undecided = false;
+    int c = cmp_first(w, e, m, 128u, clamp, lcp, &undecided);
+    if (!undecided) return c;
 #pragma unroll
-    for (int j = 0; j < 6; j++) {
-        const uint32_t off = 32u * j;
-        const uint32_t qlen = min(32u, m - off);
-        const uint32_t tlen = clamp > off ? min(32u, clamp - off) : 0u;
-        const uint64_t q = j < 4 ? w[j] : qw(off);
-        const int c = cmp_window(q, e[j], qlen, tlen, off, m, lcp);
+    for (uint32_t off = 128u; off < 192u; off += 32u) {
+        c = cmp_window(qw(off), e[off / 32u], min(32u, m - off), clamp > off ? min(32u, clamp - off) : 0u, off, m, lcp);
         if (c != 2) return c;
     }
     return cmp_suffix_qw(T, n, pos, qw, m, 192u, lcp);

@@ -30,24 +30,29 @@ namespace {
 
 constexpr int kFrontThreads = 256;
 
-// The list slot of the j-th record of the k-mer-ordered list: region by
-// region (in the largest bucket b whose regions before it hold at most j
-// records), then the overflow region.  prefix: the exclusive sums of the
-// regions' fills (kNumBuckets + 2 entries, the last their total); start: each
-// region's first slot.
+// The list slot of each lane's record j = base + lane of the k-mer-ordered
+// list: region by region (in the largest bucket b whose regions before it hold
+// at most j records), then the overflow region.  prefix: the exclusive sums of
+// the regions' fills (kNumBuckets + 2 entries, the last their total); start:
+// each region's first slot.  The warp finds base's bucket together (32 of the
+// sums, then the 9 that follow the last that is small enough: two reads of
+// shared memory against the eight a binary search makes one after the other),
+// and the few lanes past its end step on from there.
 __device__ __forceinline__ uint32_t list_slot(const uint32_t *prefix, const uint32_t *start, uint32_t ov_start,
-                                              uint32_t j) {
-    const uint32_t in_regions = prefix[kNumBuckets + 1];
+                                              uint32_t base) {
+    static_assert(kNumBuckets == 256, "the sums are looked through 9 at a time, 32 * 9 >= kNumBuckets + 1");
+    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t in_regions = prefix[kNumBuckets + 1], j = base + lane;
+    const uint32_t coarse = 9u * lane;
+    const unsigned below = __ballot_sync(0xFFFFFFFFu, coarse <= kNumBuckets && prefix[min(coarse, kNumBuckets)] <= base);
+    const uint32_t group = 9u * (31u - __clz(below));  // (prefix[0] = 0: lane 0 votes)
+    const uint32_t fine = group + lane;
+    const unsigned in_group =
+        __ballot_sync(0xFFFFFFFFu, lane < 9u && fine <= kNumBuckets && prefix[min(fine, kNumBuckets)] <= base);
+    uint32_t b = group + 31u - __clz(in_group);
     if (j >= in_regions) return ov_start + (j - in_regions);
-    uint32_t lo = 0, hi = kNumBuckets + 1;  // prefix[lo] <= j < prefix[hi]
-    while (hi - lo > 1u) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (prefix[mid] <= j)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return start[lo] + (j - prefix[lo]);
+    while (prefix[b + 1] <= j) b++;
+    return start[b] + (j - prefix[b]);
 }
 
 // kFromList: the queries come from the k-mer-ordered list of bucket.cu (one
@@ -112,7 +117,8 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         uint32_t lslot = 0;  // the record's slot in the list (list input)
         if (kFromList) {
             uint4 c0, c1, c2, c3;
-            if (live) lslot = list_slot(s_lprefix, s_lstart, ov_start, (uint32_t)(base + lane));
+            const uint32_t slot = list_slot(s_lprefix, s_lstart, ov_start, (uint32_t)base);
+            if (live) lslot = slot;
             const uint4 *src = a.wrec_in + 4 * (size_t)lslot;
             ldg32_if(live, src, &c0, &c1);
             ldg32_if(live, src + 2, &c2, &c3);
@@ -163,14 +169,20 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         Bounds bd;
         bd.start(look ? h.x - 1u : 0xFFFFFFFFu, look ? h.y : d.n);  // 0xFFFFFFFF stands for -1
 
+        // A query's result waits in lo and hi for the end of the iteration, so
+        // that the warp stores its lanes' results once.
         bool done = !live || !ok || m == 0 || (look && bd.R - bd.L <= 1u);
-        if (live && !ok) store_result_sum(a, q, ~0ull, ~0ull);
-        if (live && ok && m == 0) store_result_sum(a, q, 0, d.n);
-        if (live && ok && m > 0 && look && bd.R - bd.L <= 1u) store_result_sum(a, q, bd.R, bd.R);
-        if (live && ok && m > 0 && d.krt != nullptr && m < kk) {
-            uint32_t lo, hi;
-            brief_interval(d, w[0] >> (64u - 2u * m), m, &lo, &hi);
-            store_result_sum(a, q, lo, hi);
+        uint64_t lo = bd.R, hi = bd.R;  // a bracket without suffixes
+        if (!ok) lo = hi = ~0ull;
+        if (ok && m == 0) {
+            lo = 0;
+            hi = d.n;
+        }
+        if (ok && m > 0 && d.krt != nullptr && m < kk) {
+            uint32_t l, u;
+            brief_interval(d, w[0] >> (64u - 2u * m), m, &l, &u);
+            lo = l;
+            hi = u;
             done = true;
         }
 
@@ -185,7 +197,8 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         // pivot's own common prefixes with its neighbours).
         auto step = [&](int c, uint32_t M, uint32_t l, uint32_t lp, uint32_t ln) {
             if (bd.step(c, M, l, m, lp, ln)) {
-                store_result_sum(a, q, bd.first(), bd.R);
+                lo = bd.first();
+                hi = bd.R;
                 done = true;
                 go = false;
             }
@@ -208,12 +221,14 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
             if (go) {
                 uint32_t l;
                 bool und = false;
-                int c = cmp_record(w[0], w[1], w[2], w[3], m, r0, r1, d.n, &l, &und);
+                int c = cmp_record(w, m, r0, r1, d.n, &l, &und);
                 if (und)
                     c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
                 step(c, M, l, (r1.z >> 8) & 0xFFu, r1.z & 0xFFu);
             }
         }
+
+        if (live && done) store_result_sum(a, q, lo, hi);
 
         // The rest goes to the worklist with one bracket of both bounds:
         // phase 0 (L, R); phase 1 (L, HR) (lo in (L, M], hi in [M, HR));

@@ -380,29 +380,44 @@ __device__ __forceinline__ int cmp_window(uint64_t q, uint64_t t, uint32_t qlen,
     return 2;
 }
 
+// P (its first 128 bases in q; length m >= 1) against the first `known` <= 128
+// bases of a suffix (t; zero past them) of `left` bases: the outcome with *lcp
+// set, or CMP_PREFIX with *undecided when all known bases agree and both go
+// on.  One path for every outcome -- the first differing word and the query's
+// are picked by selects, and the highest differing bit tells the order -- as
+// the lanes of a warp end in different words: a test per word, each taken by
+// some lanes, cost twice the instructions, which bound the first pass (57 % of
+// issue slots, 1300 instructions per 32 queries).
+__device__ __forceinline__ int cmp_first(const uint64_t q[4], const uint64_t t[4], uint32_t m, uint32_t known,
+                                         uint32_t left, uint32_t *lcp, bool *undecided) {
+    const uint64_t x0 = q[0] ^ t[0], x1 = q[1] ^ t[1], x2 = q[2] ^ t[2], x3 = q[3] ^ t[3];
+    const bool low = (x0 | x1) != 0, first = (low ? x0 : x2) != 0;
+    const uint64_t x = low ? (first ? x0 : x1) : (first ? x2 : x3);
+    const uint64_t qx = low ? (first ? q[0] : q[1]) : (first ? q[2] : q[3]);
+    const uint32_t z = (uint32_t)__clzll((long long)x);  // 64 when no word differs
+    const uint32_t d = (low ? 0u : 64u) + (first ? 0u : 32u) + (z >> 1);
+    const uint32_t have = min(known, left), lim = min(m, have);
+    *lcp = min(d, lim);
+    if (d < lim) return ((qx << (z & 63u)) >> 63) != 0 ? CMP_GREATER : CMP_LESS;
+    if (have < m && have < known) return CMP_GREATER;  // the suffix ends first
+    *undecided = m > known;
+    return CMP_PREFIX;
+}
+
 // Bases a suffix record holds.
 constexpr uint32_t kRecBases = 104;
 
-// P (bases 0-63 in q0, q1, bases 64-127 in x2, x3; length m >= 1) against a
-// 32-byte suffix record (r0 = bases 0-63, r1 = bases 64-95, 96-103 with the
-// neighbours' common prefixes, and the position).  Sets *undecided when all
-// 104 bases agree, m > 104 and the suffix has 104 bases or more; the compare
-// then continues in the text.
-__device__ __forceinline__ int cmp_record(uint64_t q0, uint64_t q1, uint64_t x2, uint64_t x3, uint32_t m, uint4 r0,
-                                          uint4 r1, uint32_t n, uint32_t *lcp, bool *undecided) {
-    const uint32_t klen = min(kRecBases, n - r1.w);
-    int c = cmp_window(q0, ((uint64_t)r0.y << 32) | r0.x, min(32u, m), min(32u, klen), 0u, m, lcp);
-    if (c != 2) return c;
-    c = cmp_window(q1, ((uint64_t)r0.w << 32) | r0.z, min(32u, m - 32u), min(32u, klen - 32u), 32u, m, lcp);
-    if (c != 2) return c;
-    c = cmp_window(x2, ((uint64_t)r1.y << 32) | r1.x, min(32u, m - 64u), min(32u, klen - 64u), 64u, m, lcp);
-    if (c != 2) return c;
-    c = cmp_window(x3 & 0xFFFF000000000000ull, (uint64_t)(r1.z & 0xFFFF0000u) << 32, min(8u, m - 96u),
-                   min(8u, klen - 96u), 96u, m, lcp);
-    if (c != 2) return c;
-    *undecided = true;
-    *lcp = kRecBases;
-    return CMP_PREFIX;
+// P (its first 128 bases in q; length m >= 1) against a 32-byte suffix record
+// (r0 = bases 0-63, r1 = bases 64-95, 96-103 with the neighbours' common
+// prefixes, and the position).  Sets *undecided when all 104 bases agree, m >
+// 104 and the suffix has 104 bases or more; the compare then continues in the
+// text.
+__device__ __forceinline__ int cmp_record(const uint64_t q[4], uint32_t m, uint4 r0, uint4 r1, uint32_t n,
+                                          uint32_t *lcp, bool *undecided) {
+    const uint64_t qm[4] = {q[0], q[1], q[2], q[3] & 0xFFFF000000000000ull};
+    const uint64_t t[4] = {((uint64_t)r0.y << 32) | r0.x, ((uint64_t)r0.w << 32) | r0.z,
+                           ((uint64_t)r1.y << 32) | r1.x, (uint64_t)(r1.z & 0xFFFF0000u) << 32};
+    return cmp_first(qm, t, m, kRecBases, n - r1.w, lcp, undecided);
 }
 
 // The lengths of the common prefixes of the suffix at a rank with the

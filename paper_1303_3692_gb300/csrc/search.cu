@@ -299,7 +299,8 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             k = (c == CMP_PREFIX || nk >= (1u << depth)) ? 0u : nk;
         } else {
             bool und = false;
-            c = cmp_record(q0, q1, x2, x3, m, r0, r1, n, &l, &und);
+            const uint64_t qw4[4] = {q0, q1, x2, x3};
+            c = cmp_record(qw4, m, r0, r1, n, &l, &und);
             if (und) {
                 // query bases 96-127 are x3, 128-159 the worklist record's second word pair
                 const QueryWindows<kStrands> qw{a.tq, qa, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};

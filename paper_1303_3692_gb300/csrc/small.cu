@@ -82,7 +82,7 @@ __device__ __forceinline__ void finish_by_warp(const FrontDesc &d, const AsciiWi
         if (live) {
             uint32_t l;
             bool und = false;
-            c = cmp_record(w[0], w[1], w[2], w[3], m, r0, r1, d.n, &l, &und);
+            c = cmp_record(w, m, r0, r1, d.n, &l, &und);
             if (und) c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, kRecBases, &l);
         }
         const uint32_t cut = min(m, kLcpCap);
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kSmallThreads, kSmallPerSm) small_kernel(const
         if (go) {
             uint32_t l;
             bool und = false;
-            int c = cmp_record(w[0], w[1], w[2], w[3], m, r0, r1, d.n, &l, &und);
+            int c = cmp_record(w, m, r0, r1, d.n, &l, &und);
             if (und) c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
             step(c, M, l, (r1.z >> 8) & 0xFFu, r1.z & 0xFFu);
         }
