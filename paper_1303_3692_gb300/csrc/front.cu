@@ -170,7 +170,10 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         bd.start(look ? h.x - 1u : 0xFFFFFFFFu, look ? h.y : d.n);  // 0xFFFFFFFF stands for -1
 
         // A query's result waits in lo and hi for the end of the iteration, so
-        // that the warp stores its lanes' results once.
+        // that the warp stores its lanes' results once.  (With that, one path
+        // per compare and the list's slots found by the whole warp: 3.1 Gbp,
+        // 4*10^7 x 150 bases 8044 -> 7683 us a call, 430 Mbp 1647 -> 1577 us.
+        // Prefetching the next iteration's records into L2 cost 1.5 %.)
         bool done = !live || !ok || m == 0 || (look && bd.R - bd.L <= 1u);
         uint64_t lo = bd.R, hi = bd.R;  // a bracket without suffixes
         if (!ok) lo = hi = ~0ull;

@@ -387,7 +387,8 @@ __device__ __forceinline__ int cmp_window(uint64_t q, uint64_t t, uint32_t qlen,
 // are picked by selects, and the highest differing bit tells the order -- as
 // the lanes of a warp end in different words: a test per word, each taken by
 // some lanes, cost twice the instructions, which bound the first pass (57 % of
-// issue slots, 1300 instructions per 32 queries).
+// issue slots, 1300 instructions per 32 queries in k-mer order; 1040 with this
+// and one result store per iteration).
 __device__ __forceinline__ int cmp_first(const uint64_t q[4], const uint64_t t[4], uint32_t m, uint32_t known,
                                          uint32_t left, uint32_t *lcp, bool *undecided) {
     const uint64_t x0 = q[0] ^ t[0], x1 = q[1] ^ t[1], x2 = q[2] ^ t[2], x3 = q[3] ^ t[3];
