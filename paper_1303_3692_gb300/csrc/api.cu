@@ -271,6 +271,14 @@ bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uin
     return n_q <= kSmallQueries && total <= (wide_brackets(refs, n_refs) ? kSmallBases / 2 : kSmallBases);
 }
 
+// Whether, in k-mer order, the scatter packs the ASCII bases it needs itself,
+// tile by tile, instead of reading a packed copy of the batch that a kernel
+// before it writes: for queries of up to 192 bases on average, which its tiles
+// have room for and its records carry (longer ones are compared in the packed
+// copy past that).  Words have 32-bit numbers there.
+constexpr uint64_t kFusedBases = 192;
+bool fused_packing(uint64_t n_q, uint64_t total) { return total <= kFusedBases * n_q && total < (1ull << 36); }
+
 // The search of a batch whose inputs are in device memory: ascii holds the
 // batch's bases from offset `first` on (query q is ascii[q_off[q] - first ..
 // q_off[q + 1] - first)), q_off and q_ref are device arrays and out device
@@ -326,19 +334,20 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     // list and worklist records hold a query's first base in 48 bits (a batch
     // that large could not be resident anyway)
     if (!plain && tq_words * 32 >= kListMaxBase) return SA_ERR_ARG;
-    uint64_t *tq = sc.get<uint64_t>(SA_TQ_LEAD_WORDS + tq_words) + SA_TQ_LEAD_WORDS;
-    uint32_t *tv = sc.get<uint32_t>(tq_words);
+    const bool kmer_order = !plain && use_kmer_order(refs, n_refs, n_q, order);
+    const bool fused = kmer_order && fused_packing(n_q, total);
+    uint64_t *tq = fused ? nullptr : sc.get<uint64_t>(SA_TQ_LEAD_WORDS + tq_words) + SA_TQ_LEAD_WORDS;
+    uint32_t *tv = fused ? nullptr : sc.get<uint32_t>(tq_words);
     uint4 *wrec = plain ? nullptr : sc.get<uint4>(4 * n_q);
     uint64_t ktotal = 0;
     for (uint32_t r = 0; r < n_refs; r++)
         if (refs[r]->krt) ktotal += 1ull << (2 * refs[r]->kmer_k);
-    const bool kmer_order = !plain && use_kmer_order(refs, n_refs, n_q, order);
     uint4 *wrec_in = kmer_order ? sc.get<uint4>(4 * list_capacity(n_q)) : nullptr;
     // What starts at zero, in one block: flags [0] pack error, [1] status, [2]
     // worklist count, [3] bad reference id, [4] records of the k-mer-ordered
     // list, [5] a non-base byte in the batch; the persistent pass's counter;
     // the k-mer order's plan; the bitmap of packed words with a non-base byte.
-    const size_t plan_words = kmer_order ? kPlanWords : 0, bitmap_words = tq_words / 32 + 1;
+    const size_t plan_words = kmer_order ? kPlanWords : 0, bitmap_words = fused ? 0 : tq_words / 32 + 1;
     uint32_t *zeroed = sc.get<uint32_t>(10 + plan_words + bitmap_words);
     if (sc.failed) return SA_ERR_NOMEM;
     int *flags = reinterpret_cast<int *>(zeroed);
@@ -387,14 +396,15 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.trunc_cap = trunc_cap;
     L.tile_kept = tile_kept;
     L.tile_sum_by_warp = !kmer_order;
-    L.ktotal = ktotal;
+    L.kscale = ktotal ? ~0ull / ktotal : 0;
     L.bplan = bplan;
     L.wrec_in = wrec_in;
     L.wl_in_count = reinterpret_cast<uint32_t *>(flags + 4);
     L.bad_ref = flags + 3;
     L.batch_dirty = flags + 5;
+    L.fused = fused;
 
-    if ((err = launch_pack_batch(L, tq, tvb, tv, s)) != cudaSuccess) return status_from_cuda(err);
+    if (!fused && (err = launch_pack_batch(L, tq, tvb, tv, s)) != cudaSuccess) return status_from_cuda(err);
     return search_timed(params, s, [&] {
         if (plain) return launch_search_plain(L, s);
         cudaError_t e = kmer_order ? launch_bucketed_worklist(L, wrec_in, s) : cudaSuccess;

@@ -23,7 +23,8 @@
 //                          of the list (9/8 of its estimated size plus 256
 //                          records), in bucket order, and after them an
 //                          overflow region with room for every query;
-//   bucket_scatter_kernel  per tile of queries: offsets, strand, reference,
+//   bucket_scatter_kernel (or, for an unpacked batch, bucket_scatter_ascii_kernel)
+//                          per tile of queries: offsets, strand, reference,
 //                          validity of every base when the packing found a
 //                          non-base byte in the batch (invalid and empty
 //                          queries get their results here) and bucket; each
@@ -41,7 +42,7 @@
 // Sizing the regions from a sample spares a pass over the whole batch that
 // exact counts would need; the overflow region keeps the result exact
 // whatever the sample missed.
-#include "sa_internal.cuh"
+#include "first_pass.cuh"
 
 namespace sa {
 
@@ -77,12 +78,13 @@ __device__ __forceinline__ bool query_range(const SearchLaunch &a, uint64_t q, u
 __device__ __forceinline__ uint16_t bucket_of(const SearchLaunch &a, const BucketRef &d, uint32_t m, uint64_t w0) {
     if (d.kmer_k != 0 && m >= d.kmer_k) {
         const uint64_t x = w0 >> (64u - 2u * d.kmer_k);
-        return (uint16_t)(((d.kbase + x) * kNumBuckets) / a.ktotal);
+        static_assert(kNumBuckets == 256, "the shift below");
+        return (uint16_t)__umul64hi((d.kbase + x) << 8, a.kscale);  // about 256 (kbase + x) / ktotal
     }
     return (uint16_t)kNumBuckets;  // no k-mer bracket: the key-table descent
 }
 
-template <bool kSingle, bool kStrands>
+template <bool kSingle, Bases kBases>
 __global__ void __launch_bounds__(kSampleThreads) bucket_sample_kernel(const __grid_constant__ SearchLaunch a) {
     __shared__ uint32_t hist[kNumBuckets + 1];
     __shared__ BucketRef sref[SA_MAX_REFS];
@@ -100,8 +102,8 @@ __global__ void __launch_bounds__(kSampleThreads) bucket_sample_kernel(const __g
         uint32_t m;
         bool bad_range, bad_ref;
         // an estimate: the bases' validity is left to the scatter
-        if (query_range<kStrands>(a, q, &r, &at, &m, &bad_range, &bad_ref) && m > 0)
-            atomicAdd(&hist[bucket_of(a, sref[kSingle ? 0u : r], m, query_window<kStrands>(a.tq, at, 0))], 1u);
+        if (query_range<kBases != Bases::Packed>(a, q, &r, &at, &m, &bad_range, &bad_ref) && m > 0)
+            atomicAdd(&hist[bucket_of(a, sref[kSingle ? 0u : r], m, window_source<kBases>(a, at, m)(0))], 1u);
     }
     __syncthreads();
     for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x)
@@ -150,6 +152,39 @@ constexpr int kScatterThreads = 256;
 constexpr int kScatterItems = 2;
 constexpr uint32_t kScatterTile = (uint32_t)kScatterThreads * kScatterItems;  // 32 KB of records
 constexpr size_t kScatterSmem = (size_t)kScatterTile * 64;
+
+// A tile's runs: exclusive scan of its counts (first warp), and each run's
+// place in the list, reserved with one atomic per bucket.
+__device__ __forceinline__ void reserve_runs(const SearchLaunch &a, const uint32_t *cnt, uint32_t *off, uint32_t *base,
+                                             uint32_t *inreg, uint32_t *ovbase, uint32_t *n_valid) {
+    if (threadIdx.x < 32) {
+        const unsigned lane = threadIdx.x;
+        uint32_t carry = 0;
+        for (unsigned s0 = 0; s0 <= kNumBuckets; s0 += 32) {
+            const unsigned i = s0 + lane;
+            const uint32_t v = i <= kNumBuckets ? cnt[i] : 0u;
+            uint32_t x = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= (unsigned)o) x += y;
+            }
+            if (i <= kNumBuckets) off[i] = carry + x - v;
+            carry += __shfl_sync(0xFFFFFFFFu, x, 31);
+        }
+        if (lane == 0) *n_valid = carry;
+    }
+    for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x) {
+        const uint32_t c = cnt[i];
+        if (c == 0) continue;
+        const uint32_t start = atomicAdd(a.bplan + kPlanCursor + i, c);
+        const uint32_t end = a.bplan[kPlanStart + i] + a.bplan[kPlanCap + i];
+        const uint32_t fit = start >= end ? 0u : (end - start < c ? end - start : c);
+        base[i] = start;
+        inreg[i] = fit;
+        ovbase[i] = fit < c ? atomicAdd(a.bplan + kPlanOvCursor, c - fit) : 0u;
+    }
+}
 
 template <bool kSingle, bool kStrands>
 __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(const __grid_constant__ SearchLaunch a,
@@ -219,35 +254,7 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
 #pragma unroll
     for (int it = 0; it < kScatterItems; it++) rank[it] = b[it] != kNoQuery ? atomicAdd(&cnt[b[it]], 1u) : 0u;
     __syncthreads();
-    // the tile's runs: exclusive scan of its counts (first warp), and each
-    // run's place in the list, reserved with one atomic per bucket
-    if (threadIdx.x < 32) {
-        const unsigned lane = threadIdx.x;
-        uint32_t carry = 0;
-        for (unsigned s0 = 0; s0 <= kNumBuckets; s0 += 32) {
-            const unsigned i = s0 + lane;
-            const uint32_t v = i <= kNumBuckets ? cnt[i] : 0u;
-            uint32_t x = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= (unsigned)o) x += y;
-            }
-            if (i <= kNumBuckets) off[i] = carry + x - v;
-            carry += __shfl_sync(0xFFFFFFFFu, x, 31);
-        }
-        if (lane == 0) n_valid = carry;
-    }
-    for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x) {
-        const uint32_t c = cnt[i];
-        if (c == 0) continue;
-        const uint32_t start = atomicAdd(a.bplan + kPlanCursor + i, c);
-        const uint32_t end = a.bplan[kPlanStart + i] + a.bplan[kPlanCap + i];
-        const uint32_t fit = start >= end ? 0u : (end - start < c ? end - start : c);
-        base[i] = start;
-        inreg[i] = fit;
-        ovbase[i] = fit < c ? atomicAdd(a.bplan + kPlanOvCursor, c - fit) : 0u;
-    }
+    reserve_runs(a, cnt, off, base, inreg, ovbase, &n_valid);
     __syncthreads();
 #pragma unroll
     for (int it = 0; it < kScatterItems; it++) {
@@ -280,6 +287,209 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
         list[4 * g + (c & 3u)] = srec[c];
     }
     const unsigned lane = threadIdx.x & 31u;
+    if (__any_sync(0xFFFFFFFFu, any_bad) && lane == 0) atomicOr(a.pack_err, 1);
+    if (__any_sync(0xFFFFFFFFu, any_bad_ref) && lane == 0) atomicOr(a.bad_ref, 1);
+}
+
+// The scatter of a batch that is not packed (api.cu: fused_packing).  The CTA
+// packs its tile's bases itself, coalesced, into shared memory -- consecutive
+// queries are one stretch of the batch -- and every 16-byte piece of a record
+// is computed from there as it is stored, so the packed batch is neither
+// written nor read back: per query of 150 bases 150 + 64 bytes of HBM traffic
+// instead of 150 + 38 + 38 + 64.  What a record holds, the runs and their
+// reservation are as above.  Bound by the integer pipe (69 % busy; HBM 53 %):
+// 4*10^7 x 150 bases 1.99 ms, where the packing and the scatter took 1.19 +
+// 1.29 ms; 9*10^6 of 100-151 bases of both strands, some with an N, 0.47 ms for
+// 0.24 + 0.33.  (The same in the first pass of input order, a tile per warp, was
+// no faster at 100 bases, 586 us for 577, and slower at 20-250, 1263 for 1144:
+// its warps wait for their reads in turn.)
+constexpr uint32_t kTileWords = kScatterTile * 6;  // 192 bases per query; more: each query by itself
+constexpr uint32_t kTileLead = 6, kTilePad = 8;
+constexpr size_t kScatterAsciiSmem = (kTileLead + kTileWords + kTilePad) * 8 + kScatterTile * 16;
+
+// 16 bases of a tile as a 32-bit word, base 0 on top: the tile holds its packed
+// words' high halves before their low ones, so a window at any base is a funnel
+// shift of two neighbours.
+__device__ __forceinline__ uint32_t tile_window16(const uint32_t *half, int base) {
+    const int i = base >> 4;
+    return __funnelshift_l(half[i + 1], half[i], 2u * (uint32_t)(base & 15));
+}
+
+__device__ __forceinline__ uint32_t rc_window16(uint32_t x) {
+    const uint32_t f = __brev(~x);
+    return ((f >> 1) & 0x55555555u) | ((f & 0x55555555u) << 1);
+}
+
+// The N x 16 bases from base `off` of a query whose first base (for the other
+// strand, one past its last) is base `at` of the tile.
+template <int N>
+__device__ __forceinline__ void tile_windows(const uint32_t *half, int at, bool rc, int off, uint32_t w[N]) {
+    const int b = rc ? at - off - 16 * N : at + off;
+    uint32_t t[N];
+#pragma unroll
+    for (int j = 0; j < N; j++) t[j] = tile_window16(half, b + 16 * j);
+#pragma unroll
+    for (int j = 0; j < N; j++) w[j] = rc ? rc_window16(t[N - 1 - j]) : t[j];
+}
+
+template <bool kSingle>
+__global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kernel(const __grid_constant__ SearchLaunch a,
+                                                                                 uint4 *__restrict__ list) {
+    // the tile's words (kTileLead of no meaning before, kTilePad after), then its records' headers
+    extern __shared__ uint2 stile[];
+    uint2 *words = stile + kTileLead;
+    const uint32_t *half = reinterpret_cast<const uint32_t *>(words);
+    uint4 *head = reinterpret_cast<uint4 *>(stile + kTileLead + kTileWords + kTilePad);
+    __shared__ uint32_t cnt[kNumBuckets + 1];
+    __shared__ uint32_t off[kNumBuckets + 1];
+    __shared__ uint32_t base[kNumBuckets + 1];
+    __shared__ uint32_t inreg[kNumBuckets + 1];
+    __shared__ uint32_t ovbase[kNumBuckets + 1];
+    __shared__ uint32_t slot_to[kScatterTile];  // each slot's record in the list
+    __shared__ uint32_t marks[kTileWords / 32];
+    __shared__ BucketRef sref[SA_MAX_REFS];
+    __shared__ uint32_t n_valid, w_first, w_last, any_marked;
+    for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x) cnt[i] = 0;
+    for (unsigned r = threadIdx.x; r < a.n_refs; r += blockDim.x) {
+        const RefDesc &d = a.refs.r[r];
+        sref[r] = BucketRef{d.kbase, d.n, d.krt != nullptr ? d.kmer_k : 0u};
+    }
+    if (threadIdx.x == 0) {
+        w_first = 0xFFFFFFFFu;
+        w_last = 0;
+        any_marked = 0;
+    }
+    const unsigned lane = threadIdx.x & 31u;
+    const uint8_t *ascii = reinterpret_cast<const uint8_t *>(a.ascii);
+    const bool aligned16 = ((uintptr_t)ascii & 15u) == 0;
+    const uint64_t tile = (uint64_t)blockIdx.x * kScatterTile;
+    uint16_t b[kScatterItems];
+    uint32_t rank[kScatterItems], r[kScatterItems], m[kScatterItems];
+    uint64_t at[kScatterItems];
+    bool any_bad = false, any_bad_ref = false;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0;  // the words of this thread's queries
+#pragma unroll
+    for (int it = 0; it < kScatterItems; it++) {
+        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+        r[it] = kSingle || q >= a.n_q ? 0u : __ldg(a.q_ref + q);
+        at[it] = 0;
+        m[it] = 0;
+        b[it] = kNoQuery;
+        if (q < a.n_q) {
+            bool bad_range, bad_ref;
+            const bool ok = query_range<true>(a, q, &r[it], &at[it], &m[it], &bad_range, &bad_ref);
+            any_bad |= bad_range;
+            any_bad_ref |= bad_ref;
+            if (ok) {
+                b[it] = 0u;  // usable so far; the bucket follows
+                if (m[it] > 0) {
+                    const uint64_t qa = place_first(at[it], m[it]);
+                    lo = min(lo, (uint32_t)(qa >> 5));
+                    hi = max(hi, (uint32_t)((qa + m[it] - 1) >> 5));
+                }
+            }
+        }
+    }
+    lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+    hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+    __syncthreads();
+    if (lane == 0 && lo <= hi) {
+        atomicMin(&w_first, lo);
+        atomicMax(&w_last, hi);
+    }
+    __syncthreads();
+    const uint32_t w_lo = w_first <= w_last ? w_first : 0u;
+    const uint32_t n_words = w_first <= w_last ? w_last - w_first + 1u : 0u;
+    const bool in_tile = n_words <= kTileWords;
+    if (in_tile) {
+        const uint64_t full = aligned16 ? a.total / 32 : 0;  // words that are two 16-byte loads
+        for (uint32_t i0 = threadIdx.x - lane; i0 < n_words; i0 += kScatterThreads) {
+            const uint32_t i = i0 + lane;
+            const uint64_t w = (uint64_t)w_lo + i;
+            uint32_t bad = 0;
+            if (i < n_words) {
+                const uint4 *from = reinterpret_cast<const uint4 *>(ascii + w * 32);
+                const uint64_t x = w < full ? pack32(__ldg(from), __ldg(from + 1), &bad)
+                                            : pack_edge_word(ascii, a.total, w, &bad);
+                words[i] = make_uint2((uint32_t)(x >> 32), (uint32_t)x);
+            }
+            const unsigned marked = __ballot_sync(0xFFFFFFFFu, bad != 0u);
+            if (lane == 0) {
+                marks[i0 >> 5] = marked;
+                if (marked != 0u) any_marked = 1u;
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kScatterItems; it++) {
+        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+        if (q >= a.n_q) continue;
+        bool valid = b[it] != kNoQuery;
+        uint64_t first = 0;  // the query's first 32 bases
+        if (valid && m[it] > 0) {
+            const uint64_t qa = place_first(at[it], m[it]);
+            if (in_tile) {
+                valid = any_marked == 0u || tile_valid(marks, w_lo, ascii, qa, m[it]);
+                uint32_t f[2];
+                tile_windows<2>(half, (int)((at[it] & ~kPlaceRc) - 32ull * w_lo), (at[it] & kPlaceRc) != 0, 0, f);
+                first = ((uint64_t)f[0] << 32) | f[1];
+            } else {
+                const AsciiWindows own{ascii, a.total, qa, m[it], (at[it] & kPlaceRc) != 0};
+                uint32_t bad = 0;
+                first = own.packed(0, &bad);
+                for (uint32_t o = 32u; o < m[it]; o += 32u) (void)own.packed(o, &bad);
+                valid = bad == 0u;
+            }
+            any_bad |= !valid;
+        }
+        if (!valid) {
+            b[it] = kNoQuery;
+            store_result_sum(a, q, ~0ull, ~0ull);
+        } else if (m[it] == 0) {
+            b[it] = kNoQuery;
+            store_result_sum(a, q, 0, sref[kSingle ? 0u : r[it]].n);
+        } else {
+            b[it] = bucket_of(a, sref[kSingle ? 0u : r[it]], m[it], first);
+        }
+    }
+#pragma unroll
+    for (int it = 0; it < kScatterItems; it++) rank[it] = b[it] != kNoQuery ? atomicAdd(&cnt[b[it]], 1u) : 0u;
+    __syncthreads();
+    reserve_runs(a, cnt, off, base, inreg, ovbase, &n_valid);
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kScatterItems; it++) {
+        if (b[it] == kNoQuery) continue;
+        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+        const uint32_t bk = b[it], slot = off[bk] + rank[it];
+        head[slot] = make_uint4(m[it], (uint32_t)q, (uint32_t)at[it],
+                                place_high(at[it], r[it]) | (bk < kNumBuckets ? kListNeedsEntry : 0u));
+        slot_to[slot] = rank[it] < inreg[bk] ? base[bk] + rank[it] : ovbase[bk] + (rank[it] - inreg[bk]);
+    }
+    __syncthreads();
+    // the runs, 16 bytes per thread per step: the header, or 64 of the
+    // record's 192 bases
+    const uint32_t pieces = 4u * n_valid;
+    for (uint32_t c = threadIdx.x; c < pieces; c += kScatterThreads) {
+        const uint32_t slot = c >> 2, part = c & 3u;
+        uint4 v = head[slot];
+        if (part != 0u) {
+            const int from = 64 * ((int)part - 1);
+            if (in_tile) {
+                uint32_t w[4];
+                tile_windows<4>(half, (int)(place_of(v.z, v.w & ~kRecordRc) - 32ull * w_lo), (v.w & kRecordRc) != 0,
+                                from, w);
+                v = make_uint4(w[1], w[0], w[3], w[2]);
+            } else {
+                const uint64_t place = place_of(v.z, v.w);
+                const AsciiWindows own{ascii, a.total, place_first(place, v.x), v.x, (place & kPlaceRc) != 0};
+                const uint64_t w0 = (uint32_t)from < v.x ? own(from) : 0, w1 = from + 32u < v.x ? own(from + 32u) : 0;
+                v = make_uint4((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32));
+            }
+        }
+        list[4 * (uint64_t)slot_to[slot] + part] = v;
+    }
     if (__any_sync(0xFFFFFFFFu, any_bad) && lane == 0) atomicOr(a.pack_err, 1);
     if (__any_sync(0xFFFFFFFFu, any_bad_ref) && lane == 0) atomicOr(a.bad_ref, 1);
 }
@@ -323,16 +533,22 @@ cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, cuda
     const uint64_t scap = (uint64_t)device_sm_count() * 8;
     if (sblocks > scap) sblocks = scap;
     const bool strands = L.revcomp || L.strand_bits;
-    auto sample = single ? (strands ? bucket_sample_kernel<true, true> : bucket_sample_kernel<true, false>)
-                         : (strands ? bucket_sample_kernel<false, true> : bucket_sample_kernel<false, false>);
+    constexpr Bases P = Bases::Packed, S = Bases::PackedStrands, A = Bases::Ascii;
+    auto sample = single ? (L.fused ? bucket_sample_kernel<true, A>
+                                    : strands ? bucket_sample_kernel<true, S> : bucket_sample_kernel<true, P>)
+                         : (L.fused ? bucket_sample_kernel<false, A>
+                                    : strands ? bucket_sample_kernel<false, S> : bucket_sample_kernel<false, P>);
     sample<<<(unsigned)sblocks, kSampleThreads, 0, s>>>(L);
     bucket_plan_kernel<<<1, 32, 0, s>>>(L);
     const uint64_t stiles = (L.n_q + kScatterTile - 1) / kScatterTile;
-    auto scatter = single ? (strands ? bucket_scatter_kernel<true, true> : bucket_scatter_kernel<true, false>)
-                          : (strands ? bucket_scatter_kernel<false, true> : bucket_scatter_kernel<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
+    auto scatter = single ? (L.fused ? bucket_scatter_ascii_kernel<true>
+                                     : strands ? bucket_scatter_kernel<true, true> : bucket_scatter_kernel<true, false>)
+                          : (L.fused ? bucket_scatter_ascii_kernel<false>
+                                     : strands ? bucket_scatter_kernel<false, true> : bucket_scatter_kernel<false, false>);
+    const size_t smem = L.fused ? kScatterAsciiSmem : kScatterSmem;
+    cudaError_t e = cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    scatter<<<(unsigned)stiles, kScatterThreads, kScatterSmem, s>>>(L, wrec_in);
+    scatter<<<(unsigned)stiles, kScatterThreads, smem, s>>>(L, wrec_in);
     bucket_fill_kernel<<<1, 32, 0, s>>>(L);
     return cudaGetLastError();
 }

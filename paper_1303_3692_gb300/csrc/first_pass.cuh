@@ -68,4 +68,43 @@ __device__ __forceinline__ int cmp_entry(const uint64_t w[4], uint32_t m, const 
     return cmp_suffix_qw(T, n, pos, qw, m, 192u, lcp);
 }
 
+// The source of a record's query's windows, by where the kernel reads bases.
+template <Bases kBases>
+__device__ __forceinline__ auto window_source(const SearchLaunch &a, uint64_t at, uint32_t m) {
+    if constexpr (kBases == Bases::Ascii)
+        return AsciiWindows{reinterpret_cast<const uint8_t *>(a.ascii), a.total, place_first(at, m), m,
+                            (at & kPlaceRc) != 0};
+    else
+        return PackedWindows<kBases == Bases::PackedStrands>{a.tq, at};
+}
+
+// Word w of the batch (bases 32 w .. 32 w + 31) where it is not full or not
+// aligned.
+__device__ __forceinline__ uint64_t pack_edge_word(const uint8_t *__restrict__ ascii, uint64_t total, uint64_t w,
+                                                   uint32_t *bad) {
+    const uint64_t b0 = w * 32;
+    return pack_word(ascii, total, b0, total - b0 < 32 ? (uint32_t)(total - b0) : 32u, bad);
+}
+
+// Whether bytes [qa, qa + m) of the batch (m >= 1) are all bases, given the
+// tile's bits of words that hold a byte that is not (bit i of marks[i / 32]:
+// word w_lo + i, all of the query's words among them); the few marked words'
+// bytes are looked at again.
+__device__ __forceinline__ bool tile_valid(const uint32_t *marks, uint64_t w_lo, const uint8_t *__restrict__ ascii,
+                                           uint64_t qa, uint32_t m) {
+    const uint32_t w0 = (uint32_t)((qa >> 5) - w_lo), w1 = (uint32_t)(((qa + m - 1) >> 5) - w_lo);
+    for (uint32_t g = w0 >> 5; g <= (w1 >> 5); g++) {
+        uint32_t marked = marks[g];
+        if (g == (w0 >> 5)) marked &= 0xFFFFFFFFu << (w0 & 31u);
+        if (g == (w1 >> 5)) marked &= 0xFFFFFFFFu >> (31u - (w1 & 31u));
+        for (; marked != 0u; marked &= marked - 1u) {
+            const uint64_t b0 = (w_lo + g * 32u + (uint32_t)(__ffs(marked) - 1)) * 32;
+            const uint64_t lo = b0 > qa ? b0 : qa, hi = b0 + 32 < qa + m ? b0 + 32 : qa + m;
+            for (uint64_t b = lo; b < hi; b++)
+                if (base_code(__ldg(ascii + b)) > 3u) return false;
+        }
+    }
+    return true;
+}
+
 }  // namespace sa

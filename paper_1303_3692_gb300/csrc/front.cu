@@ -58,12 +58,14 @@ __device__ __forceinline__ uint32_t list_slot(const uint32_t *prefix, const uint
 // kFromList: the queries come from the k-mer-ordered list of bucket.cu (one
 // 64-byte record each: length, index, reference, first base in the packed
 // batch and first 192 bases, already checked) instead of the batch's offsets.
-template <bool kSingle, bool kFromList, bool kStrands>
+template <bool kSingle, bool kFromList, Bases kBases>
 __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_constant__ SearchLaunch a) {
     __shared__ FrontDesc sdesc[SA_MAX_REFS];
     __shared__ uint4 s_stage[kFrontThreads / 32][32][4];  // worklist records staged per warp
     __shared__ uint32_t s_lprefix[kNumBuckets + 2];        // the list's numbering (list input)
     __shared__ uint32_t s_lstart[kNumBuckets + 1];
+    constexpr bool kStrands = kBases != Bases::Packed;
+    static_assert(kFromList || kBases != Bases::Ascii, "in input order the queries come from the packed batch");
     for (unsigned r = threadIdx.x; r < a.n_refs; r += blockDim.x) {
         sdesc[r] = front_desc(a.refs.r[r]);
     }
@@ -98,7 +100,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
 
     const uint64_t n_items = kFromList ? (uint64_t)*a.wl_in_count : a.n_q;
     // a batch without a non-base byte needs no per-query validity check
-    const bool dirty = *a.batch_dirty != 0;
+    const bool dirty = kBases != Bases::Ascii && *a.batch_dirty != 0;
     // Offsets and reference of this lane's next query, read one query ahead.
     uint64_t nqa = 0, nqe = 0;
     uint32_t nr = 0;
@@ -192,10 +194,10 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         bool go = !done && look;
         // in list order, bases 128-191 are the record's last 16 bytes (read
         // again when a compare gets there: an L1 or L2 hit)
-        const QueryWindows<kStrands> qw{tq, qa, w[3],
-                              kFromList ? reinterpret_cast<const uint64_t *>(a.wrec_in + 4 * (size_t)lslot + 3)
-                                        : nullptr,
-                              kFromList ? 2u : 0u};
+        const auto src = window_source<kBases>(a, qa, m);
+        const RecordWindows<decltype(src)> qw{
+            src, w[3], kFromList ? reinterpret_cast<const uint64_t *>(a.wrec_in + 4 * (size_t)lslot + 3) : nullptr,
+            kFromList ? 2u : 0u};
         // One compare's outcome c at pivot M with common prefix l (lp, ln: the
         // pivot's own common prefixes with its neighbours).
         auto step = [&](int c, uint32_t M, uint32_t l, uint32_t lp, uint32_t ln) {
@@ -275,17 +277,18 @@ cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s) {
     if (L.n_q == 0) return cudaSuccess;
     const bool single = L.n_refs == 1 && L.q_ref == nullptr;
     const bool list = L.wrec_in != nullptr;
-    const bool strands = L.revcomp || L.strand_bits;
-    static int per_sm[8][64] = {};
+    static int per_sm[10][64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     using Kernel = void (*)(SearchLaunch);
-    static const Kernel kernels[8] = {front_kernel<false, false, false>, front_kernel<true, false, false>,
-                                      front_kernel<false, true, false>,  front_kernel<true, true, false>,
-                                      front_kernel<false, false, true>,  front_kernel<true, false, true>,
-                                      front_kernel<false, true, true>,   front_kernel<true, true, true>};
-    const int which = (single ? 1 : 0) + (list ? 2 : 0) + (strands ? 4 : 0);
+    constexpr Bases P = Bases::Packed, S = Bases::PackedStrands, A = Bases::Ascii;
+    static const Kernel kernels[10] = {front_kernel<false, false, P>, front_kernel<true, false, P>,
+                                       front_kernel<false, false, S>, front_kernel<true, false, S>,
+                                       front_kernel<false, true, P>,  front_kernel<true, true, P>,
+                                       front_kernel<false, true, S>,  front_kernel<true, true, S>,
+                                       front_kernel<false, true, A>,  front_kernel<true, true, A>};
+    const int which = (single ? 1 : 0) + (list ? 4 : 0) + 2 * (L.fused ? 2 : (L.revcomp || L.strand_bits ? 1 : 0));
     const Kernel kernel = kernels[which];
     int &bps = per_sm[which][dev];
     if (bps == 0) {

@@ -14,9 +14,7 @@ __global__ void pack_text_kernel(const uint8_t *__restrict__ ascii, uint64_t n, 
         if (b0 + 32 <= n && aligned16) {
             const uint4 v0 = __ldg(reinterpret_cast<const uint4 *>(ascii + b0));
             const uint4 v1 = __ldg(reinterpret_cast<const uint4 *>(ascii + b0 + 16));
-            const uint32_t v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-            for (int k = 0; k < 8; k++) word = (word << 8) | pack4_fast(v[k], &bad);
+            word = pack32(v0, v1, &bad);
         } else {
             for (int j = 0; j < 32; j++) {
                 const uint64_t b = b0 + j;
@@ -79,10 +77,7 @@ __global__ void pack_batch_kernel(const uint8_t *__restrict__ ascii, uint64_t to
         if (aligned16 && b0 + 32 <= total) {
             const uint4 v0 = __ldg(reinterpret_cast<const uint4 *>(ascii + b0));
             const uint4 v1 = __ldg(reinterpret_cast<const uint4 *>(ascii + b0 + 16));
-            const uint32_t v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-            word = 0;
-#pragma unroll
-            for (int k = 0; k < 8; k++) word = (word << 8) | pack4_fast(v[k], &bad);
+            word = pack32(v0, v1, &bad);
         } else {
             const uint64_t left = total - b0;
             word = pack_word(ascii, total, b0, left < 32 ? (uint32_t)left : 32u, &bad);

@@ -128,6 +128,33 @@ __device__ __forceinline__ uint32_t pack4_fast(uint32_t v, uint32_t *bad) {
     return (c * 0x40100401u) >> 24;
 }
 
+// A 32-base word from its 32 bytes; *bad becomes non-zero if one of them is not
+// a base.  Bits 2-1 of a letter are A 00, C 01, G 11, T 10: four of them are
+// put together by one multiply, and one x ^ (x >> 1) per word makes the codes.
+// Of a base's other bits (case folded) 7 and 3 are clear, 6 is set, 4 is set
+// exactly where bits 2-1 are 10 (T), and 0 is the opposite of 4; those are
+// collected over the 32 bytes and looked at once.  The kernels that pack are
+// bound by the integer pipe, so what can be a left shift is one (a multiply,
+// on the other pipe): about 55 logic instructions per word, where pack4_fast
+// on each four bytes takes 120.
+__device__ __forceinline__ uint64_t pack32(uint4 v0, uint4 v1, uint32_t *bad) {
+    const uint32_t v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+    uint32_t p[8], wrong = 0, any = 0, all = 0xFFFFFFFFu;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const uint32_t t = v[k] & ~(v[k] * 2u) & 0x04040404u;       // bit 2 of each byte: bits 2-1 are 10
+        wrong |= (v[k] ^ (t * 4u)) | ~(v[k] ^ (v[k] * 16u));         // at bit 4
+        any |= v[k];
+        all &= v[k];
+        p[k] = ((v[k] >> 1) & 0x03030303u) * 0x40100401u;           // the four pairs in its top byte
+    }
+    *bad |= (wrong & 0x10101010u) | (any & 0x88888888u) | (~all & 0x40404040u);
+    const uint32_t hi = __byte_perm(__byte_perm(p[3], p[2], 0x0073), __byte_perm(p[1], p[0], 0x0073), 0x5410);
+    const uint32_t lo = __byte_perm(__byte_perm(p[7], p[6], 0x0073), __byte_perm(p[5], p[4], 0x0073), 0x5410);
+    const uint64_t x = ((uint64_t)hi << 32) | lo;
+    return x ^ ((x >> 1) & 0x5555555555555555ull);
+}
+
 // Packs the 32 ASCII bases starting at byte s of a (the first nb <= 32 belong
 // to the query; the rest pack as A).  When nine aligned 32-bit words around
 // them lie inside [a, a + total) they are read and aligned with funnel
@@ -518,45 +545,58 @@ struct Bounds {
     __device__ __forceinline__ uint32_t first() const { return phase == 0 ? R : lo; }
 };
 
-// Query P (length m >= 1, at place qa of the packed batch tq) against
-// the suffix at p of a text of n < 2^32 bases, from the 32-aligned base below
-// `start` (< m; all bases before it are known equal).
-template <bool kStrands>
-__device__ __forceinline__ int cmp_suffix_tq(const uint64_t *__restrict__ T, uint32_t n, uint32_t p,
-                                             const uint64_t *__restrict__ tq, uint64_t qa, uint32_t m,
-                                             uint32_t start, uint32_t *lcp) {
-    uint32_t off = start & ~31u;
-    const uint32_t rem = n - p;
-    for (;;) {
-        const uint32_t qlen = min(32u, m - off);
-        const uint32_t tlen = off < rem ? min(32u, rem - off) : 0u;
-        const uint64_t q = query_window<kStrands>(tq, qa, off);
-        const uint64_t t = tlen ? text_window(T, (uint64_t)(p + off)) : 0ull;
-        const int c = cmp_window(q, t, qlen, tlen, off, m, lcp);
-        if (c != 2) return c;
-        off += 32u;
-    }
-}
+// Where a kernel reads a query's bases beyond those its records carry: the
+// packed batch (forward queries only, or of either strand), or the batch's
+// ASCII bytes, of either strand (a batch whose kernels pack what they need
+// themselves; api.cu: fused_packing).
+enum class Bases { Packed, PackedStrands, Ascii };
 
-// The query's 32-base window at base `off` (a multiple of 32, off >= 96): base
-// 96 from w3 (the query's fourth packed word), bases 128 .. 128 + 32
-// tail_words - 1 from `tail` (later words its record carries, read again from
-// the record when a compare gets there), the rest from the packed batch.
-template <bool kStrands>
-struct QueryWindows {
-    const uint64_t *tq;
+// A query's 32-base window at base off (a multiple of 32 below m).
+struct AsciiWindows {  // bytes [qa, qa + m) of the batch, or their reverse complement
+    const uint8_t *ascii;
+    uint64_t total;
     uint64_t qa;
+    uint32_t m;
+    bool rc;
+    __device__ __forceinline__ uint64_t packed(uint32_t off, uint32_t *bad) const {
+        const uint32_t nb = m - off < 32u ? m - off : 32u;
+        if (!rc) return pack_word(ascii, total, qa + off, nb, bad);
+        // the nb bytes that end off bases before the query's end
+        return rc_window(pack_word(ascii, total, qa + (m - off - nb), nb, bad)) << (64u - 2u * nb);
+    }
+    __device__ __forceinline__ uint64_t operator()(uint32_t off) const {
+        uint32_t bad = 0;
+        return packed(off, &bad);
+    }
+};
+
+template <bool kStrands>
+struct PackedWindows {  // the query at place `at` of the packed batch
+    const uint64_t *tq;
+    uint64_t at;
+    __device__ __forceinline__ uint64_t operator()(uint32_t off) const { return query_window<kStrands>(tq, at, off); }
+};
+
+// A query's windows from its record where that has them (off >= 96): base 96
+// from w3 (its fourth packed word), bases 128 .. 128 + 32 tail_words - 1 from
+// `tail` (later words its record carries, read again from the record when a
+// compare gets there), the rest from src.
+template <typename Source>
+struct RecordWindows {
+    Source src;
     uint64_t w3;
     const uint64_t *tail;
     uint32_t tail_words;
     __device__ __forceinline__ uint64_t operator()(uint32_t off) const {
         if (off == 96u) return w3;
         if (off >= 128u && ((off - 128u) >> 5) < tail_words) return __ldg(tail + ((off - 128u) >> 5));
-        return query_window<kStrands>(tq, qa, off);
+        return src(off);
     }
 };
 
-// cmp_suffix_tq with the query's windows from qw (start >= 96).
+// Query P (length m >= 1, its windows from qw) against the suffix at p of a
+// text of n < 2^32 bases, from the 32-aligned base below `start` (< m; all
+// bases before it known equal).
 template <typename Windows>
 __device__ __forceinline__ int cmp_suffix_qw(const uint64_t *__restrict__ T, uint32_t n, uint32_t p,
                                              const Windows &qw, uint32_t m, uint32_t start, uint32_t *lcp) {
@@ -666,12 +706,14 @@ struct SearchLaunch {
     uint32_t smem_bytes;      // shared-memory key tables
     uint32_t threads, blocks, chunk;
     uint32_t front_probes;    // probes per query in the first pass
+    bool fused;               // k-mer order: no packed batch, the scatter packs what it needs (tq, tvb, tv,
+                              // batch_dirty are not used)
     bool revcomp;             // search every query's reverse complement
     bool strand_bits;         // q_ref bit 31 selects each query's strand
     bool expire_waits;        // test hook: the bounded key-table wait gives up at once
     uint32_t trunc_cap;       // the locate cap of sa_search_locate (SA_RESULT_TRUNCATED), else ~0u
     // k-mer order (bucket.cu)
-    uint64_t ktotal;          // k-mer entries of all indexes of the call
+    uint64_t kscale;          // floor((2^64 - 1) / k-mer entries of all indexes of the call)
     uint32_t *bplan;          // the list's plan, kPlanWords words (see below; zeroed by the caller)
     // search + locate in one call: per 2^kLocateTileShift queries, the sum of
     // min(count, trunc_cap) of their results (zeroed by the caller), or null

@@ -26,7 +26,7 @@
 //   compared one at a time against the text.
 #include <type_traits>
 
-#include "sa_internal.cuh"
+#include "first_pass.cuh"
 
 namespace sa {
 
@@ -158,7 +158,7 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s for the key-table copy
 // chunk's base fetched while the previous chunk is handed out.
 // Launch bounds: 1024 threads, one CTA per SM, at most 64 registers (no
 // spills); smaller CTAs may share an SM up to 1024 threads in all.
-template <typename IdxT, bool kSingle, bool kStrands>
+template <typename IdxT, bool kSingle, Bases kBases>
 __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__ SearchLaunch a) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ SmemDesc sdesc[SA_MAX_REFS];
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             const uint32_t klen = Ktab[(16u << depth) + k];
             bool und = false;
             c = cmp_key(q0, q1, m, kv, klen, &l, &und);
-            if (und) c = cmp_suffix_tq<kStrands>(T, n, (uint32_t)sa_at<IdxT>(SAp, M), a.tq, qa, m, 64u, &l);
+            if (und) c = cmp_suffix_qw(T, n, (uint32_t)sa_at<IdxT>(SAp, M), window_source<kBases>(a, qa, m), m, 64u, &l);
             const uint32_t nk = 2u * k + (c == CMP_GREATER ? 1u : 0u);
             k = (c == CMP_PREFIX || nk >= (1u << depth)) ? 0u : nk;
         } else {
@@ -303,7 +303,8 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             c = cmp_record(qw4, m, r0, r1, n, &l, &und);
             if (und) {
                 // query bases 96-127 are x3, 128-159 the worklist record's second word pair
-                const QueryWindows<kStrands> qw{a.tq, qa, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};
+                const auto src = window_source<kBases>(a, qa, m);
+                const RecordWindows<decltype(src)> qw{src, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};
                 c = cmp_suffix_qw(T, n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
             }
             lp = (r1.z >> 8) & 0xFFu;
@@ -441,10 +442,12 @@ cudaError_t launch_search(const SearchLaunch &L, cudaStream_t s) {
     auto pick = [&](auto idx_tag, auto single_tag) {
         using I = decltype(idx_tag);
         constexpr bool S = decltype(single_tag)::value;
-        if (L.revcomp || L.strand_bits)
-            go(search_kernel<I, S, true>);
+        if (L.fused)
+            go(search_kernel<I, S, Bases::Ascii>);
+        else if (L.revcomp || L.strand_bits)
+            go(search_kernel<I, S, Bases::PackedStrands>);
         else
-            go(search_kernel<I, S, false>);
+            go(search_kernel<I, S, Bases::Packed>);
     };
     if (L.width == 4)
         single ? pick(uint32_t{}, std::true_type{}) : pick(uint32_t{}, std::false_type{});

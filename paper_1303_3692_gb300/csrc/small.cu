@@ -31,26 +31,6 @@ constexpr int kSmallThreads = 128;
 constexpr int kSmallPerSm = 8;  // CTAs
 constexpr uint32_t kLaneProbes = 2;
 
-// A query's windows packed from its ASCII bases: bytes [qa, qa + m) of the
-// batch, or their reverse complement.
-struct AsciiWindows {
-    const uint8_t *ascii;
-    uint64_t total;
-    uint64_t qa;
-    uint32_t m;
-    bool rc;
-    __device__ __forceinline__ uint64_t packed(uint32_t off, uint32_t *bad) const {  // off < m
-        const uint32_t nb = m - off < 32u ? m - off : 32u;
-        if (!rc) return pack_word(ascii, total, qa + off, nb, bad);
-        // the nb bytes that end off bases before the query's end
-        return rc_window(pack_word(ascii, total, qa + (m - off - nb), nb, bad)) << (64u - 2u * nb);
-    }
-    __device__ __forceinline__ uint64_t operator()(uint32_t off) const {
-        uint32_t bad = 0;
-        return packed(off, &bad);
-    }
-};
-
 __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
     return __shfl_sync(0xFFFFFFFFu, (unsigned long long)v, src);
 }
