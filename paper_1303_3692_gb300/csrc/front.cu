@@ -219,6 +219,12 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         // Further probes, one suffix record each; queries without a k-mer
         // bracket go straight to the worklist (the persistent kernel descends
         // the shared-memory key table first).
+        // A compare that ties on all a record holds goes on in the text.  In
+        // k-mer order (several probes) it waits for the end of the probes, so
+        // that the warp reads the text once for all its lanes that do, not once
+        // per probe: 3.1 Gbp, 4*10^7 x 150 bases 2.82 -> 2.71 ms.
+        bool pending = false;
+        uint32_t pend_pos = 0, pend_lcps = 0;
         for (uint32_t p = 1; p < a.front_probes && __any_sync(0xFFFFFFFFu, go); p++) {
             const uint32_t M = bd.pivot();
             uint4 r0, r1;
@@ -227,10 +233,22 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
                 uint32_t l;
                 bool und = false;
                 int c = cmp_record(w, m, r0, r1, d.n, &l, &und);
-                if (und)
+                if (!kFromList && und)
                     c = cmp_suffix_qw(d.text, d.n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
-                step(c, M, l, (r1.z >> 8) & 0xFFu, r1.z & 0xFFu);
+                if (kFromList && und) {
+                    pending = true;
+                    pend_pos = r1.w;
+                    pend_lcps = r1.z & 0xFFFFu;
+                    go = false;
+                } else {
+                    step(c, M, l, (r1.z >> 8) & 0xFFu, r1.z & 0xFFu);
+                }
             }
+        }
+        if (kFromList && pending) {
+            uint32_t l;
+            const int c = cmp_suffix_pairs(d.text, d.n, pend_pos, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
+            step(c, bd.pivot(), l, pend_lcps >> 8, pend_lcps & 0xFFu);
         }
 
         if (live && done) store_result_sum(a, q, lo, hi);

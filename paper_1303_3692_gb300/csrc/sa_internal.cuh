@@ -613,6 +613,36 @@ __device__ __forceinline__ int cmp_suffix_qw(const uint64_t *__restrict__ T, uin
     }
 }
 
+// The same with two windows a step, whose reads wait for each other's neither
+// in the text nor in the query: for kernels with the registers for it (in the
+// first pass of input order and in small.cu it spills or costs warps: 10^7
+// reads 353 -> 373 us, 20,011 reads 29 -> 33 us).
+template <typename Windows>
+__device__ __forceinline__ int cmp_suffix_pairs(const uint64_t *__restrict__ T, uint32_t n, uint32_t p,
+                                             const Windows &qw, uint32_t m, uint32_t start, uint32_t *lcp) {
+    uint32_t off = start & ~31u;
+    const uint32_t rem = n - p, sh = 2u * (p & 31u);
+    for (;;) {
+        const bool two = off + 32u < m;
+        const uint64_t *at = T + ((p + off) >> 5);  // (off is a multiple of 32: the shift stays)
+        const uint64_t q0 = qw(off), q1 = two ? qw(off + 32u) : 0ull;
+        uint64_t t0 = 0, t1 = 0, t2 = 0;
+        if (off < rem) {
+            t0 = ldg_u64(at);
+            t1 = ldg_u64(at + 1);
+            if (two && off + 32u < rem) t2 = ldg_u64(at + 2);
+        }
+        int c = cmp_window(q0, (t0 << sh) | ((t1 >> 1) >> (63u - sh)), min(32u, m - off),
+                           off < rem ? min(32u, rem - off) : 0u, off, m, lcp);
+        if (c != 2) return c;
+        off += 32u;
+        c = cmp_window(q1, (t1 << sh) | ((t2 >> 1) >> (63u - sh)), min(32u, m - off),
+                       off < rem ? min(32u, rem - off) : 0u, off, m, lcp);
+        if (c != 2) return c;
+        off += 32u;
+    }
+}
+
 }  // namespace sa
 
 // ---------------------------------------------------------------------------

@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
                 // query bases 96-127 are x3, 128-159 the worklist record's second word pair
                 const auto src = window_source<kBases>(a, qa, m);
                 const RecordWindows<decltype(src)> qw{src, x3, reinterpret_cast<const uint64_t *>(wrec) + 3, 1u};
-                c = cmp_suffix_qw(T, n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
+                c = cmp_suffix_pairs(T, n, r1.w, qw, m, max(kRecBases, min(bd.lcpL, bd.lcpR)), &l);
             }
             lp = (r1.z >> 8) & 0xFFu;
             ln = r1.z & 0xFFu;
