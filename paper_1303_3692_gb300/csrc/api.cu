@@ -326,6 +326,7 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
         L.strand_bits = strand_bits;
         L.trunc_cap = trunc_cap;
         L.tile_kept = tile_kept;
+        L.tile_shift = locate_tile_shift(n_q);
         L.tile_sum_by_warp = true;
         return search_timed(params, s, [&] { return launch_search_small(L, s); });
     }
@@ -395,6 +396,7 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.expire_waits = params && (params->flags & SA_PARAM_EXPIRE_WAITS);
     L.trunc_cap = trunc_cap;
     L.tile_kept = tile_kept;
+    L.tile_shift = locate_tile_shift(n_q);
     L.tile_sum_by_warp = !kmer_order;
     L.kscale = ktotal ? ~0ull / ktotal : 0;
     L.bplan = bplan;
@@ -763,7 +765,7 @@ int locate_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
                   uint64_t capacity, const uint64_t *base_in, int *overflow, cudaStream_t s, Scratch &sc,
                   uint64_t *presummed = nullptr) {
     // presummed: the tile sums, already added up by the search kernels
-    uint64_t *partials = presummed ? presummed : sc.get<uint64_t>(locate_tiles(n_q) + 1);
+    uint64_t *partials = presummed ? presummed : sc.get<uint64_t>(locate_tiles(n_q, locate_tile_shift(n_q)) + 1);
     if (sc.failed) return SA_ERR_NOMEM;
     LocateLaunch L;
     memset(&L, 0, sizeof L);
@@ -778,6 +780,7 @@ int locate_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.out_pos = pos_d;
     L.capacity = pos_d ? capacity : 0;
     L.partials = partials;
+    L.tile_shift = locate_tile_shift(n_q);
     L.presummed = presummed != nullptr;
     L.overflow = overflow;
     L.base_in = base_in;
@@ -1050,9 +1053,10 @@ int sa_search_locate(const sa_index *const *refs, uint32_t n_refs, const char *q
     // each result (so the locate need not read every result for them)
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Scratch sc{s};
-    uint64_t *tile_kept = sc.get<uint64_t>(locate_tiles(n_q) + 1);
+    const size_t sums = locate_tiles(n_q, locate_tile_shift(n_q)) + 1;
+    uint64_t *tile_kept = sc.get<uint64_t>(sums);
     if (sc.failed) return SA_ERR_NOMEM;
-    cudaError_t err = cudaMemsetAsync(tile_kept, 0, (locate_tiles(n_q) + 1) * sizeof(uint64_t), s);
+    cudaError_t err = cudaMemsetAsync(tile_kept, 0, sums * sizeof(uint64_t), s);
     if (err != cudaSuccess) return status_from_cuda(err);
     const int st = search_impl(refs, n_refs, q_bases, q_offsets, q_ref, n_q, out, stream, params, false, cap,
                                tile_kept);
@@ -1081,7 +1085,7 @@ int sa_locate_noalloc(const sa_index *const *refs, uint32_t n_refs, const uint32
     uint64_t *partials = nullptr, entries = 0;
     cudaError_t err = locate_static_partials(&partials, &entries);
     if (err != cudaSuccess) return status_from_cuda(err);
-    if (locate_tiles(n_q) + 1 > entries) return SA_ERR_CAPACITY;
+    if (locate_tiles(n_q, kLocateTileShift) + 1 > entries) return SA_ERR_CAPACITY;
     LocateLaunch L;
     memset(&L, 0, sizeof L);
     fill_ref_table(refs, n_refs, 0, &L.refs);
@@ -1095,6 +1099,7 @@ int sa_locate_noalloc(const sa_index *const *refs, uint32_t n_refs, const uint32
     L.out_pos = out_pos;
     L.capacity = out_pos ? out_pos_capacity : 0;
     L.partials = partials;
+    L.tile_shift = kLocateTileShift;
     return status_from_cuda(launch_locate(L, reinterpret_cast<cudaStream_t>(stream)));
 }
 

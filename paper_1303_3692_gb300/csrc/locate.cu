@@ -3,10 +3,11 @@
 // entries SA[lo_q], SA[lo_q + 1], ... are copied to out_pos[out_offsets[q]..].
 // (The paper reports only [LB, RB]; locate is an extension of it.)
 //
-// Three launches: per-tile sums of k_q, one CTA scanning the tile sums, and a
-// CTA per tile that scans its own k_q, writes the offsets and gathers.  Each
-// tile is kTileThreads x kItems consecutive queries; thread t of a tile owns
-// queries t, t + kTileThreads, t + 2 kTileThreads, ... of it.
+// Up to three launches: per-tile sums of k_q, one CTA scanning the tile sums
+// (large batches), and a CTA per tile that scans its own k_q, writes the
+// offsets and gathers.  Each tile is kTileThreads x kItems consecutive
+// queries; thread t of a tile owns queries t, t + kTileThreads, t + 2
+// kTileThreads, ... of it.
 #include <mutex>
 
 #include "sa_internal.cuh"
@@ -22,12 +23,10 @@ namespace sa {
 namespace {
 
 constexpr int kTileThreads = 512;
-constexpr int kItems = 8;
-constexpr uint64_t kTile = (uint64_t)kTileThreads * kItems;
-// Up to this many tiles (2^21 queries) each tile of the gather adds up the
-// sums of those before it itself, one thread per tile, and the scan's launch
-// is saved; beyond, a scan puts them in place first.
-constexpr uint64_t kDirectTiles = kTileThreads;
+// Up to this many tiles each tile of the gather adds up the sums of those
+// before it itself, and the scan's launch is saved; beyond, a scan puts them
+// in place first.
+constexpr uint64_t kDirectTiles = 2048;
 
 __device__ __forceinline__ uint64_t kept(const sa_result &r, uint32_t cap) {
     if (r.count == ~0ull) return 0;  // invalid query (reported as all-ones)
@@ -63,9 +62,10 @@ __device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t *t
     return before + x - v;
 }
 
+template <int kItems>
 __global__ void __launch_bounds__(kTileThreads) tile_sums_kernel(const sa_result *__restrict__ res, uint64_t n_q,
                                                                   uint32_t cap, uint64_t *partials) {
-    const uint64_t base = (uint64_t)blockIdx.x * kTile;
+    const uint64_t base = (uint64_t)blockIdx.x * (kTileThreads * kItems);
     uint64_t s = 0;
 #pragma unroll
     for (int i = 0; i < kItems; i++) {
@@ -98,15 +98,54 @@ __global__ void __launch_bounds__(1024) scan_partials_kernel(uint64_t *partials,
     if (threadIdx.x == 0) partials[ntiles] = carry_s;
 }
 
-// One CTA per tile of kTile queries; warp w owns the tile's queries
-// [w * 256, w * 256 + 256), lane l its queries w * 256 + i * 32 + l for
-// i < kItems, so every load of results and store of offsets is coalesced.  A
+// Copies the positions of a warp's 32 queries, lane l's being SA[lo .. lo + k)
+// of its reference, to pos[first ..) one run after the other (l's run starts
+// `before` entries in; total: all runs; a run with !within is left out).  The
+// lanes take the output entry by entry, 32 in a row, and each finds the run its
+// entry is in (five shuffles), so the stores are whole lines and a query with
+// many positions keeps all lanes busy instead of its own.
+template <typename IdxT>
+__device__ __forceinline__ void copy_runs(const LocateLaunch &a, IdxT *pos, uint64_t first, uint64_t before,
+                                          uint64_t total, uint32_t k, uint64_t lo, uint32_t ref, bool within) {
+    const unsigned lane = threadIdx.x & 31u;
+    const IdxT *sa = reinterpret_cast<const IdxT *>(a.refs.r[ref].sa) + lo;
+    if (total > 0xFFFFFFFFull - 32) {  // enormous caps: run by run
+        for (int j = 0; j < 32; j++) {
+            const bool in = __shfl_sync(0xFFFFFFFFu, (int)within, j) != 0;
+            const uint32_t kj = __shfl_sync(0xFFFFFFFFu, k, j);
+            const uint64_t at = first + __shfl_sync(0xFFFFFFFFu, (unsigned long long)before, j);
+            const IdxT *from = reinterpret_cast<const IdxT *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)sa, j));
+            if (!in) continue;
+            for (uint64_t t = lane; t < kj; t += 32)
+                if (at + t < a.capacity) pos[at + t] = __ldg(from + t);
+        }
+        return;
+    }
+    const uint32_t mine = (uint32_t)before;
+    const unsigned ok = __ballot_sync(0xFFFFFFFFu, within);
+    for (uint32_t t = 0; t < (uint32_t)total; t += 32u) {
+        const uint32_t p = t + lane;
+        // the last lane whose run starts at or before p
+        int j = 0;
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            const uint32_t start = __shfl_sync(0xFFFFFFFFu, mine, j + s);
+            if (start <= p) j += s;
+        }
+        const uint32_t start = __shfl_sync(0xFFFFFFFFu, mine, j);
+        const IdxT *from = reinterpret_cast<const IdxT *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)sa, j));
+        if (p < (uint32_t)total && ((ok >> j) & 1u) && first + p < a.capacity) pos[first + p] = __ldg(from + (p - start));
+    }
+}
+
+// One CTA per tile; warp w owns the tile's 32 kItems queries from w * 32 kItems
+// on, lane l those at i * 32 + l of them for i < kItems, so every load of results and store of offsets is coalesced.  A
 // first pass reads the lane's results once and sums its items, keeping each
 // item's count and lower bound in shared memory; one exchange of warp totals
 // (one barrier) places the warps within the tile; a second pass places each
 // item within the warp's run by a warp scan (shuffles), writes its offset and
 // copies its positions.
-template <typename IdxT>
+template <typename IdxT, int kItems>
 __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __grid_constant__ LocateLaunch a) {
     constexpr int kWarps = kTileThreads / 32;
     __shared__ uint64_t s_warp[kWarps], s_before[kWarps];
@@ -115,7 +154,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __gr
     // longer holds them by then
     __shared__ uint32_t s_k[kItems][kTileThreads];
     __shared__ uint32_t s_lo[kItems][kTileThreads];
-    const uint64_t tile_base = (uint64_t)blockIdx.x * kTile;
+    const uint64_t tile_base = (uint64_t)blockIdx.x * (kTileThreads * kItems);
     const uint64_t ntiles = gridDim.x;
     const bool direct = ntiles <= kDirectTiles;  // the partials are the tile sums themselves
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -140,8 +179,9 @@ __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __gr
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xFFFFFFFFu, tot, o);
     if (lane == 0) s_warp[warp] = tot;
-    if (direct) {  // the tiles before this one, a thread each
-        uint64_t before = threadIdx.x < blockIdx.x ? a.partials[threadIdx.x] : 0;
+    if (direct) {  // the tiles before this one
+        uint64_t before = 0;
+        for (unsigned i = threadIdx.x; i < blockIdx.x; i += kTileThreads) before += a.partials[i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
         if (lane == 0) s_before[warp] = before;
@@ -155,7 +195,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __gr
     if (blockIdx.x == ntiles - 1 && threadIdx.x == kTileThreads - 1) a.out_offsets[a.n_q] = run + tot;
 
     // Second pass over the items, from shared memory.
-#pragma unroll
+#pragma unroll 1
     for (int i = 0; i < kItems; i++) {
         const uint64_t q = warp_base + (uint64_t)i * 32 + lane;
         const uint32_t k = s_k[i][threadIdx.x];
@@ -166,28 +206,28 @@ __global__ void __launch_bounds__(kTileThreads, 3) tile_gather_kernel(const __gr
             const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
             if (lane >= (unsigned)o) x += y;
         }
+        const uint64_t first = run;  // the offset of the item's first query
         const uint64_t off = run + x - k;
-        run += __shfl_sync(0xFFFFFFFFu, x, 31);
-        if (q >= a.n_q) continue;
-        a.out_offsets[q] = off;
-        if (pos == nullptr || k == 0) continue;
-        const uint32_t ref = a.q_ref ? (a.q_ref[q] & ~kStrandBit) : 0u;  // bit 31: the strand, not the reference
-        const RefDesc &d = a.refs.r[ref < a.n_refs ? ref : 0];
-        const uint64_t kk = (ref < a.n_refs && lo <= d.n && k <= d.n - lo) ? k : 0;  // never past SA
-        const IdxT *sa = reinterpret_cast<const IdxT *>(d.sa);
-        for (uint64_t t = 0; t < kk; t++) {
-            if (off + t < a.capacity) pos[off + t] = __ldg(sa + lo + t);
-        }
-        if (a.overflow != nullptr && off + kk > a.capacity) atomicOr(a.overflow, 1);
+        const uint64_t total = __shfl_sync(0xFFFFFFFFu, x, 31);
+        run += total;
+        if (q < a.n_q) a.out_offsets[q] = off;
+        if (pos == nullptr || total == 0) continue;
+        const uint32_t q_ref = a.q_ref && q < a.n_q ? (a.q_ref[q] & ~kStrandBit) : 0u;  // bit 31: the strand
+        const uint32_t ref = q_ref < a.n_refs ? q_ref : 0u;
+        const uint64_t n = a.refs.r[ref].n;
+        const bool within = q_ref < a.n_refs && lo <= n && k <= n - lo;  // never past SA
+        copy_runs<IdxT>(a, pos, first, (uint64_t)(x - k), total, k, lo, ref, within);
+        if (a.overflow != nullptr && k != 0 && off + (within ? k : 0) > a.capacity) atomicOr(a.overflow, 1);
     }
 }
 
 }  // namespace
 
-uint64_t locate_tiles(uint64_t n_q) { return (n_q + kTile - 1) / kTile; }
+uint64_t locate_tiles(uint64_t n_q, uint32_t shift) { return (n_q + (1ull << shift) - 1) >> shift; }
 
-static_assert(kTile == 4096, "the static scratch below is sized for 4096-query tiles");
-static_assert(kTile == (1ull << kLocateTileShift), "the search kernels sum kept counts per locate tile");
+static_assert((1u << kLocateTileShift) == kTileThreads * 8 && (1u << kLocateSmallTileShift) == kTileThreads * 2,
+              "the tiles of the kernels' two forms");
+static_assert(kLocateTileShift == 12, "the static scratch below is sized for 4096-query tiles");
 
 cudaError_t locate_static_partials(uint64_t **ptr, uint64_t *entries) {
     static std::mutex mu;
@@ -221,16 +261,25 @@ cudaError_t locate_static_partials(uint64_t **ptr, uint64_t *entries) {
 
 
 cudaError_t launch_locate(const LocateLaunch &L, cudaStream_t s) {
-    const uint64_t tiles = locate_tiles(L.n_q);
+    const uint64_t tiles = locate_tiles(L.n_q, L.tile_shift);
     if (tiles == 0) {
         return cudaMemsetAsync(L.out_offsets, 0, sizeof(uint64_t), s);
     }
-    if (!L.presummed) tile_sums_kernel<<<(unsigned)tiles, kTileThreads, 0, s>>>(L.res, L.n_q, L.cap, L.partials);
+    const unsigned grid = (unsigned)tiles;
+    const bool small = L.tile_shift == kLocateSmallTileShift;
+    if (!L.presummed) {
+        if (small)
+            tile_sums_kernel<2><<<grid, kTileThreads, 0, s>>>(L.res, L.n_q, L.cap, L.partials);
+        else
+            tile_sums_kernel<8><<<grid, kTileThreads, 0, s>>>(L.res, L.n_q, L.cap, L.partials);
+    }
     if (tiles > kDirectTiles) scan_partials_kernel<<<1, 1024, 0, s>>>(L.partials, tiles, L.base_in);
     if (L.width == 4)
-        tile_gather_kernel<uint32_t><<<(unsigned)tiles, kTileThreads, 0, s>>>(L);
+        small ? tile_gather_kernel<uint32_t, 2><<<grid, kTileThreads, 0, s>>>(L)
+              : tile_gather_kernel<uint32_t, 8><<<grid, kTileThreads, 0, s>>>(L);
     else
-        tile_gather_kernel<uint64_t><<<(unsigned)tiles, kTileThreads, 0, s>>>(L);
+        small ? tile_gather_kernel<uint64_t, 2><<<grid, kTileThreads, 0, s>>>(L)
+              : tile_gather_kernel<uint64_t, 8><<<grid, kTileThreads, 0, s>>>(L);
     return cudaGetLastError();
 }
 

@@ -745,14 +745,20 @@ struct SearchLaunch {
     // k-mer order (bucket.cu)
     uint64_t kscale;          // floor((2^64 - 1) / k-mer entries of all indexes of the call)
     uint32_t *bplan;          // the list's plan, kPlanWords words (see below; zeroed by the caller)
-    // search + locate in one call: per 2^kLocateTileShift queries, the sum of
+    // search + locate in one call: per 2^tile_shift queries, the sum of
     // min(count, trunc_cap) of their results (zeroed by the caller), or null
     uint64_t *tile_kept;
+    uint32_t tile_shift;
     bool tile_sum_by_warp;    // input order: the lanes storing together mostly share a tile
 };
 
-// Queries per tile of the locate's scan (locate.cu).
-constexpr uint32_t kLocateTileShift = 12;
+// Queries per tile of the locate's scan (locate.cu): 4096, and 1024 for batches
+// of up to 2^21 queries, whose 4096-query tiles would fill the GPU's 456
+// resident CTAs a little more than once (2*10^6 queries: 489) or not at all.
+constexpr uint32_t kLocateTileShift = 12, kLocateSmallTileShift = 10;
+inline uint32_t locate_tile_shift(uint64_t n_q) {
+    return n_q <= (1ull << 21) ? kLocateSmallTileShift : kLocateTileShift;
+}
 
 // store_result for the search kernels; in a search + locate call it also
 // adds the query's kept count min(count, cap) to its locate tile's sum, so
@@ -765,7 +771,7 @@ __device__ __forceinline__ void store_result_sum(const SearchLaunch &a, uint64_t
     if (a.tile_kept == nullptr) return;
     const uint64_t c = lo == ~0ull ? 0ull : hi - lo;
     const uint32_t k = c < (uint64_t)a.trunc_cap ? (uint32_t)c : a.trunc_cap;
-    const uint64_t tile = q >> kLocateTileShift;
+    const uint64_t tile = q >> a.tile_shift;
     unsigned long long *sum_at = reinterpret_cast<unsigned long long *>(a.tile_kept) + tile;
     if (a.tile_sum_by_warp) {
         const unsigned same = __match_any_sync(__activemask(), tile);
@@ -818,11 +824,12 @@ struct LocateLaunch {
     void *out_pos;
     uint64_t capacity;
     uint64_t *partials;       // scratch: one entry per scan tile + 1
+    uint32_t tile_shift;      // kLocateTileShift or kLocateSmallTileShift
     bool presummed;           // partials already hold the tile sums (from the search kernels)
     int *overflow;            // optional device flag: a position fell at or beyond capacity
     const uint64_t *base_in;  // optional device value added to every offset (a chunk of a larger batch)
 };
-uint64_t locate_tiles(uint64_t n_q);
+uint64_t locate_tiles(uint64_t n_q, uint32_t shift);
 // Device address of the static scratch of sa_locate_noalloc on the current
 // device (looked up once per device) and the number of partial sums it holds.
 cudaError_t locate_static_partials(uint64_t **ptr, uint64_t *entries);
