@@ -1,5 +1,6 @@
 // api.cu -- the extern "C" entry points declared in include/sa.h: argument
 // checks, host/device staging, scratch memory and the index life cycle.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -874,10 +875,16 @@ int search_pipelined(const sa_index *const *refs, uint32_t n_refs, uint32_t widt
                      const uint64_t *q_offsets, const uint32_t *q_ref, uint64_t n_q, sa_result *out,
                      cudaStream_t s, const sa_search_params *params, bool locate, uint32_t cap,
                      uint64_t *out_offsets, void *out_pos, uint64_t capacity) {
-    // Chunks of about n_q / 12 queries (at least 2^20); the last such chunk's
+    // Chunks of about n_q / 12 queries, at least 2^20 of them, or n_q / 6 when
+    // that is less, at least 2^19: what is uploaded before the first kernel and
+    // what is left after the last upload are a chunk's, while more and smaller
+    // chunks cost the copies of both directions that run at the same time
+    // (reads of 100 bases, us a call: 3*10^6 queries in chunks of 2^18, 2^19,
+    // 2^20: 2200, 2086, 2264; 9*10^6: 5880, 5855, 5580).  The last such chunk's
     // queries go in four quarter chunks, so that less work is left after the
     // final upload.
-    const uint64_t per = (n_q + 11) / 12 > (1ull << 20) ? (n_q + 11) / 12 : (1ull << 20);
+    const uint64_t sixth = std::min<uint64_t>(std::max<uint64_t>((n_q + 5) / 6, 1ull << 19), 1ull << 20);
+    const uint64_t per = std::max<uint64_t>((n_q + 11) / 12, sixth);
     std::vector<uint64_t> cut;  // chunk c is [cut[c], cut[c + 1])
     try {
         cut.push_back(0);
