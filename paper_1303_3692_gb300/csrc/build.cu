@@ -91,9 +91,10 @@ __device__ __forceinline__ int order_beyond(const uint64_t *__restrict__ T, uint
 // heads.  A member's first window beyond depth is read once, into shared
 // memory, where the others find it; only members equal there are compared in
 // the text, over at most kRefineWindows windows per item in all.  Bound by
-// those random reads: 2.0 ms for 10^8 human-like bases, of whose suffixes the
-// first sort leaves about a third in groups, 20 ms for 6*10^8 (the text past
-// L2).  Sorting by 64-bit keys of 29 bases instead, eight passes of 24 bytes,
+// those random reads and its members' compares: 1.4 ms for 10^8 human-like
+// bases, of whose suffixes the first sort leaves about a third in groups, 10.4
+// ms for 6*10^8 (2.0 and 20.3 with the rule for suffixes that end nearby in
+// every compare).  Sorting by 64-bit keys of 29 bases instead, eight passes of 24 bytes,
 // and prefix doubling for the rest took 15 ms in all at 10^8, this 9.
 constexpr int kRefineThreads = 512;
 constexpr int kSmallGroup = 32;
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const K *__restr
                                                                 uint8_t *headb) {
     __shared__ uint32_t heads[kRefineThreads / 32];
     __shared__ uint64_t next[kRefineThreads];
+    __shared__ uint32_t ends_near;  // some suffix of the tile ends within the next window
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint64_t tiles = (cnt + kRefineOut - 1) / kRefineOut;
     for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const K *__restr
         }
         const unsigned word = __ballot_sync(0xFFFFFFFFu, head);
         if (lane == 0) heads[warp] = word;
+        if (threadIdx.x == 0) ends_near = 0;
         __syncthreads();
         // the group's start (at or before t) and end (after t)
         const uint32_t upto = word & (0xFFFFFFFFu >> (31u - lane));
@@ -142,8 +145,10 @@ __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const K *__restr
         // into it: no head between them and it)
         const bool left_of = warp == 0, right_of = warp == kRefineThreads / 32 - 1;
         const bool reaches = left_of ? above == 0u : !right_of || upto == 0u;
-        if (live && reaches && size > 1u && size <= (uint32_t)kSmallGroup)
+        if (live && reaches && size > 1u && size <= (uint32_t)kSmallGroup) {
             next[threadIdx.x] = text_window(T, (uint64_t)i + depth);
+            if (n - i < depth + 32) ends_near = 1;
+        }
         __syncthreads();
         if (live && !left_of && !right_of) {
             uint64_t at = t;  // the item's place in the list
@@ -156,21 +161,40 @@ __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const K *__restr
                 const uint32_t windows = kRefineWindows / size;
                 const uint64_t mine = next[threadIdx.x];
                 uint32_t less = 0, ties = 0, ties_before = 0;
-                for (uint32_t u = 0; u < size; u++) {
-                    if (u == back) continue;
-                    const uint64_t theirs = next[threadIdx.x - back + u];
-                    int c = theirs < mine ? -1 : 1;
-                    const uint32_t j = vals[a + u];
-                    const uint64_t x = mine ^ theirs;
-                    const uint64_t same = x ? (uint64_t)(__clzll((long long)x) >> 1) : 32u;
-                    const uint64_t left = n - (i > j ? i : j) - depth;  // bases of the shorter one there
-                    if (same >= left)
-                        c = j > i ? -1 : 1;  // it ends first
-                    else if (x == 0)
-                        c = left > 32 ? order_beyond(T, n, i, j, depth + 32, windows) : (j > i ? -1 : 1);
-                    less += c < 0 ? 1u : 0u;
-                    ties += c == 0 ? 1u : 0u;
-                    ties_before += (c == 0 && u < back) ? 1u : 0u;
+                const uint64_t *group = next + (threadIdx.x - back);
+                if (!ends_near) {  // nearly always: the windows decide, but for equal ones
+                    uint32_t equal = 0;  // members with the same window
+                    for (uint32_t u = 0; u < size; u++) {
+                        const uint64_t theirs = group[u];
+                        less += theirs < mine ? 1u : 0u;
+                        equal |= theirs == mine ? 1u << u : 0u;
+                    }
+                    for (equal &= ~(1u << back); equal != 0u; equal &= equal - 1u) {
+                        const uint32_t u = __ffs(equal) - 1;
+                        const uint32_t j = vals[a + u];
+                        const bool ended = n - (i > j ? i : j) == depth + 32;
+                        const int c = ended ? (j > i ? -1 : 1) : order_beyond(T, n, i, j, depth + 32, windows);
+                        less += c < 0 ? 1u : 0u;
+                        ties += c == 0 ? 1u : 0u;
+                        ties_before += (c == 0 && u < back) ? 1u : 0u;
+                    }
+                } else {
+                    for (uint32_t u = 0; u < size; u++) {
+                        if (u == back) continue;
+                        const uint64_t theirs = group[u];
+                        int c = theirs < mine ? -1 : 1;
+                        const uint32_t j = vals[a + u];
+                        const uint64_t x = mine ^ theirs;
+                        const uint64_t same = x ? (uint64_t)(__clzll((long long)x) >> 1) : 32u;
+                        const uint64_t left = n - (i > j ? i : j) - depth;  // bases of the shorter one there
+                        if (same >= left)
+                            c = j > i ? -1 : 1;  // it ends first
+                        else if (x == 0)
+                            c = left > 32 ? order_beyond(T, n, i, j, depth + 32, windows) : (j > i ? -1 : 1);
+                        less += c < 0 ? 1u : 0u;
+                        ties += c == 0 ? 1u : 0u;
+                        ties_before += (c == 0 && u < back) ? 1u : 0u;
+                    }
                 }
                 at = a + less + ties_before;
                 more = ties != 0u;
