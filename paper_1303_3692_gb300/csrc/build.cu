@@ -538,14 +538,23 @@ cudaError_t launch_build_keys(sa_index *idx, cudaStream_t s) {
 // the outer two lanes only serve as neighbours.  The reads of the text (four
 // windows per rank, random) bound it, 6 % more of them for the two outer
 // lanes.
+//
+// The k-mer counts come from the same windows (k > 0).  For rank i let f(i) be
+// the smallest k-base string x with S_SA[i] < x: the suffix's k-base prefix
+// plus one when it has k bases or more, else the suffix padded with A (a
+// suffix that is a proper prefix of x sorts before x).  f is non-decreasing
+// along the suffix array, and kmer[x] = #{i : f(i) <= x} = #{suffixes sorting
+// before x}.  Rank i writes kmer[x] = i for f(i-1) <= x < f(i), with f(-1) = 0
+// and f(n) = 4^k + 1, so every entry is written once.  (A kernel of its own
+// read all records again for them: 3.7 ms at 6*10^8 bases.)
 constexpr int kRecRanks = 30;  // ranks per warp
 
 template <typename IdxT>
 __global__ void build_records_kernel(const uint64_t *__restrict__ T, const IdxT *__restrict__ sa, uint64_t n,
-                                     uint4 *rec) {
+                                     uint4 *rec, uint32_t k, uint32_t *kmer) {
     const unsigned lane = threadIdx.x & 31u;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    const uint64_t groups = (n + kRecRanks - 1) / kRecRanks;
+    const uint64_t groups = n / kRecRanks + 1;  // ranks 0 .. n: the last one ends the k-mer counts
     for (uint64_t g = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < groups; g += warps) {
         const uint64_t i = g * kRecRanks + lane - 1u;  // lane 0 of the first group: no rank (wraps)
         const bool live = i < n;
@@ -586,30 +595,13 @@ __global__ void build_records_kernel(const uint64_t *__restrict__ T, const IdxT 
             rec[2 * i + 1] = make_uint4((uint32_t)w[2], (uint32_t)(w[2] >> 32),
                                         ((uint32_t)(w[3] >> 32) & 0xFFFF0000u) | (lp << 8) | ln, (uint32_t)pos);
         }
-    }
-}
-
-// k-mer table.  For rank i let f(i) be the smallest k-base string x with
-// S_SA[i] < x: the suffix's k-base prefix plus one when it has k bases or
-// more, else the suffix padded with A (a suffix that is a proper prefix of x
-// sorts before x).  f is non-decreasing along the suffix array, and
-// kmer[x] = #{i : f(i) <= x} = #{suffixes sorting before x}.  Thread i writes
-// kmer[x] = i for f(i-1) <= x < f(i), with f(-1) = 0 and f(n) = 4^k + 1, so
-// every entry is written once.
-__device__ __forceinline__ uint64_t kmer_f(const uint4 *rec, uint64_t i, uint64_t n, uint32_t k) {
-    const uint4 r0 = rec[2 * i];
-    const uint32_t pos = rec[2 * i + 1].w;
-    const uint64_t w0 = ((uint64_t)r0.y << 32) | r0.x;
-    const uint64_t x = w0 >> (64u - 2u * k);
-    return (n - pos) >= k ? x + 1 : x;
-}
-
-__global__ void build_kmer_kernel(const uint4 *__restrict__ rec, uint64_t n, uint32_t k, uint32_t *kmer) {
-    const uint64_t top = (1ull << (2 * k)) + 1;
-    GS_LOOP(i, n + 1) {
-        const uint64_t fa = i == 0 ? 0 : kmer_f(rec, i - 1, n, k);
-        const uint64_t fb = i == n ? top : kmer_f(rec, i, n, k);
-        for (uint64_t x = fa; x < fb; x++) kmer[x] = (uint32_t)i;
+        if (k == 0) continue;
+        // the counts of the k-mers between this suffix and the one before it
+        uint64_t f = i < n ? (w[0] >> (64u - 2u * k)) + (n - pos >= k ? 1u : 0u) : 0;
+        if (i == n) f = (1ull << (2 * k)) + 1;
+        const uint64_t before = __shfl_up_sync(0xFFFFFFFFu, f, 1);  // 0 at rank 0
+        if (i <= n && lane >= 1u && lane <= (unsigned)kRecRanks)
+            for (uint64_t x = before; x < f; x++) kmer[x] = (uint32_t)i;
     }
 }
 
@@ -686,17 +678,24 @@ __global__ void krt_lo_kernel(const uint4 *__restrict__ krt, uint64_t n, uint32_
     GS_LOOP(x, entries + 1) out[x] = x < entries ? krt[4 * x].x : (uint32_t)n;
 }
 
+// The counts kmer[0 .. 4^k] wait in the end of the entries' own memory, so that
+// they need none of their own (4.3 GB at k = 15, mapped and unmapped for every
+// build).
+uint32_t *counts_of(const sa_index *idx) {
+    const uint64_t entries = 1ull << (2 * idx->kmer_k);
+    return reinterpret_cast<uint32_t *>(idx->krt) + 16 * entries - (entries + 1);
+}
+
+// The k-mer entries from the records and the counts that launch_build_records
+// left.
 cudaError_t launch_build_kmer(sa_index *idx, cudaStream_t s) {
     if (!idx->krt) return cudaSuccess;
-    // The counts kmer[0 .. 4^k] wait in the end of the entries' own memory, so
-    // that they need none of their own (4.3 GB at k = 15, mapped and unmapped
-    // for every build).  Each launch writes the entries from s on that lie
+    // Each launch writes the entries from s on that lie
     // before the counts from s on, all but a sixteenth of the rest, and the
     // counts of those it wrote are free to be written over by the next.
     constexpr uint64_t kLast = 256;
     const uint64_t entries = 1ull << (2 * idx->kmer_k);
-    uint32_t *kmer = reinterpret_cast<uint32_t *>(idx->krt) + 16 * entries - (entries + 1);
-    build_kmer_kernel<<<grid_for(idx->n + 1), kThreads, 0, s>>>(idx->rec, idx->n, idx->kmer_k, kmer);
+    const uint32_t *kmer = counts_of(idx);
     uint64_t done = 0;
     while (entries - done > kLast) {
         const uint64_t end = entries - (entries - done + 1 + 15) / 16;
@@ -715,13 +714,15 @@ cudaError_t launch_copy_kmer_counts(const sa_index *idx, uint32_t *dst, cudaStre
 }
 
 cudaError_t launch_build_records(sa_index *idx, cudaStream_t s) {
-    const unsigned g = grid_for((idx->n + kRecRanks - 1) / kRecRanks * 32);
+    const unsigned g = grid_for((idx->n / kRecRanks + 1) * 32);
+    const uint32_t k = idx->krt ? idx->kmer_k : 0u;
+    uint32_t *kmer = idx->krt ? counts_of(idx) : nullptr;
     if (idx->width == 4)
         build_records_kernel<uint32_t><<<g, kThreads, 0, s>>>(idx->text, reinterpret_cast<const uint32_t *>(idx->sa),
-                                                              idx->n, idx->rec);
+                                                              idx->n, idx->rec, k, kmer);
     else
         build_records_kernel<uint64_t><<<g, kThreads, 0, s>>>(idx->text, reinterpret_cast<const uint64_t *>(idx->sa),
-                                                              idx->n, idx->rec);
+                                                              idx->n, idx->rec, k, kmer);
     return cudaGetLastError();
 }
 
