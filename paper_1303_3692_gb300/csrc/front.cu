@@ -58,7 +58,9 @@ __device__ __forceinline__ uint32_t list_slot(const uint32_t *prefix, const uint
 // kFromList: the queries come from the k-mer-ordered list of bucket.cu (one
 // 64-byte record each: length, index, reference, first base in the packed
 // batch and first 192 bases, already checked) instead of the batch's offsets.
-template <bool kSingle, bool kFromList, Bases kBases>
+// kOneProbe: the entry's pivot is the only probe (input order's default), in
+// kernels of their own without the loop's registers (1 % of a call).
+template <bool kSingle, bool kFromList, Bases kBases, bool kOneProbe = false>
 __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_constant__ SearchLaunch a) {
     __shared__ FrontDesc sdesc[SA_MAX_REFS];
     __shared__ uint4 s_stage[kFrontThreads / 32][32][4];  // worklist records staged per warp
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
         // per probe: 3.1 Gbp, 4*10^7 x 150 bases 2.82 -> 2.71 ms.
         bool pending = false;
         uint32_t pend_pos = 0, pend_lcps = 0;
-        for (uint32_t p = 1; p < a.front_probes && __any_sync(0xFFFFFFFFu, go); p++) {
+        for (uint32_t p = 1; !kOneProbe && p < a.front_probes && __any_sync(0xFFFFFFFFu, go); p++) {
             const uint32_t M = bd.pivot();
             uint4 r0, r1;
             ldg32_if(go, d.rec + 2 * (size_t)M, &r0, &r1);
@@ -295,18 +297,21 @@ cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s) {
     if (L.n_q == 0) return cudaSuccess;
     const bool single = L.n_refs == 1 && L.q_ref == nullptr;
     const bool list = L.wrec_in != nullptr;
-    static int per_sm[10][64] = {};
+    static int per_sm[14][64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     using Kernel = void (*)(SearchLaunch);
     constexpr Bases P = Bases::Packed, S = Bases::PackedStrands, A = Bases::Ascii;
-    static const Kernel kernels[10] = {front_kernel<false, false, P>, front_kernel<true, false, P>,
+    static const Kernel kernels[14] = {front_kernel<false, false, P>, front_kernel<true, false, P>,
                                        front_kernel<false, false, S>, front_kernel<true, false, S>,
                                        front_kernel<false, true, P>,  front_kernel<true, true, P>,
                                        front_kernel<false, true, S>,  front_kernel<true, true, S>,
-                                       front_kernel<false, true, A>,  front_kernel<true, true, A>};
-    const int which = (single ? 1 : 0) + (list ? 4 : 0) + 2 * (L.fused ? 2 : (L.revcomp || L.strand_bits ? 1 : 0));
+                                       front_kernel<false, true, A>,  front_kernel<true, true, A>,
+                                       front_kernel<false, false, P, true>, front_kernel<true, false, P, true>,
+                                       front_kernel<false, false, S, true>, front_kernel<true, false, S, true>};
+    const int bases = L.fused ? 2 : (L.revcomp || L.strand_bits ? 1 : 0);
+    const int which = (single ? 1 : 0) + 2 * bases + (list ? 4 : L.front_probes == 1 ? 10 : 0);
     const Kernel kernel = kernels[which];
     int &bps = per_sm[which][dev];
     if (bps == 0) {
