@@ -272,13 +272,13 @@ bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uin
     return n_q <= kSmallQueries && total <= (wide_brackets(refs, n_refs) ? kSmallBases / 2 : kSmallBases);
 }
 
-// Whether, in k-mer order, the scatter packs the ASCII bases it needs itself,
-// tile by tile, instead of reading a packed copy of the batch that a kernel
-// before it writes: for queries of up to 192 bases on average, which its tiles
-// have room for and its records carry (longer ones are compared in the packed
-// copy past that).  Words have 32-bit numbers there.
-constexpr uint64_t kFusedBases = 192;
-bool fused_packing(uint64_t n_q, uint64_t total) { return total <= kFusedBases * n_q && total < (1ull << 36); }
+// Queries of up to this many bases on average have room in the k-mer order's
+// records and in the scatter's tiles, which then pack the ASCII bases they need
+// themselves instead of reading a packed copy of the batch that a kernel before
+// them writes (with 32-bit numbers for its words).  Longer ones are compared
+// with more of the text than their records carry, from the packed copy, and the
+// persistent pass does that in iterations of its own.
+constexpr uint64_t kRecordBases = 192;
 
 // The search of a batch whose inputs are in device memory: ascii holds the
 // batch's bases from offset `first` on (query q is ascii[q_off[q] - first ..
@@ -337,7 +337,8 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     // that large could not be resident anyway)
     if (!plain && tq_words * 32 >= kListMaxBase) return SA_ERR_ARG;
     const bool kmer_order = !plain && use_kmer_order(refs, n_refs, n_q, order);
-    const bool fused = kmer_order && fused_packing(n_q, total);
+    const bool long_queries = total > kRecordBases * n_q;
+    const bool fused = kmer_order && !long_queries && total < (1ull << 36);
     uint64_t *tq = fused ? nullptr : sc.get<uint64_t>(SA_TQ_LEAD_WORDS + tq_words) + SA_TQ_LEAD_WORDS;
     uint32_t *tv = fused ? nullptr : sc.get<uint32_t>(tq_words);
     uint4 *wrec = plain ? nullptr : sc.get<uint4>(4 * n_q);
@@ -405,6 +406,7 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.wl_in_count = reinterpret_cast<uint32_t *>(flags + 4);
     L.bad_ref = flags + 3;
     L.batch_dirty = flags + 5;
+    L.long_queries = long_queries;
     L.fused = fused;
 
     if (!fused && (err = launch_pack_batch(L, tq, tvb, tv, s)) != cudaSuccess) return status_from_cuda(err);

@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
     if (__any_sync(0xFFFFFFFFu, any_bad_ref) && lane == 0) atomicOr(a.bad_ref, 1);
 }
 
-// The scatter of a batch that is not packed (api.cu: fused_packing).  The CTA
+// The scatter of a batch that is not packed (api.cu: kRecordBases).  The CTA
 // packs its tile's bases itself, coalesced, into shared memory -- consecutive
 // queries are one stretch of the batch -- and every 16-byte piece of a record
 // is computed from there as it is stored, so the packed batch is neither

@@ -548,7 +548,7 @@ struct Bounds {
 // Where a kernel reads a query's bases beyond those its records carry: the
 // packed batch (forward queries only, or of either strand), or the batch's
 // ASCII bytes, of either strand (a batch whose kernels pack what they need
-// themselves; api.cu: fused_packing).
+// themselves; api.cu: kRecordBases).
 enum class Bases { Packed, PackedStrands, Ascii };
 
 // A query's 32-base window at base off (a multiple of 32 below m).
@@ -736,6 +736,7 @@ struct SearchLaunch {
     uint32_t smem_bytes;      // shared-memory key tables
     uint32_t threads, blocks, chunk;
     uint32_t front_probes;    // probes per query in the first pass
+    bool long_queries;        // the queries' average length is past what their records carry
     bool fused;               // k-mer order: no packed batch, the scatter packs what it needs (tq, tvb, tv,
                               // batch_dirty are not used)
     bool revcomp;             // search every query's reverse complement

@@ -152,13 +152,18 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s for the key-table copy
 //   deep      load the suffix record of rank M = L + (R - L)/2 (32 bytes: 104
 //             bases, the common prefixes with the ranks beside M, SA[M]) -- with query bases 64-127 from the worklist
 //             record in the same round -- and compare; only when all 104
-//             bases tie does the compare continue in the packed text.
+//             bases tie does the compare continue in the packed text;
+//   text      (kLong: batches of long queries) such a compare in iterations of
+//             its own, 64 bases each, so that the warp's other lanes go on:
+//             2^20 queries of 1024 bases 250 -> 190 us.  For queries a compare
+//             or two beyond their records its registers spill and cost more
+//             than they save (150 bases: 1.64 -> 1.84 ms).
 // (The bounds' own arithmetic: Bounds in sa_internal.cuh.)
 // Warps take chunks of worklist entries from one global counter, each
 // chunk's base fetched while the previous chunk is handed out.
 // Launch bounds: 1024 threads, one CTA per SM, at most 64 registers (no
 // spills); smaller CTAs may share an SM up to 1024 threads in all.
-template <typename IdxT, bool kSingle, Bases kBases>
+template <typename IdxT, bool kSingle, Bases kBases, bool kLong>
 __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__ SearchLaunch a) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ SmemDesc sdesc[SA_MAX_REFS];
@@ -220,6 +225,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
     Bounds bd;
     bd.start(0, 0);
     uint32_t k = 0;
+    uint32_t toff = 0, tpos = 0, tlcps = 0;  // (text) the next base, the suffix, its record's common prefixes
 
     for (;;) {
         unsigned need = __ballot_sync(0xFFFFFFFFu, !active);
@@ -251,7 +257,8 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
         // This iteration's one round of loads: the worklist record (init) or
         // the suffix record at the pivot and query bases 64-127 (deep).
         const bool init = fresh;
-        const bool deep = !init && k == 0;
+        const bool text = kLong && !init && toff != 0;
+        const bool deep = !init && !text && k == 0;
         uint32_t M = bd.pivot();
         const uint4 *wrec = a.wrec + 4 * (size_t)wi;
         uint4 r0, r1;
@@ -259,6 +266,21 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
         // the query's bases 0-63 (init) or 64-127 (deep) from its worklist record
         uint64_t x2 = 0, x3 = 0;
         ldg16_if(init || (deep && m > 64u), wrec + (init ? 2 : 3), &x2, &x3);
+        uint64_t t0 = 0, t1 = 0, t2 = 0, p0 = 0, p1 = 0;  // (text) 64 bases of the suffix and of the query
+        if (kLong && text) {
+            const uint32_t rem = n - tpos;
+            const uint64_t *at = T + ((tpos + toff) >> 5);
+            if (toff < rem) {
+                t0 = ldg_u64(at);
+                t1 = ldg_u64(at + 1);
+                if (toff + 32u < rem) t2 = ldg_u64(at + 2);
+            }
+            const auto src = window_source<kBases>(a, qa, m);
+            // bases 96-127 and 128-159 are the record's eighth and fourth words
+            const uint64_t *rec_words = reinterpret_cast<const uint64_t *>(wrec);
+            p0 = toff == 96u ? __ldg(rec_words + 7) : toff == 128u ? __ldg(rec_words + 3) : src(toff);
+            if (toff + 32u < m) p1 = toff == 96u ? __ldg(rec_words + 3) : src(toff + 32u);
+        }
 
         if (init) {
             fresh = false;
@@ -280,6 +302,7 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             q1 = x3;
             bd.start(r0.x, r0.y);
             k = KM != nullptr ? 0u : (depth ? 1u : 0u);
+            toff = 0;
             continue;
         }
 
@@ -297,10 +320,31 @@ __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__
             if (und) c = cmp_suffix_qw(T, n, (uint32_t)sa_at<IdxT>(SAp, M), window_source<kBases>(a, qa, m), m, 64u, &l);
             const uint32_t nk = 2u * k + (c == CMP_GREATER ? 1u : 0u);
             k = (c == CMP_PREFIX || nk >= (1u << depth)) ? 0u : nk;
+        } else if (kLong && text) {
+            const uint32_t rem = n - tpos, sh = 2u * ((tpos + toff) & 31u);
+            const uint64_t w0 = (t0 << sh) | ((t1 >> 1) >> (63u - sh)), w1 = (t1 << sh) | ((t2 >> 1) >> (63u - sh));
+            c = cmp_window(p0, w0, min(32u, m - toff), toff < rem ? min(32u, rem - toff) : 0u, toff, m, &l);
+            if (c == 2) {
+                const uint32_t o = toff + 32u;
+                c = cmp_window(p1, w1, min(32u, m - o), o < rem ? min(32u, rem - o) : 0u, o, m, &l);
+            }
+            if (c == 2) {
+                toff += 64u;
+                continue;
+            }
+            toff = 0;
+            lp = tlcps >> 8;
+            ln = tlcps & 0xFFu;
         } else {
             bool und = false;
             const uint64_t qw4[4] = {q0, q1, x2, x3};
             c = cmp_record(qw4, m, r0, r1, n, &l, &und);
+            if (kLong && und) {
+                toff = max(kRecBases, min(bd.lcpL, bd.lcpR)) & ~31u;
+                tpos = r1.w;
+                tlcps = r1.z & 0xFFFFu;
+                continue;
+            }
             if (und) {
                 // query bases 96-127 are x3, 128-159 the worklist record's second word pair
                 const auto src = window_source<kBases>(a, qa, m);
@@ -442,12 +486,14 @@ cudaError_t launch_search(const SearchLaunch &L, cudaStream_t s) {
     auto pick = [&](auto idx_tag, auto single_tag) {
         using I = decltype(idx_tag);
         constexpr bool S = decltype(single_tag)::value;
+        const bool strands = L.revcomp || L.strand_bits;
         if (L.fused)
-            go(search_kernel<I, S, Bases::Ascii>);
-        else if (L.revcomp || L.strand_bits)
-            go(search_kernel<I, S, Bases::PackedStrands>);
+            go(search_kernel<I, S, Bases::Ascii, false>);
+        else if (L.long_queries)
+            strands ? go(search_kernel<I, S, Bases::PackedStrands, true>) : go(search_kernel<I, S, Bases::Packed, true>);
         else
-            go(search_kernel<I, S, Bases::Packed>);
+            strands ? go(search_kernel<I, S, Bases::PackedStrands, false>)
+                    : go(search_kernel<I, S, Bases::Packed, false>);
     };
     if (L.width == 4)
         single ? pick(uint32_t{}, std::true_type{}) : pick(uint32_t{}, std::false_type{});
