@@ -70,7 +70,7 @@ TRAFFIC = {"kernel_sha": "b52eb447dc121722", "kernel": "search",
 # Sources of each phase's kernels (the traffic figure is tied to them).
 PHASE_SOURCES = {
     "pack_batch_kernel": ("pack.cu", "sa_internal.cuh"),
-    "search": ("bucket.cu", "front.cu", "search.cu", "sa_internal.cuh"),
+    "search": ("bucket.cu", "front.cu", "search.cu", "first_pass.cuh", "sa_internal.cuh"),
     "locate": ("locate.cu", "sa_internal.cuh"),
 }
 
@@ -484,7 +484,7 @@ def run_plain_small(args, world, rank, local):
         "config": {"workload": "plain-1Mbp-100k-q32", "n": int(w.ref.size), "queries_per_step": n_q, "m": 32,
                    "mode": "count", "kmer_k": idx.kmer_k, "l2": "flushed between steps; index L2-resident size"},
         "query_bases_per_s": value * 32, "search_kernel_ms": statistics.mean(kern_ms), "step_ms_all": step_ms,
-        "build_s": build_s, "gpu_launches": args.steps * 3, "clocks": clocks,
+        "build_s": build_s, "gpu_launches": args.steps * (3 if args.front_probes else 1), "clocks": clocks,
     }
     print(json.dumps(line), flush=True)
 
@@ -520,8 +520,9 @@ def verified_suffix_array(idx, ref):
 def human_byte_model(T, sa_h, w, k: int, cap: int, sample: int = 20000, seed: int = 7, kmer_order: bool = False):
     """Algorithmic bytes and random reads per query of each phase, from the
     oracle's byte model (oracle.probe_model_bracket: the lockstep search over
-    each query's k-mer bracket, 32-byte records of 112 bases, text windows
-    past them) on a seeded sample of the batch.  The bracket of a query is
+    each query's k-mer bracket, 32-byte records of 104 bases with the common
+    prefixes of the ranks beside them, text windows past them) on a seeded
+    sample of the batch.  The bracket of a query is
     found by the oracle's binary search for its first k bases and their
     successor over the verified suffix array (no 4^k table)."""
     import oracle
@@ -556,11 +557,15 @@ def human_byte_model(T, sa_h, w, k: int, cap: int, sample: int = 20000, seed: in
     per = {key: v / c for key, v in tot.items()}
     m = per["m"]
     probes = 64 * per["entry"] + 32 * per["further"] + 32 * per["windows"] + 32  # + the 32-byte result
-    if kmer_order:
-        # sampling pass (offsets and the first two packed words of every 32nd
-        # query), scatter pass (offsets and packed bases read -- a batch the
-        # packing found clean needs no validity masks -- and a 64-byte record
-        # written), first pass reads the record
+    pack = m + m / 4  # ASCII read, packed words written (no validity masks for a clean batch)
+    if kmer_order and m <= 192:
+        # sampling pass (offsets and the first bases of every 32nd query),
+        # scatter pass (offsets and ASCII bases read, packed on the way, and a
+        # 64-byte record written), first pass reads the record
+        pack = 0.0
+        reorder = (8 + 36) / 32 + (8 + m + 64)
+        search = reorder + 64 + probes
+    elif kmer_order:  # the same from the packed copy of the batch
         reorder = (8 + 16) / 32 + (8 + m / 4 + 64)
         search = reorder + 64 + probes
     else:
@@ -568,11 +573,11 @@ def human_byte_model(T, sa_h, w, k: int, cap: int, sample: int = 20000, seed: in
         search = 8 + m / 4 + probes
     return {
         "sample": int(c), "k": k,
-        # pack: ASCII read, packed words written (no validity masks for a clean batch)
-        "bytes_per_query": {"pack_batch_kernel": m + m / 4, "search": search,
+        "bytes_per_query": {"pack_batch_kernel": pack, "search": search,
                             "locate": 32 + 8 + 16 * per["kept"]},
-        # random sectors per query: 2 for the 64-byte entry, 1 per record, 1 per text window
-        "random_sectors_per_query": 2 * per["entry"] + per["further"] + per["windows"],
+        # random reads per query: the 64-byte entry (two lanes' halves of one
+        # line, one request), a record, a text window
+        "random_reads_per_query": per["entry"] + per["further"] + per["windows"],
         "entry_reads_per_query": per["entry"], "record_probes_per_query": per["further"],
         "text_windows_per_query": per["windows"], "mean_count": per["count"], "mean_kept": per["kept"],
         "reorder_bytes_per_query": reorder, "order": "kmer" if kmer_order else "input",
@@ -661,8 +666,9 @@ def run_human_sized(args, world, rank, local):
     pos = torch.empty(max(1, total_pos), dtype=torch.int64, device=dev)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     order = sa.sa_search_order(idx, n_q, p)
-    # pack, [bucket count, scan, scatter,] first pass, persistent pass, 3 locate kernels
-    launches = 1 + (3 if order == "kmer" else 0) + 2 + 3
+    # pack, or in k-mer order bucket sample, plan, scatter (which packs) and
+    # fill; first pass, persistent pass, 2 locate kernels
+    launches = (4 if order == "kmer" else 1) + 2 + 2
 
     def timed(mode, steps, clk_needed=False):
         ts, ks, pk, lc = [], [], [], []
@@ -776,18 +782,18 @@ def run_human_sized(args, world, rank, local):
         traffic = (HUMAN_TRAFFIC["dram_bytes_per_launch"]
                    if HUMAN_TRAFFIC["kernel"] == dominant and HUMAN_TRAFFIC["kernel_sha"] == kernel_sha(dominant)
                    else None)
-        sect = model["random_sectors_per_query"] * n_q / (phases["search"] / 1e3) / 1e9
+        rand = model["random_reads_per_query"] * n_q / (phases["search"] / 1e3) / 1e9
         rr64 = ceiling.get("64GB_32B")
         rrix = ceiling.get(f"{at_index >> 30}GB_32B")
         roof = {"bound": "hbm", "achieved": per_kernel[dominant]["achieved_gbs"], "peak": peak, "unit": "GB/s",
                 "frac": per_kernel[dominant]["frac"], "traffic": traffic, "kernel": dominant, "peak_kind": peak_kind,
                 "bytes_per_query": model["bytes_per_query"][dominant], "bytes_source": model["source"],
                 "per_kernel": per_kernel,
-                "random_reads": {"kernel": "search", "achieved": sect, "unit": "G sectors/s",
-                                 "sectors_per_query": model["random_sectors_per_query"],
-                                 "peak_64GB": rr64, "frac_64GB": sect / rr64 if rr64 else None,
+                "random_reads": {"kernel": "search", "achieved": rand, "unit": "G reads/s",
+                                 "reads_per_query": model["random_reads_per_query"],
+                                 "peak_64GB": rr64, "frac_64GB": rand / rr64 if rr64 else None,
                                  "peak_at_index_size": rrix, "index_size_GB": at_index >> 30,
-                                 "frac_at_index_size": sect / rrix if rrix else None,
+                                 "frac_at_index_size": rand / rrix if rrix else None,
                                  "ceilings_G_reads_per_s": ceiling,
                                  "peak_source": "sa_random_read_rate_ex(size, 1024 threads/SM, 64 dependent reads)"},
                 "model": model}
@@ -1240,7 +1246,7 @@ def run_ours(args, world, rank, local):
                                                                         phases["search"])},
         "e2e": {"value": n_q / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": e2e_s * 1e3},
-        "gpu_launches": args.steps * 6,
+        "gpu_launches": args.steps * 5,  # pack, first pass, persistent pass, 2 locate kernels
         "roofline": roof,
         "cpu_baseline": cpu,
         "clocks": clocks,

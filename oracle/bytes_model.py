@@ -15,13 +15,14 @@ the 64-base chunks those probes compare, starting at min(lcp(P,S_L),
 lcp(P,S_R)).  Locate adds w * min(count, cap) written plus the same read.
 
 The second figure models the search with a k-mer table of plain counts and
-32-byte suffix records of 112 bases (oracle_probe_model_kmer):
+32-byte suffix records of 104 bases and the common prefixes with the ranks
+beside them (oracle_probe_model_kmer):
 
     B_q = ceil(m/4) + 32 * [m >= k] + 32 * P'_q + 32 * W_q + 3 * w
 
 P'_q probes read one record sector each (below depth d0 only when no k-mer
 bracket applies), W_q counts the 32-base text windows of compares that tie on
-a record's 112 bases.  The third is the CUDA path's layout, whose 64-byte k-mer
+a record's 104 bases (or the 192 of the first pivot).  The third is the CUDA path's layout, whose 64-byte k-mer
 entries carry the bracket's first pivot, so that probe costs no access of its
 own:
 

@@ -577,15 +577,58 @@ void oracle_kmer_table(const uint8_t *T, int64_t n, const int64_t *sa, int k, in
 }
 
 /* Byte model of the search as the CUDA path runs it on an index with a k-mer
- * table and 16-byte suffix records (measurement, not a parity output).
+ * table and 32-byte suffix records (measurement, not a parity output).
  * A query of m >= k bases starts between ranks table[x] - 1 and table[x + 1]
- * (x = its first k bases) and costs one table sector; shorter queries start
- * at [-1, n) and their first d0 probes are free (shared-memory key table).
- * Every other probe of the lockstep lower/upper-bound search reads one
- * 32-byte record sector holding the suffix's first 112 bases; a compare that
- * agrees on all 112 (m > 112, suffix >= 112 bases) also reads the 32-base
- * text windows from base 96 up to the one where it is decided.  *probes,
- * *windows count them; *table_reads is 1 or 0. */
+ * (x = its first k bases) and costs one read of the table's entry, which also
+ * holds the first 192 bases of the suffix its first probe compares with;
+ * shorter queries start at [-1, n) and their first d0 probes are free
+ * (shared-memory key table).  Every other probe of the lockstep lower/upper-
+ * bound search reads one 32-byte record holding the suffix's first 104 bases.
+ * A compare that agrees on all an entry or record holds (m and the suffix
+ * both longer) also reads the 32-base text windows from the 32-aligned base
+ * at or below that length up to the one where it is decided.  Entry and
+ * record also hold the suffix's common prefixes with the suffixes at the
+ * ranks beside it, at most 255, and a neighbour whose compare they decide is
+ * not probed: see bracket_neighbours.  *probes, *windows count them;
+ * *table_reads is 1 or 0. */
+
+/* Bases that the suffixes at p and q share, at most 255. */
+static int64_t shared_bases(const uint8_t *T, int64_t n, int64_t p, int64_t q)
+{
+    int64_t l = 0;
+    while (l < 255 && p + l < n && q + l < n && T[p + l] == T[q + l])
+        l++;
+    return l;
+}
+
+/* What the compare at rank M (outcome c, l common bases, query length m) says
+ * of the ranks beside it, from their common prefixes with S_sa[M].  *before and
+ * *after become 1 when that rank has the query as a prefix or lies on the same
+ * side of it as M, 0 when it has not or lies on the other side, and stay -1
+ * when that is not known (255 stands for 255 or more). */
+static void bracket_neighbours(const uint8_t *T, int64_t n, const int64_t *sa, int64_t M, int c, int64_t l, int64_t m,
+                               int *before, int *after)
+{
+    int64_t side[2];
+    side[0] = M > 0 ? shared_bases(T, n, sa[M - 1], sa[M]) : 0;
+    side[1] = M + 1 < n ? shared_bases(T, n, sa[M], sa[M + 1]) : 0;
+    int *out[2];
+    out[0] = before;
+    out[1] = after;
+    for (int i = 0; i < 2; i++) {
+        *out[i] = -1;
+        int64_t need = c == 0 ? m : l; /* bases the neighbour shares with the query, if with S_sa[M] */
+        if ((i == 0 && M == 0) || (i == 1 && M + 1 == n))
+            *out[i] = 0; /* no such rank */
+        else if (c == 0 && side[i] >= need)
+            *out[i] = 1;
+        else if (c != 0 && side[i] > need)
+            *out[i] = 1;
+        else if (side[i] < need && side[i] < 255)
+            *out[i] = 0;
+    }
+}
+
 /* The same model for one query given its k-mer bracket: has_bracket says
  * whether the query starts between ranks tlo - 1 and thi (tlo = table[x],
  * thi = table[x + 1] for its first k bases x), else it starts at [-1, n) with
@@ -626,21 +669,38 @@ void oracle_probe_model_bracket(const uint8_t *T, int64_t n, const int64_t *sa, 
         int c = query_cmp(T, n, sa[M], P, m, &l);
         if (depth >= free_levels) {
             (*probes)++;
-            if (m > 112 && n - sa[M] >= 112 && l >= 112) {
+            int64_t held = has_bracket && depth == 0 ? 192 : 104;
+            if (m > held && n - sa[M] >= held && l >= held) {
                 int64_t last = l < m - 1 ? l : m - 1;
-                *windows += last / 32 - 3 + 1; /* windows from base 96 to the deciding one */
+                *windows += last / 32 - held / 32 + 1; /* windows up to the deciding one */
             }
         }
+        int before = -1, after = -1;
+        if (depth >= free_levels)
+            bracket_neighbours(T, n, sa, M, c, l, m, &before, &after);
         depth++;
-        if (c == 0 && phase == 0) {
-            HL = M;
-            HR = R;
-            R = M;
-            phase = 1;
-        } else if (c < 0 || (c == 0 && phase == 1)) {
-            R = M;
+        if (c == 0) {
+            if (phase == 0) {
+                HL = after == 1 ? M + 1 : M;
+                HR = after == 0 ? M + 1 : R;
+                phase = 1;
+            } else if (phase == 2) {
+                L = after == 1 ? M + 1 : M;
+                if (after == 0)
+                    R = M + 1;
+                continue;
+            }
+            R = before == 1 ? M - 1 : M;
+            if (before == 0)
+                L = M - 1;
+        } else if (c < 0) {
+            R = before == 1 ? M - 1 : M;
+            if (before == 0)
+                L = M - 1;
         } else {
-            L = M;
+            L = after == 1 ? M + 1 : M;
+            if (after == 0)
+                R = M + 1;
         }
     }
 }
