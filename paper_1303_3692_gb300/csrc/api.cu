@@ -658,9 +658,15 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
     // took 17 of 49 ms at 10^8 bases.  The other constructions' scratch is
     // returned first, so that it never coexists with the two.
     const bool scratch_in_place = !(flags & (SA_BUILD_HOST | SA_BUILD_DC3));
-    if (scratch_in_place && (st = alloc_search_arrays(idx)) != SA_OK) {
-        free_index(idx);
-        return st;
+    if (scratch_in_place) {
+        // what the pool keeps of earlier calls (and of a host text's copy) must
+        // not stand in the way of the index's own memory
+        cudaStreamSynchronize(s);
+        cudaMemPoolTrimTo(scratch_pool(idx->device), 0);
+        if ((st = alloc_search_arrays(idx)) != SA_OK) {
+            free_index(idx);
+            return st;
+        }
     }
     if (flags & SA_BUILD_HOST) {
         std::vector<char> copy;
