@@ -39,9 +39,9 @@ WORKLOAD = "repetitive-100Mbp-10M-q100-locate64"
 
 # Algorithmic bytes per query of each phase of a step on this workload
 # (m = 100, k = 14), from the oracle's byte model (oracle/bytes_model.py:
-# oracle_probe_model_kmer on 20,000 seeded queries: 1.19375 record probes per
-# query, 0.41265 of them after the one that comes with the 64-byte k-mer entry,
-# 6.58 occurrences on average, 0.51 positions kept at cap 64):
+# oracle_probe_model_kmer on 20,000 seeded queries: 1.04195 record probes per
+# query, 0.26620 of them after the one that comes with the 64-byte k-mer entry,
+# 7.72 occurrences on average, 0.55 positions kept at cap 64):
 #   pack_batch_kernel: 100 ASCII bytes read + 25 packed bytes written (a batch
 #       without a non-base byte needs no validity masks)        = 125
 #   search (front_kernel + search_kernel): 8 offset bytes + 25 packed query
@@ -51,13 +51,13 @@ WORKLOAD = "repetitive-100Mbp-10M-q100-locate64"
 #       position bytes (suffix-array entry read and written)   = 44.1
 KERNEL_BYTES_PER_QUERY = {
     "pack_batch_kernel": 100 + 25,  # a clean batch: no validity masks written
-    "search": 8 + 25 + 64 + 32 * 0.41265 + 32,
-    "locate": 32 + 8 + 4.1072,
+    "search": 8 + 25 + 64 + 32 * 0.26620 + 32,
+    "locate": 32 + 8 + 4.4308,
 }
 # Random DRAM accesses per query of the search phase (the k-mer entry, further
 # record probes, text windows), from the same model: random 32- or 64-byte
 # reads are bounded by the DRAM's row activations, not by its bandwidth.
-RANDOM_ACCESSES_PER_QUERY = {"search": 1.41265}
+RANDOM_ACCESSES_PER_QUERY = {"search": 1.26620}
 BYTES_SOURCE = "oracle/bytes_model.py --workload repetitive-100m (k = 14)"
 
 # DRAM bytes (read + write) per step of the dominant phase from one ncu
@@ -878,10 +878,10 @@ def serve_on_index(idxs, q_bases, q_offsets, seconds: float, rate: float = 2000.
 
 
 # DRAM bytes (read + write) of one 3.1 Gbp search phase (bucket sample, plan,
-# scatter and fill, first pass, persistent pass) from one single-pass ncu capture of the
+# scatter with the packing, fill, first pass, persistent pass) from one single-pass ncu capture of the
 # default bench command (the median of its 13 full-size steps), valid only
 # while the phase's sources hash to kernel_sha.
-HUMAN_TRAFFIC = {"kernel_sha": "fc28c78cf4b08d9b", "kernel": "search", "dram_bytes_per_launch": 72_274_846_976}
+HUMAN_TRAFFIC = {"kernel_sha": "90b181caf3b7b549", "kernel": "search", "dram_bytes_per_launch": 75_726_573_056}
 
 
 def cpu_baseline_sa(T, sa_h, w, args, sa_note: str):
