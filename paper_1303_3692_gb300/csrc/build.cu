@@ -526,6 +526,32 @@ cudaError_t launch_build_keys(sa_index *idx, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The kN windows of 32 bases from base b of the text on (zeros past its end), by
+// 16-byte loads of the pairs of words they lie in (three, where a window by
+// itself takes two of 8 bytes): at 6*10^8 bases the records take 15.3 -> 14.0 ms
+// and the entries 21.0 -> 20.3.
+template <int kN>
+__device__ __forceinline__ void text_windows(const uint64_t *__restrict__ T, uint64_t n, uint64_t b, uint64_t *w) {
+    constexpr int kPairs = (kN + 3) / 2;  // kN + 1 words, from an even one on
+    const uint64_t first = b >> 5, even = first & ~1ull;
+    const bool odd = (first & 1u) != 0;
+    uint64_t x[2 * kPairs];
+#pragma unroll
+    for (int p = 0; p < kPairs; p++) {
+        const uint64_t at = even + 2u * p;
+        const bool need = at * 32 < n && (2 * p <= kN || odd);  // its second word is at most the first of the padding
+        const ulonglong2 v = need ? __ldg(reinterpret_cast<const ulonglong2 *>(T + at)) : make_ulonglong2(0, 0);
+        x[2 * p] = v.x;
+        x[2 * p + 1] = v.y;
+    }
+    const unsigned sh = (unsigned)(b & 31u) * 2u;
+#pragma unroll
+    for (int j = 0; j < kN; j++) {
+        const uint64_t hi = odd ? x[j + 1] : x[j], lo = odd ? x[j + 2] : x[j + 1];
+        w[j] = (hi << sh) | ((lo >> 1) >> (63u - sh));
+    }
+}
+
 // Suffix records: for rank i, the first 104 bases of suffix SA[i], its common
 // prefixes with the suffixes at the ranks beside it, and SA[i] itself in one
 // 32-byte entry (one DRAM sector), so that a probe of the search reads one
@@ -536,7 +562,7 @@ cudaError_t launch_build_keys(sa_index *idx, cudaStream_t s) {
 // suffixes' first 128 bases, each lane counts the bases it shares with the
 // next lane's (reading on in the text past 128 equal ones, up to 255), and
 // the outer two lanes only serve as neighbours.  The reads of the text (four
-// windows per rank, random) bound it, 6 % more of them for the two outer
+// windows per rank, random: 160 bytes of DRAM traffic) bound it, 6 % more of them for the two outer
 // lanes.
 //
 // The k-mer counts come from the same windows (k > 0).  For rank i let f(i) be
@@ -560,13 +586,7 @@ __global__ void build_records_kernel(const uint64_t *__restrict__ T, const IdxT 
         const bool live = i < n;
         const uint64_t pos = live ? (uint64_t)sa[i] : 0;
         uint64_t w[4] = {0, 0, 0, 0};
-        if (live) {
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint64_t b = pos + 32ull * j;
-                w[j] = b < n ? text_window(T, b) : 0ull;
-            }
-        }
+        if (live) text_windows<4>(T, n, pos, w);
         // bases shared with the next lane's suffix
         const uint64_t npos = __shfl_down_sync(0xFFFFFFFFu, pos, 1);
         const bool nlive = __shfl_down_sync(0xFFFFFFFFu, (int)live, 1) != 0 && lane < 31u;
@@ -620,7 +640,8 @@ __global__ void build_records_kernel(const uint64_t *__restrict__ T, const IdxT 
 // the second 96 are read from the text (random; the records are read in
 // order), and each half entry is one 32-byte store: 10^8 bases (17 GB of
 // entries) 5.2 -> 3.9 ms against six text windows and four 16-byte stores,
-// 6*10^8 (69 GB) 23.7 -> 21.1 ms, bound there by the text reads.
+// 6*10^8 (69 GB) 23.7 -> 21.0 ms (20.3 with text_windows), bound there by the text
+// reads.
 __device__ __forceinline__ void st32(void *p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
     asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
@@ -639,11 +660,7 @@ __device__ __forceinline__ void write_krt_entry(uint64_t x, uint32_t lo, uint32_
         e[0] = ((uint64_t)r0.y << 32) | r0.x;
         e[1] = ((uint64_t)r0.w << 32) | r0.z;
         e[2] = ((uint64_t)r1.y << 32) | r1.x;
-#pragma unroll
-        for (int i = 3; i < 6; i++) {
-            const uint64_t b = pos + 32ull * i;
-            e[i] = b < n ? text_window(T, b) : 0ull;
-        }
+        text_windows<3>(T, n, pos + 96, e + 3);
     }
     uint4 *dst = krt + 4 * x;
     st32(dst, ((uint64_t)hi << 32) | lo, ((uint64_t)last << 32) | pos, e[0], e[1]);

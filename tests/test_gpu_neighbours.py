@@ -74,3 +74,14 @@ def test_sizes_around_a_warps_ranks(sa, n):
         qs = [text[s:s + m].encode() for m in (1, 2, 3, 7, n) for s in range(0, n, 3)]
         qs += [q + b"A" for q in qs[:20]] + [b"T" + q for q in qs[:20]]
         _check(sa, ref, [q for q in qs if q])
+
+
+@pytest.mark.parametrize("n", [63, 64, 65, 95, 96, 97, 127, 128, 129, 159, 160, 161, 191, 192, 193, 223, 224, 225, 256, 257])
+def test_windows_at_the_texts_end(sa, n):
+    # the windows of records (4 words on from a suffix) and entries (3 more) come
+    # by pairs of words: the last pairs of the text, at either parity
+    ref = datagen.reference(n, n, gc=0.5)
+    qs = [ref[s:s + m].tobytes() for s in range(n) for m in (40, 100, 104, 105, 128, 192, n) if s + m <= n]
+    qs += [q + b"A" for q in qs[::5]] + [q[:-1] + b"T" for q in qs[::7]]
+    _check(sa, ref, qs, 2)
+    _check(sa, ref, qs)
