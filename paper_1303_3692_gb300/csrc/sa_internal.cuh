@@ -766,7 +766,9 @@ inline uint32_t locate_tile_shift(uint64_t n_q) {
 // the locate need not read every result to find the tile sums.
 // In input order the lanes storing at the same time hold consecutive queries,
 // so those sharing a tile add their counts with one atomic; in k-mer order
-// each lane adds its own.
+// each lane adds its own.  32 counts of up to trunc_cap may not fit 32 bits
+// (an enormous cap and short or empty queries of a large text): the warp then
+// adds their halves apart.
 __device__ __forceinline__ void store_result_sum(const SearchLaunch &a, uint64_t q, uint64_t lo, uint64_t hi) {
     store_result(a.out, q, lo, hi, a.trunc_cap);
     if (a.tile_kept == nullptr) return;
@@ -776,8 +778,13 @@ __device__ __forceinline__ void store_result_sum(const SearchLaunch &a, uint64_t
     unsigned long long *sum_at = reinterpret_cast<unsigned long long *>(a.tile_kept) + tile;
     if (a.tile_sum_by_warp) {
         const unsigned same = __match_any_sync(__activemask(), tile);
-        const uint32_t sum = __reduce_add_sync(same, k);
-        if (sum != 0u && (threadIdx.x & 31u) == (unsigned)(__ffs(same) - 1)) atomicAdd(sum_at, (unsigned long long)sum);
+        unsigned long long sum;
+        if (a.trunc_cap <= 0xFFFFFFFFu / 32u)
+            sum = __reduce_add_sync(same, k);
+        else
+            sum = __reduce_add_sync(same, k & 0xFFFFu) +
+                  ((unsigned long long)__reduce_add_sync(same, k >> 16) << 16);
+        if (sum != 0u && (threadIdx.x & 31u) == (unsigned)(__ffs(same) - 1)) atomicAdd(sum_at, sum);
     } else if (k != 0u) {
         atomicAdd(sum_at, (unsigned long long)k);
     }
