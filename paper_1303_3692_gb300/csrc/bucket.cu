@@ -306,6 +306,8 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
 constexpr uint32_t kTileWords = kScatterTile * 6;  // 192 bases per query; more: each query by itself
 constexpr uint32_t kTileLead = 6, kTilePad = 8;
 constexpr size_t kScatterAsciiSmem = (kTileLead + kTileWords + kTilePad) * 8 + kScatterTile * 16;
+static_assert((kTileLead + kTileWords + kTilePad) * sizeof(uint2) % alignof(uint4) == 0,
+              "the headers after the tile's words are read and written as uint4");
 
 // 16 bases of a tile as a 32-bit word, base 0 on top: the tile holds its packed
 // words' high halves before their low ones, so a window at any base is a funnel
@@ -336,7 +338,7 @@ template <bool kSingle>
 __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kernel(const __grid_constant__ SearchLaunch a,
                                                                                  uint4 *__restrict__ list) {
     // the tile's words (kTileLead of no meaning before, kTilePad after), then its records' headers
-    extern __shared__ uint2 stile[];
+    extern __shared__ __align__(16) uint2 stile[];
     uint2 *words = stile + kTileLead;
     const uint32_t *half = reinterpret_cast<const uint32_t *>(words);
     uint4 *head = reinterpret_cast<uint4 *>(stile + kTileLead + kTileWords + kTilePad);
