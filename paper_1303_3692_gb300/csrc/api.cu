@@ -254,21 +254,30 @@ int search_timed(const sa_search_params *params, cudaStream_t s, Launch launch) 
 }
 
 // Whether a batch is searched by one kernel from its ASCII bases (small.cu):
-// the cost of the other path's launches and passes, about 50 us, against that
+// the cost of the other path's launches and passes, 20-50 us, against that
 // kernel's slower rate per query and base.  Measured on the GB300, one kernel
-// against the other path, us a call: 5*10^5 queries of 100 bases at 100 Mbp 99
-// against 126, of 20-300 bases (84 M) 224 against 197, 65,536 of 1024 bases
-// (67 M) 233 against 309, 131,072 of them 379 against 343.  With more suffixes
-// than k-mers more brackets are wide and finished by whole warps: at 3.1 Gbp
-// 262,144 queries of 32 bases 101 against 109, of 150 bases (39 M) 162 against
-// 155.  Without a k-mer table every query is: 32,768 queries 64-87 against
-// 80-97, 65,536 99-150 against 81-110.
+// against the other path, us a call, random queries and (after the slash) 80 %
+// copied ones: at 100 Mbp 5*10^5 of 100 bases 69 against 92 / 84 against 113,
+// 670,000 of them 99 against 101 / 143 against 144, 220,000 of 300 74 against 83
+// / 137 against 175, 65,536 of 1024 (67 M) 73 against 79 / 175 against 195,
+// 13,000 of 5000 52 against 72 / 394 against 515.  With more suffixes than
+// k-mers more brackets are wide and finished by whole warps: at 3.1 Gbp 262,144
+// of 32 bases 70 against 88 / 121 against 130, of 150 bases (39 M) 100 against 97
+// / 164 against 165.  Without a k-mer table every query is: 32,768 queries 64-87
+// against 80-97, 65,536 99-150 against 81-110.  Queries of more than kSmallMean
+// bases on average are packed by the other path: what its lanes then compare in
+// the text takes 9.6 ms for 10^6 copied bases, 12.1 here.
 constexpr uint64_t kSmallQueries = 1ull << 19;
 constexpr uint64_t kSmallQueriesNoTable = 1ull << 15;
 constexpr uint64_t kSmallBases = 1ull << 26;
+constexpr uint64_t kSmallMean = 1ull << 17;
+// Beyond this many bases a second kernel checks the longest queries' bytes (1-4
+// us a call); below, the longest one there can be takes its warp 0.35 ms.
+constexpr uint64_t kSmallWarpBases = 1ull << 22;
 bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uint64_t total) {
     for (uint32_t r = 0; r < n_refs; r++)
         if (!refs[r]->krt && n_q > kSmallQueriesNoTable) return false;
+    if (total > kSmallMean * n_q) return false;
     return n_q <= kSmallQueries && total <= (wide_brackets(refs, n_refs) ? kSmallBases / 2 : kSmallBases);
 }
 
@@ -329,6 +338,7 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
         L.tile_kept = tile_kept;
         L.tile_shift = locate_tile_shift(n_q);
         L.tile_sum_by_warp = true;
+        L.check_longest = total > kSmallWarpBases;
         return search_timed(params, s, [&] { return launch_search_small(L, s); });
     }
     const uint64_t nwords = (total + 31) / 32;

@@ -155,6 +155,20 @@ __device__ __forceinline__ uint64_t pack32(uint4 v0, uint4 v1, uint32_t *bad) {
     return x ^ ((x >> 1) & 0x5555555555555555ull);
 }
 
+// Non-zero when one of 16 bytes is not a base (the check of pack32 alone).
+__device__ __forceinline__ uint32_t not_bases(uint4 x) {
+    const uint32_t v[4] = {x.x, x.y, x.z, x.w};
+    uint32_t wrong = 0, any = 0, all = 0xFFFFFFFFu;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const uint32_t t = v[k] & ~(v[k] * 2u) & 0x04040404u;
+        wrong |= (v[k] ^ (t * 4u)) | ~(v[k] ^ (v[k] * 16u));
+        any |= v[k];
+        all &= v[k];
+    }
+    return (wrong & 0x10101010u) | (any & 0x88888888u) | (~all & 0x40404040u);
+}
+
 // Packs the 32 ASCII bases starting at byte s of a (the first nb <= 32 belong
 // to the query; the rest pack as A).  When nine aligned 32-bit words around
 // them lie inside [a, a + total) they are read and aligned with funnel
@@ -751,6 +765,7 @@ struct SearchLaunch {
     uint64_t *tile_kept;
     uint32_t tile_shift;
     bool tile_sum_by_warp;    // input order: the lanes storing together mostly share a tile
+    bool check_longest;       // small.cu: the longest queries' bytes are checked by a kernel of their own
 };
 
 // Queries per tile of the locate's scan (locate.cu): 4096, and 1024 for batches
