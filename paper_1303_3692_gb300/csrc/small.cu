@@ -141,11 +141,13 @@ __device__ __forceinline__ void finish_by_warp(const FrontDesc &d, const AsciiWi
         const unsigned g = greater & lo_lanes, p = match & lo_lanes, s = less & lo_lanes;
         const uint32_t last_g = rank_of(g ? 31 - __clz(g) : 0), first_p = rank_of(p ? __ffs(p) - 1 : 0);
         const uint32_t last_p = rank_of(p ? 31 - __clz(p) : 0), first_s = rank_of(s ? __ffs(s) - 1 : 0);
-        // the new bounds' common prefixes (R's, or once split hR's: no rank below R sorts after the query)
-        __syncwarp();
-        if (g && lane == 31u - __clz(g)) known[0] = l;
-        if (less && lane == (unsigned)__ffs(less) - 1u) known[1] = l;
-        __syncwarp();
+        // the new bounds' common prefixes (R's, or once split hR's: no rank
+        // below R sorts after the query), for a query that goes on past a record
+        if (m > kRecBases) {
+            if (g && lane == 31u - __clz(g)) known[0] = l;
+            if (less && lane == (unsigned)__ffs(less) - 1u) known[1] = l;
+            __syncwarp();
+        }
         const bool low_known = p && ((low_end >> (__ffs(p) - 1)) & 1u);
         const bool high_known = p && ((high_end >> (31 - __clz(p))) & 1u);
         // the upper end's lanes after the split
@@ -282,7 +284,6 @@ __global__ void __launch_bounds__(kSmallThreads, kSmallPerSm) small_kernel(const
         for (int j = 0; j < 4; j++) wq[j] = shfl64(w[j], src);
         const uint32_t mq = __shfl_sync(0xFFFFFFFFu, m, src), rq = __shfl_sync(0xFFFFFFFFu, r, src);
         const AsciiWindows qwq{qw.ascii, qw.total, shfl64(qa, src), mq, __shfl_sync(0xFFFFFFFFu, (int)rc, src) != 0};
-        __syncwarp();
         if ((int)lane == src) {
             s_known[threadIdx.x >> 5][0] = bd.phase == 2 ? 0u : bd.lcpL;
             s_known[threadIdx.x >> 5][1] = bd.phase == 1 ? bd.hlcpR : bd.lcpR;
