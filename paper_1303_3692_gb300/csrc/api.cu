@@ -268,7 +268,20 @@ int search_timed(const sa_search_params *params, cudaStream_t s, Launch launch) 
 // bases on average are packed by the other path: what its lanes then compare in
 // the text takes 9.6 ms for 10^6 copied bases, 12.1 here.
 constexpr uint64_t kSmallQueries = 1ull << 19;
-constexpr uint64_t kSmallQueriesNoTable = 1ull << 15;
+// The queries whose brackets whole warps finish one after the other: all of an
+// index without a k-mer table, and nearly all of one whose k the caller chose so
+// small that a bracket holds many suffixes (the automatic k leaves at most 4 per
+// k-mer).  One kernel against the other path, us a call of 100-base queries at
+// 100 Mbp, 80 % copied: 6 suffixes per k-mer, 2^18 queries 70 against 105; 24,
+// 2^17 81 against 86, 2^18 121 against 112; 95, 2^17 95 against 95, 2^18 142
+// against 124; 1500, 2^15 68 against 87, 2^17 140 against 109; 25,000,000, 2^15
+// 96 against 109, 2^16 150 against 117.
+constexpr uint64_t kSmallQueriesWide = 1ull << 17, kWide = 8;
+constexpr uint64_t kSmallQueriesNoTable = 1ull << 15, kLikeNoTable = 128;
+uint64_t most_small_queries(const sa_index *x) {
+    const uint64_t per_kmer = x->krt ? x->n >> (2 * x->kmer_k) : ~0ull;
+    return per_kmer > kLikeNoTable ? kSmallQueriesNoTable : per_kmer > kWide ? kSmallQueriesWide : kSmallQueries;
+}
 constexpr uint64_t kSmallBases = 1ull << 26;
 constexpr uint64_t kSmallMean = 1ull << 17;
 // Beyond this many bases a second kernel checks the longest queries' bytes (1-4
@@ -276,9 +289,9 @@ constexpr uint64_t kSmallMean = 1ull << 17;
 constexpr uint64_t kSmallWarpBases = 1ull << 22;
 bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uint64_t total) {
     for (uint32_t r = 0; r < n_refs; r++)
-        if (!refs[r]->krt && n_q > kSmallQueriesNoTable) return false;
+        if (n_q > most_small_queries(refs[r])) return false;
     if (total > kSmallMean * n_q) return false;
-    return n_q <= kSmallQueries && total <= (wide_brackets(refs, n_refs) ? kSmallBases / 2 : kSmallBases);
+    return total <= (wide_brackets(refs, n_refs) ? kSmallBases / 2 : kSmallBases);
 }
 
 // Queries of up to this many bases on average have room in the k-mer order's

@@ -3,7 +3,8 @@ that a query's bytes are bases depends on its length -- its lane, its warp, its
 CTA, a kernel over the whole grid -- and a batch of very long queries takes the
 other path: results, marks and locate offsets equal the other path's at the
 lengths where that changes, and one long query costs no more than a few times
-what it costs there."""
+what it costs there.  Batches whose brackets hold many suffixes are small up to
+fewer queries: that path is known by the scratch it takes, none here."""
 import time
 
 import numpy as np
@@ -129,3 +130,26 @@ def test_one_long_query_costs_little(env, lens):
     p = other(sa)
     theirs = shortest(lambda: sa.sa_search_batch(idxs[0], bases, offs, out=out, params=p))
     assert mine < 3 * theirs, (mine * 1e6, theirs * 1e6)
+
+
+# n = 12,000,000: 187,500 suffixes per k-mer at k = 3, 183 and 45 around the line
+# at 128, 11 and 2.9 around the one at 8
+@pytest.mark.parametrize("k, most", [(0, 1 << 15), (3, 1 << 15), (8, 1 << 15), (9, 1 << 17), (10, 1 << 17), (11, 1 << 19),
+                                     (None, 1 << 19)])
+def test_wide_brackets_are_small_batches_of_fewer_queries(env, k, most):
+    sa, text, _ = env
+    idx = sa.sa_build(torch.from_numpy(text).cuda(), kmer_k=k)
+    rng = np.random.default_rng(14)
+    at = rng.integers(0, N - 40, most + 1)
+    qb = text[at[:, None] + np.arange(40)]
+    swap = rng.random(most + 1) < 0.3
+    qb[swap, rng.integers(0, 40, int(swap.sum()))] = ord("G")
+    bases = torch.from_numpy(qb.reshape(-1)).cuda()
+    for n_q in (most, most + 1):
+        offs = torch.arange(0, 40 * n_q + 1, 40, device="cuda", dtype=torch.int64)
+        torch.cuda.synchronize()
+        sa.sa_scratch_info(reset_high=True)
+        got = sa.sa_search_batch(idx, bases, offs)
+        torch.cuda.synchronize()
+        assert (sa.sa_scratch_info()["used_high"] == 0) == (n_q <= most)
+        assert torch.equal(got, sa.sa_search_batch(idx, bases, offs, params=other(sa)))
