@@ -297,9 +297,11 @@ bool small_batch(const sa_index *const *refs, uint32_t n_refs, uint64_t n_q, uin
 // Queries of up to this many bases on average have room in the k-mer order's
 // records and in the scatter's tiles, which then pack the ASCII bases they need
 // themselves instead of reading a packed copy of the batch that a kernel before
-// them writes (with 32-bit numbers for its words).  Longer ones are compared
-// with more of the text than their records carry, from the packed copy, and the
-// persistent pass does that in iterations of its own.
+// them writes (with 32-bit numbers for its words).  Of longer queries among them
+// the scatter writes the packed copy after all, and tiles that do not fit are
+// packed by a kernel of their own.  Batches of longer ones are compared with more
+// of the text than their records carry, and the persistent pass does that in
+// iterations of its own.
 constexpr uint64_t kRecordBases = 192;
 
 // The search of a batch whose inputs are in device memory: ascii holds the
@@ -362,18 +364,21 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     const bool kmer_order = !plain && use_kmer_order(refs, n_refs, n_q, order);
     const bool long_queries = total > kRecordBases * n_q;
     const bool fused = kmer_order && !long_queries && total < (1ull << 36);
-    uint64_t *tq = fused ? nullptr : sc.get<uint64_t>(SA_TQ_LEAD_WORDS + tq_words) + SA_TQ_LEAD_WORDS;
+    uint64_t *tq = sc.get<uint64_t>(SA_TQ_LEAD_WORDS + tq_words);
+    if (tq != nullptr) tq += SA_TQ_LEAD_WORDS;
     uint32_t *tv = fused ? nullptr : sc.get<uint32_t>(tq_words);
     uint4 *wrec = plain ? nullptr : sc.get<uint4>(4 * n_q);
     uint64_t ktotal = 0;
     for (uint32_t r = 0; r < n_refs; r++)
         if (refs[r]->krt) ktotal += 1ull << (2 * refs[r]->kmer_k);
     uint4 *wrec_in = kmer_order ? sc.get<uint4>(4 * list_capacity(n_q)) : nullptr;
+    uint4 *spoiled = fused ? sc.get<uint4>(scatter_tiles(n_q)) : nullptr;
     // What starts at zero, in one block: flags [0] pack error, [1] status, [2]
     // worklist count, [3] bad reference id, [4] records of the k-mer-ordered
-    // list, [5] a non-base byte in the batch; the persistent pass's counter;
-    // the k-mer order's plan; the bitmap of packed words with a non-base byte.
-    const size_t plan_words = kmer_order ? kPlanWords : 0, bitmap_words = fused ? 0 : tq_words / 32 + 1;
+    // list, [5] a non-base byte in the batch, [6] the fused scatter's spoiled
+    // tiles; the persistent pass's counter; the k-mer order's plan; the bitmap
+    // of packed words with a non-base byte.
+    const size_t plan_words = kmer_order ? kPlanWords : 0, bitmap_words = tq_words / 32 + 1;
     uint32_t *zeroed = sc.get<uint32_t>(10 + plan_words + bitmap_words);
     if (sc.failed) return SA_ERR_NOMEM;
     int *flags = reinterpret_cast<int *>(zeroed);
@@ -431,11 +436,13 @@ int search_device(const sa_index *const *refs, uint32_t n_refs, uint32_t width, 
     L.batch_dirty = flags + 5;
     L.long_queries = long_queries;
     L.fused = fused;
+    L.spoiled = spoiled;
+    L.n_spoiled = reinterpret_cast<uint32_t *>(flags + 6);
 
     if (!fused && (err = launch_pack_batch(L, tq, tvb, tv, s)) != cudaSuccess) return status_from_cuda(err);
     return search_timed(params, s, [&] {
         if (plain) return launch_search_plain(L, s);
-        cudaError_t e = kmer_order ? launch_bucketed_worklist(L, wrec_in, s) : cudaSuccess;
+        cudaError_t e = kmer_order ? launch_bucketed_worklist(L, wrec_in, tq, tvb, s) : cudaSuccess;
         if (e == cudaSuccess) e = launch_front(L, s);
         return e == cudaSuccess ? launch_search(L, s) : e;
     });

@@ -23,7 +23,8 @@
 //                          of the list (9/8 of its estimated size plus 256
 //                          records), in bucket order, and after them an
 //                          overflow region with room for every query;
-//   bucket_scatter_kernel (or, for an unpacked batch, bucket_scatter_ascii_kernel)
+//   bucket_scatter_kernel (or, for an unpacked batch, bucket_scatter_ascii_kernel,
+//                          and then for the few tiles it leaves out)
 //                          per tile of queries: offsets, strand, reference,
 //                          validity of every base when the packing found a
 //                          non-base byte in the batch (invalid and empty
@@ -150,7 +151,7 @@ __global__ void bucket_plan_kernel(const __grid_constant__ SearchLaunch a) {
 // overflow region.
 constexpr int kScatterThreads = 256;
 constexpr int kScatterItems = 2;
-constexpr uint32_t kScatterTile = (uint32_t)kScatterThreads * kScatterItems;  // 32 KB of records
+static_assert(kScatterTile == (uint32_t)kScatterThreads * kScatterItems, "a tile's queries (32 KB of records)");
 constexpr size_t kScatterSmem = (size_t)kScatterTile * 64;
 
 // A tile's runs: exclusive scan of its counts (first warp), and each run's
@@ -186,7 +187,49 @@ __device__ __forceinline__ void reserve_runs(const SearchLaunch &a, const uint32
     }
 }
 
-template <bool kSingle, bool kStrands>
+// Whether the m > 0 bases from base qa on are all bases, by the bitmap alone and
+// the bytes of the few words it marks; a very long query's by the whole warp.
+// Called by all 32 lanes.
+__device__ __forceinline__ bool spoiled_valid(const SearchLaunch &a, bool look, uint64_t qa, uint32_t m) {
+    const uint8_t *ascii = reinterpret_cast<const uint8_t *>(a.ascii);
+    const unsigned lane = threadIdx.x & 31u;
+    constexpr uint32_t kByLane = 1u << 15;
+    bool valid = true;
+    for (unsigned left = __ballot_sync(0xFFFFFFFFu, look); left != 0u;) {
+        // all lanes with a shorter query at once, then the others one by one
+        const unsigned shorter = __ballot_sync(0xFFFFFFFFu, ((left >> lane) & 1u) && m <= kByLane);
+        const int src = shorter ? (int)lane : __ffs(left) - 1;
+        const uint64_t q0 = __shfl_sync(0xFFFFFFFFu, (unsigned long long)qa, src);
+        const uint32_t len = __shfl_sync(0xFFFFFFFFu, m, src);
+        const bool mine = shorter == 0u || ((shorter >> lane) & 1u);
+        bool ok = true;
+        if (mine) {
+            const uint64_t w0 = q0 >> 5, w1 = (q0 + len - 1) >> 5;
+            for (uint64_t g = (w0 >> 5) + (shorter ? 0u : lane); ok && g <= (w1 >> 5); g += shorter ? 1u : 32u) {
+                uint32_t marked = __ldg(a.tvb + g);
+                if (g == (w0 >> 5)) marked &= 0xFFFFFFFFu << (w0 & 31u);
+                if (g == (w1 >> 5)) marked &= 0xFFFFFFFFu >> (31u - (uint32_t)(w1 & 31u));
+                for (; ok && marked != 0u; marked &= marked - 1u) {
+                    const uint64_t b0 = (g * 32 + (__ffs(marked) - 1)) * 32;
+                    ok = bytes_valid(ascii, b0 > q0 ? b0 : q0, b0 + 32 < q0 + len ? b0 + 32 : q0 + len);
+                }
+            }
+        }
+        const bool all = __all_sync(0xFFFFFFFFu, ok);
+        if (shorter) {
+            valid = valid && ok;
+            left &= ~shorter;
+        } else {
+            if ((int)lane == src) valid = all;
+            left &= left - 1u;
+        }
+    }
+    return valid;
+}
+
+// kListed: the tiles are those the scatter of an unpacked batch left out,
+// packed since (fused launches; a few CTAs go through them).
+template <bool kSingle, bool kStrands, bool kListed = false>
 __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(const __grid_constant__ SearchLaunch a,
                                                                            uint4 *__restrict__ list) {
     extern __shared__ uint4 srec[];  // kScatterTile records of 4 uint4
@@ -198,97 +241,103 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
     __shared__ uint16_t slot_bucket[kScatterTile];
     __shared__ BucketRef sref[SA_MAX_REFS];
     __shared__ uint32_t n_valid;
-    for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x) cnt[i] = 0;
     for (unsigned r = threadIdx.x; r < a.n_refs; r += blockDim.x) {
         const RefDesc &d = a.refs.r[r];
         sref[r] = BucketRef{d.kbase, d.n, d.krt != nullptr ? d.kmer_k : 0u};
     }
     // a batch without a non-base byte needs no validity masks
     const bool dirty = *a.batch_dirty != 0;
-    const uint64_t tile = (uint64_t)blockIdx.x * kScatterTile;
-    uint16_t b[kScatterItems];
-    uint32_t rank[kScatterItems], r[kScatterItems], m[kScatterItems];
-    uint64_t at[kScatterItems], w[kScatterItems][4];
-    bool any_bad = false, any_bad_ref = false;
-    __syncthreads();
-    // Every item's loads are issued before the tile's bookkeeping, so that
-    // their DRAM round trips overlap each other and the scans below.
+    const uint32_t n_tiles = kListed ? *a.n_spoiled : gridDim.x;
+    for (uint32_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
+        for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x) cnt[i] = 0;
+        const uint64_t tile = (uint64_t)(kListed ? a.spoiled[ti].x : ti) * kScatterTile;
+        uint16_t b[kScatterItems];
+        uint32_t rank[kScatterItems], r[kScatterItems], m[kScatterItems];
+        uint64_t at[kScatterItems], w[kScatterItems][4];
+        bool any_bad = false, any_bad_ref = false;
+        __syncthreads();
+        // Every item's loads are issued before the tile's bookkeeping, so that
+        // their DRAM round trips overlap each other and the scans below.
 #pragma unroll
-    for (int it = 0; it < kScatterItems; it++) {
-        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
-        r[it] = kSingle || q >= a.n_q ? 0u : __ldg(a.q_ref + q);
-    }
-#pragma unroll
-    for (int it = 0; it < kScatterItems; it++) {
-        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
-        at[it] = 0;
-        m[it] = 0;
-        b[it] = kNoQuery;
-        if (q < a.n_q) {
-            bool bad_range, bad_ref;
-            const bool ok = query_range<kStrands>(a, q, &r[it], &at[it], &m[it], &bad_range, &bad_ref);
-            any_bad |= bad_range;
-            any_bad_ref |= bad_ref;
-            b[it] = ok ? 0u : kNoQuery;  // usable so far; the bucket follows
+        for (int it = 0; it < kScatterItems; it++) {
+            const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+            r[it] = kSingle || q >= a.n_q ? 0u : __ldg(a.q_ref + q);
         }
-    }
 #pragma unroll
-    for (int it = 0; it < kScatterItems; it++) {
-        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
-        // a query without a record reads the batch's first words (always there)
-        const bool ok = b[it] != kNoQuery;
-        query_windows<4, kStrands>(a.tq, ok ? at[it] : 0, 0, w[it]);
-        const bool valid = !(ok && m[it] > 0 && dirty) || query_valid(a.tvb, a.tv, place_first(at[it], m[it]), m[it]);
-        if (q >= a.n_q) continue;
-        if (!ok || !valid) {
-            if (ok) any_bad = true;
+        for (int it = 0; it < kScatterItems; it++) {
+            const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+            at[it] = 0;
+            m[it] = 0;
             b[it] = kNoQuery;
-            store_result_sum(a, q, ~0ull, ~0ull);
-        } else if (m[it] == 0) {
-            b[it] = kNoQuery;
-            store_result_sum(a, q, 0, sref[kSingle ? 0u : r[it]].n);
-        } else {
-            b[it] = bucket_of(a, sref[kSingle ? 0u : r[it]], m[it], w[it][0]);
+            if (q < a.n_q) {
+                bool bad_range, bad_ref;
+                const bool ok = query_range<kStrands>(a, q, &r[it], &at[it], &m[it], &bad_range, &bad_ref);
+                any_bad |= bad_range;
+                any_bad_ref |= bad_ref;
+                b[it] = ok ? 0u : kNoQuery;  // usable so far; the bucket follows
+            }
         }
-    }
 #pragma unroll
-    for (int it = 0; it < kScatterItems; it++) rank[it] = b[it] != kNoQuery ? atomicAdd(&cnt[b[it]], 1u) : 0u;
-    __syncthreads();
-    reserve_runs(a, cnt, off, base, inreg, ovbase, &n_valid);
-    __syncthreads();
+        for (int it = 0; it < kScatterItems; it++) {
+            const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+            // a query without a record reads the batch's first words (always there)
+            const bool ok = b[it] != kNoQuery;
+            query_windows<4, kStrands>(a.tq, ok ? at[it] : 0, 0, w[it]);
+            const bool look = ok && m[it] > 0 && dirty;
+            const uint64_t qa = place_first(at[it], m[it]);
+            const bool valid = kListed ? spoiled_valid(a, look, qa, m[it]) : !look || query_valid(a.tvb, a.tv, qa, m[it]);
+            if (q >= a.n_q) continue;
+            if (!ok || !valid) {
+                if (ok) any_bad = true;
+                b[it] = kNoQuery;
+                store_result_sum(a, q, ~0ull, ~0ull);
+            } else if (m[it] == 0) {
+                b[it] = kNoQuery;
+                store_result_sum(a, q, 0, sref[kSingle ? 0u : r[it]].n);
+            } else {
+                b[it] = bucket_of(a, sref[kSingle ? 0u : r[it]], m[it], w[it][0]);
+            }
+        }
 #pragma unroll
-    for (int it = 0; it < kScatterItems; it++) {
-        if (b[it] == kNoQuery) continue;
-        const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
-        const bool entry = b[it] < kNumBuckets;
-        const uint32_t slot = off[b[it]] + rank[it];
-        // bases 128-191 (the first pass then reads none of a query of up to
-        // 192 bases from the batch)
-        uint64_t t[2] = {0, 0};
-        if (m[it] > 128u) query_windows<2, kStrands>(a.tq, at[it], 128u, t);
-        uint4 *dst = srec + 4 * slot;
-        dst[0] = make_uint4(m[it], (uint32_t)q, (uint32_t)at[it],
-                            place_high(at[it], r[it]) | (entry ? kListNeedsEntry : 0u));
-        dst[1] = make_uint4((uint32_t)w[it][0], (uint32_t)(w[it][0] >> 32), (uint32_t)w[it][1],
-                            (uint32_t)(w[it][1] >> 32));
-        dst[2] = make_uint4((uint32_t)w[it][2], (uint32_t)(w[it][2] >> 32), (uint32_t)w[it][3],
-                            (uint32_t)(w[it][3] >> 32));
-        dst[3] = make_uint4((uint32_t)t[0], (uint32_t)(t[0] >> 32), (uint32_t)t[1], (uint32_t)(t[1] >> 32));
-        slot_bucket[slot] = b[it];
+        for (int it = 0; it < kScatterItems; it++) rank[it] = b[it] != kNoQuery ? atomicAdd(&cnt[b[it]], 1u) : 0u;
+        __syncthreads();
+        reserve_runs(a, cnt, off, base, inreg, ovbase, &n_valid);
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < kScatterItems; it++) {
+            if (b[it] == kNoQuery) continue;
+            const uint64_t q = tile + (uint64_t)it * kScatterThreads + threadIdx.x;
+            const bool entry = b[it] < kNumBuckets;
+            const uint32_t slot = off[b[it]] + rank[it];
+            // bases 128-191 (the first pass then reads none of a query of up to
+            // 192 bases from the batch)
+            uint64_t t[2] = {0, 0};
+            if (m[it] > 128u) query_windows<2, kStrands>(a.tq, at[it], 128u, t);
+            uint4 *dst = srec + 4 * slot;
+            dst[0] = make_uint4(m[it], (uint32_t)q, (uint32_t)at[it],
+                                place_high(at[it], r[it]) | (entry ? kListNeedsEntry : 0u));
+            dst[1] = make_uint4((uint32_t)w[it][0], (uint32_t)(w[it][0] >> 32), (uint32_t)w[it][1],
+                                (uint32_t)(w[it][1] >> 32));
+            dst[2] = make_uint4((uint32_t)w[it][2], (uint32_t)(w[it][2] >> 32), (uint32_t)w[it][3],
+                                (uint32_t)(w[it][3] >> 32));
+            dst[3] = make_uint4((uint32_t)t[0], (uint32_t)(t[0] >> 32), (uint32_t)t[1], (uint32_t)(t[1] >> 32));
+            slot_bucket[slot] = b[it];
+        }
+        __syncthreads();
+        // copy the runs out, 16 bytes per thread per step
+        const uint32_t words = 4u * n_valid;
+        for (uint32_t c = threadIdx.x; c < words; c += kScatterThreads) {
+            const uint32_t slot = c >> 2;
+            const uint32_t bk = slot_bucket[slot];
+            const uint32_t k = slot - off[bk];
+            const uint64_t g = k < inreg[bk] ? (uint64_t)base[bk] + k : (uint64_t)ovbase[bk] + (k - inreg[bk]);
+            list[4 * g + (c & 3u)] = srec[c];
+        }
+        const unsigned lane = threadIdx.x & 31u;
+        if (__any_sync(0xFFFFFFFFu, any_bad) && lane == 0) atomicOr(a.pack_err, 1);
+        if (__any_sync(0xFFFFFFFFu, any_bad_ref) && lane == 0) atomicOr(a.bad_ref, 1);
+        if (kListed) __syncthreads();  // the next tile's counts and records go over these
     }
-    __syncthreads();
-    // copy the runs out, 16 bytes per thread per step
-    const uint32_t words = 4u * n_valid;
-    for (uint32_t c = threadIdx.x; c < words; c += kScatterThreads) {
-        const uint32_t slot = c >> 2;
-        const uint32_t bk = slot_bucket[slot];
-        const uint32_t k = slot - off[bk];
-        const uint64_t g = k < inreg[bk] ? (uint64_t)base[bk] + k : (uint64_t)ovbase[bk] + (k - inreg[bk]);
-        list[4 * g + (c & 3u)] = srec[c];
-    }
-    const unsigned lane = threadIdx.x & 31u;
-    if (__any_sync(0xFFFFFFFFu, any_bad) && lane == 0) atomicOr(a.pack_err, 1);
-    if (__any_sync(0xFFFFFFFFu, any_bad_ref) && lane == 0) atomicOr(a.bad_ref, 1);
 }
 
 // The scatter of a batch that is not packed (api.cu: kRecordBases).  The CTA
@@ -297,13 +346,21 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_kernel(cons
 // is computed from there as it is stored, so the packed batch is neither
 // written nor read back: per query of 150 bases 150 + 64 bytes of HBM traffic
 // instead of 150 + 38 + 38 + 64.  What a record holds, the runs and their
-// reservation are as above.  Bound by the integer pipe (69 % busy; HBM 53 %):
+// reservation are as above.  A tile with a query longer than compares read from
+// its records writes its words to the packed batch for them.  One whose words
+// do not fit -- a query far longer than the others -- is left to
+// pack_spoiled_kernel and bucket_scatter_kernel (two launches, 4 us when there is
+// none).  2^21 queries of 100 bases at 100 Mbp, us a call, with every compare
+// past the records from the ASCII bases and every query of such a tile packed by
+// one thread, and as it is: a tenth of them of 600 bases, 80 % copied, 750, 580;
+// 400 of 10^5 random bases 1850, 320; one of 10^7 136,700, 298; none of either
+// 275, 283.  Bound by the integer pipe (69 % busy; HBM 53 %):
 // 4*10^7 x 150 bases 1.99 ms, where the packing and the scatter took 1.19 +
 // 1.29 ms; 9*10^6 of 100-151 bases of both strands, some with an N, 0.47 ms for
 // 0.24 + 0.33.  (The same in the first pass of input order, a tile per warp, was
 // no faster at 100 bases, 586 us for 577, and slower at 20-250, 1263 for 1144:
 // its warps wait for their reads in turn.)
-constexpr uint32_t kTileWords = kScatterTile * 6;  // 192 bases per query; more: each query by itself
+constexpr uint32_t kTileWords = kScatterTile * 6;  // 192 bases per query
 constexpr uint32_t kTileLead = 6, kTilePad = 8;
 constexpr size_t kScatterAsciiSmem = (kTileLead + kTileWords + kTilePad) * 8 + kScatterTile * 16;
 static_assert((kTileLead + kTileWords + kTilePad) * sizeof(uint2) % alignof(uint4) == 0,
@@ -336,7 +393,8 @@ __device__ __forceinline__ void tile_windows(const uint32_t *half, int at, bool 
 
 template <bool kSingle>
 __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kernel(const __grid_constant__ SearchLaunch a,
-                                                                                 uint4 *__restrict__ list) {
+                                                                                 uint4 *__restrict__ list,
+                                                                                 uint64_t *__restrict__ tq) {
     // the tile's words (kTileLead of no meaning before, kTilePad after), then its records' headers
     extern __shared__ __align__(16) uint2 stile[];
     uint2 *words = stile + kTileLead;
@@ -350,7 +408,7 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
     __shared__ uint32_t slot_to[kScatterTile];  // each slot's record in the list
     __shared__ uint32_t marks[kTileWords / 32];
     __shared__ BucketRef sref[SA_MAX_REFS];
-    __shared__ uint32_t n_valid, w_first, w_last, any_marked;
+    __shared__ uint32_t n_valid, w_first, w_last, any_marked, any_longer;
     for (unsigned i = threadIdx.x; i <= kNumBuckets; i += blockDim.x) cnt[i] = 0;
     for (unsigned r = threadIdx.x; r < a.n_refs; r += blockDim.x) {
         const RefDesc &d = a.refs.r[r];
@@ -360,6 +418,7 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
         w_first = 0xFFFFFFFFu;
         w_last = 0;
         any_marked = 0;
+        any_longer = 0;
     }
     const unsigned lane = threadIdx.x & 31u;
     const uint8_t *ascii = reinterpret_cast<const uint8_t *>(a.ascii);
@@ -402,24 +461,25 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
     __syncthreads();
     const uint32_t w_lo = w_first <= w_last ? w_first : 0u;
     const uint32_t n_words = w_first <= w_last ? w_last - w_first + 1u : 0u;
-    const bool in_tile = n_words <= kTileWords;
-    if (in_tile) {
-        const uint64_t full = aligned16 ? a.total / 32 : 0;  // words that are two 16-byte loads
-        for (uint32_t i0 = threadIdx.x - lane; i0 < n_words; i0 += kScatterThreads) {
-            const uint32_t i = i0 + lane;
-            const uint64_t w = (uint64_t)w_lo + i;
-            uint32_t bad = 0;
-            if (i < n_words) {
-                const uint4 *from = reinterpret_cast<const uint4 *>(ascii + w * 32);
-                const uint64_t x = w < full ? pack32(__ldg(from), __ldg(from + 1), &bad)
-                                            : pack_edge_word(ascii, a.total, w, &bad);
-                words[i] = make_uint2((uint32_t)(x >> 32), (uint32_t)x);
-            }
-            const unsigned marked = __ballot_sync(0xFFFFFFFFu, bad != 0u);
-            if (lane == 0) {
-                marks[i0 >> 5] = marked;
-                if (marked != 0u) any_marked = 1u;
-            }
+    if (n_words > kTileWords) {  // for pack_spoiled_kernel and bucket_scatter_kernel
+        if (threadIdx.x == 0) a.spoiled[atomicAdd(a.n_spoiled, 1u)] = make_uint4(blockIdx.x, w_lo, n_words, 0u);
+        return;
+    }
+    const uint64_t full = aligned16 ? a.total / 32 : 0;  // words that are two 16-byte loads
+    for (uint32_t i0 = threadIdx.x - lane; i0 < n_words; i0 += kScatterThreads) {
+        const uint32_t i = i0 + lane;
+        const uint64_t w = (uint64_t)w_lo + i;
+        uint32_t bad = 0;
+        if (i < n_words) {
+            const uint4 *from = reinterpret_cast<const uint4 *>(ascii + w * 32);
+            const uint64_t x = w < full ? pack32(__ldg(from), __ldg(from + 1), &bad)
+                                        : pack_edge_word(ascii, a.total, w, &bad);
+            words[i] = make_uint2((uint32_t)(x >> 32), (uint32_t)x);
+        }
+        const unsigned marked = __ballot_sync(0xFFFFFFFFu, bad != 0u);
+        if (lane == 0) {
+            marks[i0 >> 5] = marked;
+            if (marked != 0u) any_marked = 1u;
         }
     }
     __syncthreads();
@@ -430,19 +490,10 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
         bool valid = b[it] != kNoQuery;
         uint64_t first = 0;  // the query's first 32 bases
         if (valid && m[it] > 0) {
-            const uint64_t qa = place_first(at[it], m[it]);
-            if (in_tile) {
-                valid = any_marked == 0u || tile_valid(marks, w_lo, ascii, qa, m[it]);
-                uint32_t f[2];
-                tile_windows<2>(half, (int)((at[it] & ~kPlaceRc) - 32ull * w_lo), (at[it] & kPlaceRc) != 0, 0, f);
-                first = ((uint64_t)f[0] << 32) | f[1];
-            } else {
-                const AsciiWindows own{ascii, a.total, qa, m[it], (at[it] & kPlaceRc) != 0};
-                uint32_t bad = 0;
-                first = own.packed(0, &bad);
-                for (uint32_t o = 32u; o < m[it]; o += 32u) (void)own.packed(o, &bad);
-                valid = bad == 0u;
-            }
+            valid = any_marked == 0u || tile_valid(marks, w_lo, ascii, place_first(at[it], m[it]), m[it]);
+            uint32_t f[2];
+            tile_windows<2>(half, (int)((at[it] & ~kPlaceRc) - 32ull * w_lo), (at[it] & kPlaceRc) != 0, 0, f);
+            first = ((uint64_t)f[0] << 32) | f[1];
             any_bad |= !valid;
         }
         if (!valid) {
@@ -453,6 +504,9 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
             store_result_sum(a, q, 0, sref[kSingle ? 0u : r[it]].n);
         } else {
             b[it] = bucket_of(a, sref[kSingle ? 0u : r[it]], m[it], first);
+            // (the worklist's records carry 160 bases; the key tables' descent
+            // goes on in the text after 64)
+            if (m[it] > (b[it] < kNumBuckets ? 160u : 64u)) any_longer = 1u;
         }
     }
 #pragma unroll
@@ -470,6 +524,10 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
         slot_to[slot] = rank[it] < inreg[bk] ? base[bk] + rank[it] : ovbase[bk] + (rank[it] - inreg[bk]);
     }
     __syncthreads();
+    // compares that go on past the records read the packed batch
+    if (any_longer != 0u)
+        for (uint32_t i = threadIdx.x; i < n_words; i += kScatterThreads)
+            tq[(uint64_t)w_lo + i] = ((uint64_t)words[i].x << 32) | words[i].y;
     // the runs, 16 bytes per thread per step: the header, or 64 of the
     // record's 192 bases
     const uint32_t pieces = 4u * n_valid;
@@ -477,18 +535,10 @@ __global__ void __launch_bounds__(kScatterThreads, 5) bucket_scatter_ascii_kerne
         const uint32_t slot = c >> 2, part = c & 3u;
         uint4 v = head[slot];
         if (part != 0u) {
-            const int from = 64 * ((int)part - 1);
-            if (in_tile) {
-                uint32_t w[4];
-                tile_windows<4>(half, (int)(place_of(v.z, v.w & ~kRecordRc) - 32ull * w_lo), (v.w & kRecordRc) != 0,
-                                from, w);
-                v = make_uint4(w[1], w[0], w[3], w[2]);
-            } else {
-                const uint64_t place = place_of(v.z, v.w);
-                const AsciiWindows own{ascii, a.total, place_first(place, v.x), v.x, (place & kPlaceRc) != 0};
-                const uint64_t w0 = (uint32_t)from < v.x ? own(from) : 0, w1 = from + 32u < v.x ? own(from + 32u) : 0;
-                v = make_uint4((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32));
-            }
+            uint32_t w[4];
+            tile_windows<4>(half, (int)(place_of(v.z, v.w & ~kRecordRc) - 32ull * w_lo), (v.w & kRecordRc) != 0,
+                            64 * ((int)part - 1), w);
+            v = make_uint4(w[1], w[0], w[3], w[2]);
         }
         list[4 * (uint64_t)slot_to[slot] + part] = v;
     }
@@ -527,7 +577,8 @@ __global__ void bucket_fill_kernel(const __grid_constant__ SearchLaunch a) {
 
 }  // namespace
 
-cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, cudaStream_t s) {
+cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, uint64_t *tq, uint32_t *tvb,
+                                     cudaStream_t s) {
     if (L.n_q == 0) return cudaSuccess;
     const bool single = L.n_refs == 1 && L.q_ref == nullptr;
     const uint64_t n_s = (L.n_q + kListSampleStride - 1) / kListSampleStride;
@@ -542,15 +593,31 @@ cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, cuda
                                     : strands ? bucket_sample_kernel<false, S> : bucket_sample_kernel<false, P>);
     sample<<<(unsigned)sblocks, kSampleThreads, 0, s>>>(L);
     bucket_plan_kernel<<<1, 32, 0, s>>>(L);
-    const uint64_t stiles = (L.n_q + kScatterTile - 1) / kScatterTile;
-    auto scatter = single ? (L.fused ? bucket_scatter_ascii_kernel<true>
-                                     : strands ? bucket_scatter_kernel<true, true> : bucket_scatter_kernel<true, false>)
-                          : (L.fused ? bucket_scatter_ascii_kernel<false>
-                                     : strands ? bucket_scatter_kernel<false, true> : bucket_scatter_kernel<false, false>);
-    const size_t smem = L.fused ? kScatterAsciiSmem : kScatterSmem;
-    cudaError_t e = cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const unsigned tiles = (unsigned)scatter_tiles(L.n_q);
+    cudaError_t e = cudaSuccess;
+    auto packed = [&](auto kernel, unsigned blocks) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
+        if (e == cudaSuccess) kernel<<<blocks, kScatterThreads, kScatterSmem, s>>>(L, wrec_in);
+    };
+    if (L.fused) {
+        auto scatter = single ? bucket_scatter_ascii_kernel<true> : bucket_scatter_ascii_kernel<false>;
+        e = cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterAsciiSmem);
+        if (e != cudaSuccess) return e;
+        scatter<<<tiles, kScatterThreads, kScatterAsciiSmem, s>>>(L, wrec_in, tq);
+        if ((e = launch_pack_spoiled(L, tq, tvb, s)) != cudaSuccess) return e;
+        const unsigned all = (unsigned)device_sm_count() * 5u, blocks = tiles < all ? tiles : all;
+        if (single)
+            strands ? packed(bucket_scatter_kernel<true, true, true>, blocks)
+                    : packed(bucket_scatter_kernel<true, false, true>, blocks);
+        else
+            strands ? packed(bucket_scatter_kernel<false, true, true>, blocks)
+                    : packed(bucket_scatter_kernel<false, false, true>, blocks);
+    } else if (single) {
+        strands ? packed(bucket_scatter_kernel<true, true>, tiles) : packed(bucket_scatter_kernel<true, false>, tiles);
+    } else {
+        strands ? packed(bucket_scatter_kernel<false, true>, tiles) : packed(bucket_scatter_kernel<false, false>, tiles);
+    }
     if (e != cudaSuccess) return e;
-    scatter<<<(unsigned)stiles, kScatterThreads, smem, s>>>(L, wrec_in);
     bucket_fill_kernel<<<1, 32, 0, s>>>(L);
     return cudaGetLastError();
 }

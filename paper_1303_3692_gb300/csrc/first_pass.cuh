@@ -99,9 +99,7 @@ __device__ __forceinline__ bool tile_valid(const uint32_t *marks, uint64_t w_lo,
         if (g == (w1 >> 5)) marked &= 0xFFFFFFFFu >> (31u - (w1 & 31u));
         for (; marked != 0u; marked &= marked - 1u) {
             const uint64_t b0 = (w_lo + g * 32u + (uint32_t)(__ffs(marked) - 1)) * 32;
-            const uint64_t lo = b0 > qa ? b0 : qa, hi = b0 + 32 < qa + m ? b0 + 32 : qa + m;
-            for (uint64_t b = lo; b < hi; b++)
-                if (base_code(__ldg(ascii + b)) > 3u) return false;
+            if (!bytes_valid(ascii, b0 > qa ? b0 : qa, b0 + 32 < qa + m ? b0 + 32 : qa + m)) return false;
         }
     }
     return true;

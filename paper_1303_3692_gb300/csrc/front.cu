@@ -67,7 +67,6 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
     __shared__ uint32_t s_lprefix[kNumBuckets + 2];        // the list's numbering (list input)
     __shared__ uint32_t s_lstart[kNumBuckets + 1];
     constexpr bool kStrands = kBases != Bases::Packed;
-    static_assert(kFromList || kBases != Bases::Ascii, "in input order the queries come from the packed batch");
     for (unsigned r = threadIdx.x; r < a.n_refs; r += blockDim.x) {
         sdesc[r] = front_desc(a.refs.r[r]);
     }
@@ -102,7 +101,7 @@ __global__ void __launch_bounds__(kFrontThreads, 4) front_kernel(const __grid_co
 
     const uint64_t n_items = kFromList ? (uint64_t)*a.wl_in_count : a.n_q;
     // a batch without a non-base byte needs no per-query validity check
-    const bool dirty = kBases != Bases::Ascii && *a.batch_dirty != 0;
+    const bool dirty = !kFromList && *a.batch_dirty != 0;
     // Offsets and reference of this lane's next query, read one query ahead.
     uint64_t nqa = 0, nqe = 0;
     uint32_t nr = 0;
@@ -297,21 +296,20 @@ cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s) {
     if (L.n_q == 0) return cudaSuccess;
     const bool single = L.n_refs == 1 && L.q_ref == nullptr;
     const bool list = L.wrec_in != nullptr;
-    static int per_sm[14][64] = {};
+    static int per_sm[12][64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     using Kernel = void (*)(SearchLaunch);
-    constexpr Bases P = Bases::Packed, S = Bases::PackedStrands, A = Bases::Ascii;
-    static const Kernel kernels[14] = {front_kernel<false, false, P>, front_kernel<true, false, P>,
+    constexpr Bases P = Bases::Packed, S = Bases::PackedStrands;
+    static const Kernel kernels[12] = {front_kernel<false, false, P>, front_kernel<true, false, P>,
                                        front_kernel<false, false, S>, front_kernel<true, false, S>,
                                        front_kernel<false, true, P>,  front_kernel<true, true, P>,
                                        front_kernel<false, true, S>,  front_kernel<true, true, S>,
-                                       front_kernel<false, true, A>,  front_kernel<true, true, A>,
                                        front_kernel<false, false, P, true>, front_kernel<true, false, P, true>,
                                        front_kernel<false, false, S, true>, front_kernel<true, false, S, true>};
-    const int bases = L.fused ? 2 : (L.revcomp || L.strand_bits ? 1 : 0);
-    const int which = (single ? 1 : 0) + 2 * bases + (list ? 4 : L.front_probes == 1 ? 10 : 0);
+    const int bases = L.revcomp || L.strand_bits ? 1 : 0;
+    const int which = (single ? 1 : 0) + 2 * bases + (list ? 4 : L.front_probes == 1 ? 8 : 0);
     const Kernel kernel = kernels[which];
     int &bps = per_sm[which][dev];
     if (bps == 0) {

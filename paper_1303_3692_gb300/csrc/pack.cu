@@ -109,4 +109,80 @@ cudaError_t launch_pack_batch(const SearchLaunch &L, uint64_t *tq, uint32_t *tvb
     return cudaGetLastError();
 }
 
+// Word w of the batch, packed; its bit in the bitmap when it holds a byte that
+// is not a base.
+__device__ __forceinline__ void pack_one(const SearchLaunch &a, uint64_t w, bool aligned16, uint64_t *__restrict__ tq,
+                                         uint32_t *__restrict__ tvb) {
+    const uint8_t *ascii = reinterpret_cast<const uint8_t *>(a.ascii);
+    uint32_t bad = 0;
+    if (aligned16 && w * 32 + 32 <= a.total) {
+        const uint4 *from = reinterpret_cast<const uint4 *>(ascii + w * 32);
+        tq[w] = pack32(__ldg(from), __ldg(from + 1), &bad);
+    } else {
+        const uint64_t left = a.total - w * 32;
+        tq[w] = pack_word(ascii, a.total, w * 32, left < 32 ? (uint32_t)left : 32u, &bad);
+    }
+    if (bad) {
+        atomicOr(tvb + (w >> 5), 1u << (w & 31u));
+        if (*(volatile int *)a.batch_dirty == 0) atomicOr(a.batch_dirty, 1);
+    }
+}
+
+// The words of the k-mer order's tiles whose bases did not fit the scatter's
+// shared memory (bucket.cu): each tile's by one CTA, but those with a very long
+// query's by all of them.  Tiles with more words than the batch in all (offsets
+// that go back) have it packed once.  Nearly always there are none, and the
+// launch costs 1.5 us.
+constexpr uint32_t kPackThreads = 256;
+constexpr uint32_t kOneCtaWords = 1u << 14;
+
+__global__ void __launch_bounds__(kPackThreads) pack_spoiled_kernel(const __grid_constant__ SearchLaunch a,
+                                                                   uint64_t *__restrict__ tq,
+                                                                   uint32_t *__restrict__ tvb) {
+    __shared__ unsigned long long in_all;
+    __shared__ uint32_t larger[kPackThreads], n_larger;
+    const bool aligned16 = ((uintptr_t)a.ascii & 15u) == 0;
+    const uint32_t n = *a.n_spoiled;
+    if (n == 0) return;
+    if (threadIdx.x == 0) in_all = 0;
+    __syncthreads();
+    unsigned long long mine = 0;
+    for (uint32_t e = threadIdx.x; e < n; e += kPackThreads) mine += a.spoiled[e].z;
+    atomicAdd(&in_all, mine);
+    __syncthreads();
+    if (in_all >= a.nwords) {
+        for (uint64_t w = (uint64_t)blockIdx.x * kPackThreads + threadIdx.x; w < a.nwords;
+             w += (uint64_t)gridDim.x * kPackThreads)
+            pack_one(a, w, aligned16, tq, tvb);
+        return;
+    }
+    // a tile of ordinary size is one CTA's
+    for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) {
+        const uint4 t = a.spoiled[e];
+        for (uint32_t i = threadIdx.x; t.z <= kOneCtaWords && i < t.z; i += kPackThreads)
+            pack_one(a, (uint64_t)t.y + i, aligned16, tq, tvb);
+    }
+    // the others are dealt out to all
+    for (uint32_t e0 = 0; e0 < n; e0 += kPackThreads) {
+        const bool large = e0 + threadIdx.x < n && a.spoiled[e0 + threadIdx.x].z > kOneCtaWords;
+        if (!__syncthreads_or(large)) continue;
+        if (threadIdx.x == 0) n_larger = 0;
+        __syncthreads();
+        if (large) larger[atomicAdd(&n_larger, 1u)] = e0 + threadIdx.x;
+        __syncthreads();
+        for (uint32_t j = 0; j < n_larger; j++) {
+            const uint4 t = a.spoiled[larger[j]];
+            for (uint64_t i = (uint64_t)blockIdx.x * kPackThreads + threadIdx.x; i < t.z;
+                 i += (uint64_t)gridDim.x * kPackThreads)
+                pack_one(a, t.y + i, aligned16, tq, tvb);
+        }
+        __syncthreads();
+    }
+}
+
+cudaError_t launch_pack_spoiled(const SearchLaunch &L, uint64_t *tq, uint32_t *tvb, cudaStream_t s) {
+    pack_spoiled_kernel<<<(unsigned)device_sm_count() * 8u, kPackThreads, 0, s>>>(L, tq, tvb);
+    return cudaGetLastError();
+}
+
 }  // namespace sa

@@ -81,6 +81,10 @@ __host__ __device__ constexpr uint64_t list_capacity(uint64_t n_q) {
     return (n_q + kListSampleStride) * 9 / 8 + 256ull * (kNumBuckets + 1) + n_q;
 }
 
+// Queries per tile of the k-mer order's scatter (bucket.cu).
+constexpr uint32_t kScatterTile = 512;
+__host__ __device__ constexpr uint64_t scatter_tiles(uint64_t n_q) { return (n_q + kScatterTile - 1) / kScatterTile; }
+
 // The compare outcome of the three cases of Section IV.
 enum : int { CMP_LESS = -1, CMP_PREFIX = 0, CMP_GREATER = 1 };
 
@@ -288,6 +292,13 @@ __device__ __forceinline__ uint64_t query_window(const uint64_t *__restrict__ tq
 __device__ __forceinline__ uint32_t bit_range(uint32_t lo, uint32_t hi) {
     const uint32_t upto = hi >= 32u ? 0xFFFFFFFFu : ((1u << hi) - 1u);
     return upto & ~((1u << lo) - 1u);
+}
+
+// Whether byte range [lo, hi) of the batch, within one of its words, is all bases.
+__device__ __forceinline__ bool bytes_valid(const uint8_t *__restrict__ ascii, uint64_t lo, uint64_t hi) {
+    for (uint64_t b = lo; b < hi; b++)
+        if (base_code(__ldg(ascii + b)) > 3u) return false;
+    return true;
 }
 
 // Whether all m >= 1 bases from base qa of the batch on are bases: the bits of
@@ -561,8 +572,7 @@ struct Bounds {
 
 // Where a kernel reads a query's bases beyond those its records carry: the
 // packed batch (forward queries only, or of either strand), or the batch's
-// ASCII bytes, of either strand (a batch whose kernels pack what they need
-// themselves; api.cu: kRecordBases).
+// ASCII bytes, of either strand.
 enum class Bases { Packed, PackedStrands, Ascii };
 
 // A query's 32-base window at base off (a multiple of 32 below m).
@@ -751,8 +761,10 @@ struct SearchLaunch {
     uint32_t threads, blocks, chunk;
     uint32_t front_probes;    // probes per query in the first pass
     bool long_queries;        // the queries' average length is past what their records carry
-    bool fused;               // k-mer order: no packed batch, the scatter packs what it needs (tq, tvb, tv,
-                              // batch_dirty are not used)
+    bool fused;               // k-mer order: the scatter packs its tiles' bases itself; tq holds only the
+                              // words of tiles with longer queries, tv is null
+    uint4 *spoiled;           // fused: the tiles that did not fit, {tile, first word, words, 0} each
+    uint32_t *n_spoiled;      // fused: their number
     bool revcomp;             // search every query's reverse complement
     bool strand_bits;         // q_ref bit 31 selects each query's strand
     bool expire_waits;        // test hook: the bounded key-table wait gives up at once
@@ -813,10 +825,13 @@ __device__ __forceinline__ void store_result_sum(const SearchLaunch &a, uint64_t
 //   {w0, w1}, {w2, w3}      its first 128 bases (packed words)
 // Packs L.ascii; tvb is zero before, or null (then tv receives every word's mask).
 cudaError_t launch_pack_batch(const SearchLaunch &L, uint64_t *tq, uint32_t *tvb, uint32_t *tv, cudaStream_t s);
+// Packs the words of the tiles in L.spoiled, as above but without masks.
+cudaError_t launch_pack_spoiled(const SearchLaunch &L, uint64_t *tq, uint32_t *tvb, cudaStream_t s);
 cudaError_t launch_front(const SearchLaunch &L, cudaStream_t s);
 // The batch's queries as records in k-mer order (wrec_in), the first pass's
 // input in that order.
-cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, cudaStream_t s);
+cudaError_t launch_bucketed_worklist(const SearchLaunch &L, uint4 *wrec_in, uint64_t *tq, uint32_t *tvb,
+                                     cudaStream_t s);
 cudaError_t launch_search(const SearchLaunch &L, cudaStream_t s);
 // A small batch in one kernel, straight from its ASCII bases (L.tq, L.tv,
 // L.wrec and the like are not used; L.pack_err and L.bad_ref may be null).

@@ -487,9 +487,7 @@ cudaError_t launch_search(const SearchLaunch &L, cudaStream_t s) {
         using I = decltype(idx_tag);
         constexpr bool S = decltype(single_tag)::value;
         const bool strands = L.revcomp || L.strand_bits;
-        if (L.fused)
-            go(search_kernel<I, S, Bases::Ascii, false>);
-        else if (L.long_queries)
+        if (L.long_queries)
             strands ? go(search_kernel<I, S, Bases::PackedStrands, true>) : go(search_kernel<I, S, Bases::Packed, true>);
         else
             strands ? go(search_kernel<I, S, Bases::PackedStrands, false>)

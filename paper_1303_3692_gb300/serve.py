@@ -56,12 +56,13 @@ def scratch_bytes(n_q: int, n_bases: int, both_strands: bool = False) -> int:
     the packed batch (8 bytes per 32 bases), its validity masks (4 bytes per 32
     bases) and the bitmap of words that have one (a bit per 32 bases); 64
     bytes of worklist room per query; in k-mer order the ordered list (64-byte
-    records, room for about 2.125 per query plus 257 * 256); small flags, and
+    records, room for about 2.125 per query plus 257 * 256) and 16 bytes per
+    512 queries for tiles that do not fit; small flags, and
     256 bytes of alignment per allocation.  Queries of both strands
     (both_strands) take no more: they are read from one packing."""
     words = (n_bases + 31) // 32 + 12
     listed = ((n_q + 32) * 9 // 8 + 256 * 257 + n_q) * 64
-    return 12 * words + words // 8 + 4 + 64 * n_q + listed + 1288 * 4 + 80 + 8 * 256
+    return 12 * words + words // 8 + 4 + 64 * n_q + n_q // 32 + 16 + listed + 1288 * 4 + 80 + 8 * 256
 
 
 def kept(counts: np.ndarray, cap: int) -> np.ndarray:
