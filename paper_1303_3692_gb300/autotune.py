@@ -4,10 +4,14 @@ Times sa_search_batch_ex on a sample of a batch for a grid of candidate
 (threads per block, blocks per SM, shared-memory key-table depth, queries per
 warp chunk of the persistent pass, probes of the first pass), checks that
 every candidate returns identical results, and keeps the fastest.  A
-candidate of four values leaves the first pass at the library's default.
+candidate of four values leaves the first pass at the library's default, and
+a value of 0 is the library's default too: the first candidate sets nothing,
+as only such a call of few queries runs as one kernel (include/sa.h), which the
+others are up to twice as slow as.  What is timed is the whole call on the
+stream, packing included, since the paths pack in different places.
 Results are cached in a JSON file keyed by GPU name, the references' sizes,
-the suffix-array width and the batch's length bucket, so a serving process
-tunes once per workload shape.
+the suffix-array width, the batch's length bucket and whether it is one of few
+queries, so a serving process tunes once per workload shape.
 """
 from __future__ import annotations
 
@@ -25,10 +29,12 @@ from . import sa
 # registers a thread, so more resident threads cannot fit (the library
 # reduces such requests) and shapes that forced fewer registers spilled.
 DEFAULT_CANDIDATES: Tuple[Tuple[int, ...], ...] = (
+    (0, 0, 0, 0, 0),
     (1024, 1, 13, 64, 3), (1024, 1, 13, 64, 1), (1024, 1, 13, 64, 2), (1024, 1, 13, 64, 4),
     (1024, 1, 12, 64, 3), (1024, 1, 13, 32, 3), (512, 2, 12, 64, 3), (256, 4, 11, 64, 3),
 )
 
+FEW_QUERIES = 1 << 19  # batches of at most this many may run as one kernel
 LENGTH_BUCKETS = (64, 128, 192, 300, 1 << 62)
 
 
@@ -40,9 +46,10 @@ def length_bucket(mean_len: float) -> int:
     return len(LENGTH_BUCKETS) - 1
 
 
-def cache_key(gpu: str, refs: Sequence["sa.Index"], mean_len: float) -> str:
+def cache_key(gpu: str, refs: Sequence["sa.Index"], mean_len: float, n_q: int) -> str:
     ns = ",".join(str(r.n) for r in refs)
-    return f"{gpu}|w{refs[0].width}|k{','.join(str(r.kmer_k) for r in refs)}|n{ns}|b{length_bucket(mean_len)}"
+    return (f"{gpu}|w{refs[0].width}|k{','.join(str(r.kmer_k) for r in refs)}|n{ns}|b{length_bucket(mean_len)}"
+            f"|{'few' if n_q <= FEW_QUERIES else 'many'}")
 
 
 def default_cache_path() -> str:
@@ -99,7 +106,7 @@ def autotune(refs, q_bases, q_offsets, q_ref=None, sample: int = 1_000_000,
     qo = q_offsets[:n_q + 1]
     mean_len = float((qo[-1] - qo[0]).item()) / max(1, n_q)
     gpu = torch.cuda.get_device_name()
-    key = cache_key(gpu, refs, mean_len)
+    key = cache_key(gpu, refs, mean_len, n_q)
     path = cache_path or default_cache_path()
     cache = load_cache(path) if use_cache else {}
     if key in cache:
@@ -122,11 +129,11 @@ def autotune(refs, q_bases, q_offsets, q_ref=None, sample: int = 1_000_000,
         p = params_from(cand)
         p.flags = sa.SA_PARAM_Q_RANGE
         p.q_first, p.q_total = first, total
-        e0, e1 = ev(), ev()
-        p.search_events[0], p.search_events[1] = e0.cuda_event, e1.cuda_event
         ts = []
         for it in range(reps + 1):
+            e0 = ev()
             sa.sa_search_batch(refs, q_bases, qo, q_ref=qr, out=out, params=p)
+            e1 = ev()
             torch.cuda.synchronize()
             if it:
                 ts.append(timer(e0, e1) if timer else e0.elapsed_time(e1))
