@@ -231,20 +231,31 @@ int sa_build(const char *text, uint64_t n, uint32_t flags, void *stream, sa_inde
  *             since each result is stored as one 32-byte sector).
  *  stream     CUDA stream or NULL.
  *
- * A small batch (up to 2^19 queries and 2^26 bases; less where brackets are
- * wide or an index has no k-mer table) runs as one kernel that packs each
- * query itself, brackets it by the k-mer table and finishes wide brackets
- * with whole warps; it takes no scratch.  The tuning knobs and search orders
- * of sa_search_params, when set, select the path below.
+ * A small batch runs as one kernel that packs each query itself, brackets it by
+ * the k-mer table and finishes wide brackets with whole warps (and a second
+ * one that checks the longest queries' bytes, when the batch has more than 2^22).
+ * Small is up to 2^19 queries (2^17 with more than 8 suffixes per k-mer in some
+ * index, 2^15 with more than 128 or no k-mer table), 2^26 bases (2^25 with more
+ * suffixes than k-mers) and 2^17 bases per query on average.  The tuning knobs
+ * and search orders of sa_search_params, when set, select the path below.
  *
  * A larger one runs as three kernels on the stream: the batch's bases are packed
  * 2 bits each beside a validity bitmap; a one-thread-per-query pass
  * brackets each query of m >= k bases by the k-mer table and probes it up to
  * sa_search_params.front_probes times, and answers a shorter query from the
  * table's counts; a persistent kernel finishes the queries that remain (and
- * every query of an index without a k-mer table).  Scratch device memory from the library pool: about
- * 12 * ceil(total / 32) + 64 n_q bytes (total = the batch's bases), plus the
- * staging copies of host inputs.
+ * every query of an index without a k-mer table).  In k-mer order (sa_search_order)
+ * kernels before the first pass write the batch as a list in that order; with up
+ * to 192 bases per query on average they pack what it needs themselves, six
+ * kernels in front of the two passes, else the packing and four.
+ *
+ * Scratch device memory from the library pool, total being the batch's bases:
+ *  - the one kernel: none, or 16 bytes with device_status or host outputs;
+ *  - otherwise about 12 * ceil(total / 32) + 64 n_q bytes, and in k-mer order
+ *    136 n_q + 4,210,688 more for the list (64 bytes per record, with room for
+ *    9/8 n_q + 256 * 257 records and an overflow of n_q);
+ *  - sa_search_locate adds 8 bytes per 1024 queries (4096 in large batches);
+ *  - the staging copies of host inputs and outputs.
  *
  * A query that cannot be searched -- a byte outside {A,C,G,T,a,c,g,t}, an
  * out-of-range q_ref, or offsets inconsistent with the batch's range -- gets

@@ -727,7 +727,7 @@ cudaError_t launch_build_kmer(sa_index *idx, cudaStream_t s);
 cudaError_t launch_copy_kmer_counts(const sa_index *idx, uint32_t *dst, cudaStream_t s);
 
 // Descriptors of every index a call uses, passed by value as a kernel
-// parameter (64 x 72 bytes; kernel parameters may take up to 32 KB).
+// parameter (64 x 80 bytes; kernel parameters may take up to 32 KB).
 struct RefTable {
     RefDesc r[SA_MAX_REFS];
 };

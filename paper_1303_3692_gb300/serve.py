@@ -58,8 +58,8 @@ def scratch_bytes(n_q: int, n_bases: int, both_strands: bool = False) -> int:
     bytes of worklist room per query; in k-mer order the ordered list (64-byte
     records, room for about 2.125 per query plus 257 * 256) and 16 bytes per
     512 queries for tiles that do not fit; small flags, and
-    256 bytes of alignment per allocation.  Queries of both strands
-    (both_strands) take no more: they are read from one packing."""
+    256 bytes of alignment per allocation.  both_strands changes nothing:
+    queries of both strands are read from one packing."""
     words = (n_bases + 31) // 32 + 12
     listed = ((n_q + 32) * 9 // 8 + 256 * 257 + n_q) * 64
     return 12 * words + words // 8 + 4 + 64 * n_q + n_q // 32 + 16 + listed + 1288 * 4 + 80 + 8 * 256
@@ -86,17 +86,13 @@ def form_batch(queue: List[Request], max_q: int, max_bases: int, budget: int):
     library scratch stay within max_q, max_bases and the device-memory budget;
     the first request that does not fit ends the batch (no reordering)."""
     nq = nb = 0
-    both = False
     i = 0
     while i < len(queue):
         r = queue[i]
-        b2 = both or r.rc
-        if (nq + r.n > max_q or nb + r.nbases > max_bases
-                or scratch_bytes(nq + r.n, nb + r.nbases, both_strands=b2) > budget):
+        if nq + r.n > max_q or nb + r.nbases > max_bases or scratch_bytes(nq + r.n, nb + r.nbases) > budget:
             break
         nq += r.n
         nb += r.nbases
-        both = b2
         i += 1
     return queue[:i], queue[i:]
 
