@@ -782,7 +782,12 @@ struct SearchLaunch {
 
 // Queries per tile of the locate's scan (locate.cu): 4096, and 1024 for batches
 // of up to 2^21 queries, whose 4096-query tiles would fill the GPU's 456
-// resident CTAs a little more than once (2*10^6 queries: 489) or not at all.
+// resident CTAs a little more than once or not at all, and whose 1024-query
+// tiles are few enough (kDirectTiles) to add up the sums of those before them
+// without the scan's launch.  sa_locate, 1024 against 4096, us: 1.9*10^6 queries
+// 80 against 88, 2^21 85 against 93; past it 2.2*10^6 91 against 93 and 87
+// against 85 (14-base and 100-base queries), 3*10^6 113 against 107 and 106
+// against 100, 9*10^6 273 against 269 and 254 against 259.
 constexpr uint32_t kLocateTileShift = 12, kLocateSmallTileShift = 10;
 inline uint32_t locate_tile_shift(uint64_t n_q) {
     return n_q <= (1ull << 21) ? kLocateSmallTileShift : kLocateTileShift;
