@@ -918,17 +918,24 @@ int search_pipelined(const sa_index *const *refs, uint32_t n_refs, uint32_t widt
     // what is left after the last upload are a chunk's, while more and smaller
     // chunks cost the copies of both directions that run at the same time
     // (reads of 100 bases, us a call: 3*10^6 queries in chunks of 2^18, 2^19,
-    // 2^20: 2200, 2086, 2264; 9*10^6: 5880, 5855, 5580).  The last such chunk's
-    // queries go in four quarter chunks, so that less work is left after the
-    // final upload.
+    // 2^20: 2225, 2122, 2300; 9*10^6: 6035, 5520, 5628).  A chunk of 2^19 of them
+    // is also the largest that is searched by one kernel (small_batch): without
+    // that 2434, 2247, 2340 and 6466, 5750, 5670.  The last such chunk's queries
+    // go in four quarter chunks, so that less work is left after the final
+    // upload.  Chunks are multiples of kChunkStep and kQuarterStep queries, so
+    // that offsets and results (and bases, with equal lengths) are copied from
+    // and to aligned addresses: 4*10^6 queries in chunks of 666,667 take 3000,
+    // of 666,624 2735.
+    constexpr uint64_t kChunkStep = 4096, kQuarterStep = 64;
+    auto rounded = [](uint64_t x, uint64_t step) { return (x + step - 1) / step * step; };
     const uint64_t sixth = std::min<uint64_t>(std::max<uint64_t>((n_q + 5) / 6, 1ull << 19), 1ull << 20);
-    const uint64_t per = std::max<uint64_t>((n_q + 11) / 12, sixth);
+    const uint64_t per = rounded(std::max<uint64_t>((n_q + 11) / 12, sixth), kChunkStep);
     std::vector<uint64_t> cut;  // chunk c is [cut[c], cut[c + 1])
     try {
         cut.push_back(0);
         while (n_q - cut.back() > per) cut.push_back(cut.back() + per);
-        const uint64_t rest = n_q - cut.back(), quarter = (rest + 3) / 4;
-        for (int j = 0; j < 4 && cut.back() < n_q; j++) cut.push_back(cut.back() + quarter < n_q ? cut.back() + quarter : n_q);
+        const uint64_t rest = n_q - cut.back(), quarter = rounded((rest + 3) / 4, kQuarterStep);
+        while (cut.back() < n_q) cut.push_back(std::min(cut.back() + quarter, n_q));
     } catch (const std::bad_alloc &) {
         return SA_ERR_NOMEM;
     }
