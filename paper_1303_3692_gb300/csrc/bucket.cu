@@ -12,8 +12,8 @@
 // query's k-mer entry and every suffix record of its bracket lie in its
 // slice.
 //
-// Four kernels put the batch in that order before the first pass (front.cu),
-// which then reads its queries from the list they write:
+// Four kernels (six for an unpacked batch) put the batch in that order before the
+// first pass (front.cu), which then reads its queries from the list they write:
 //   bucket_sample_kernel   every kListSampleStride-th query's bucket -- its
 //                          first k bases as a fraction of all k-mer entries
 //                          of the call's indexes, in kNumBuckets equal

@@ -161,8 +161,9 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s for the key-table copy
 // (The bounds' own arithmetic: Bounds in sa_internal.cuh.)
 // Warps take chunks of worklist entries from one global counter, each
 // chunk's base fetched while the previous chunk is handed out.
-// Launch bounds: 1024 threads, one CTA per SM, at most 64 registers (no
-// spills); smaller CTAs may share an SM up to 1024 threads in all.
+// Launch bounds: 1024 threads, one CTA per SM, at most 64 registers (no spills,
+// but 24-68 bytes in the variants for long queries); smaller CTAs may share an
+// SM up to 1024 threads in all.
 template <typename IdxT, bool kSingle, Bases kBases, bool kLong>
 __global__ void __launch_bounds__(1024, 1) search_kernel(const __grid_constant__ SearchLaunch a) {
     extern __shared__ __align__(128) uint8_t smem[];
