@@ -29,7 +29,7 @@ def test_small_batch_is_left_to_the_default(tmp_path):
     idx = sa.sa_build(torch.from_numpy(r.copy()).cuda())
     qb, qo, _ = datagen.queries(r, 20_000, 22, m=(20, 200), frac_sampled=0.7, subs=(0, 1))
     bases, offs = torch.from_numpy(qb).cuda(), torch.from_numpy(qo).cuda()
-    p, rep = autotune.autotune(idx, bases, offs, cache_path=str(tmp_path / "tune.json"))
+    p, rep = autotune.autotune(idx, bases, offs, reps=7, cache_path=str(tmp_path / "tune.json"))
     assert rep["best"] == [0, 0, 0, 0, 0] and len(rep["all"]) == len(autotune.DEFAULT_CANDIDATES)
     torch.cuda.synchronize()
     sa.sa_scratch_info(reset_high=True)
